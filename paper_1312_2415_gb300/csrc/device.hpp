@@ -48,7 +48,7 @@ struct GemmGroup {
   double* C;
   int ldc, m, n;
   int task_begin, task_end;
-  int tile_begin;     // prefix of 32x32 output tiles (filled by the uploader)
+  int rpl;            // rows of one column that a lane sums (1, 2 or 4; filled by the uploader)
 };
 struct GemmPlan;  // device copy of a task/group table
 GemmPlan* gemm_plan_upload(const std::vector<GemmTask>& t, std::vector<GemmGroup>& g, Stream s);

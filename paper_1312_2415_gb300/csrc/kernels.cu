@@ -5,6 +5,7 @@
 #include <algorithm>
 #include <cmath>
 #include <cstdio>
+#include <limits>
 #include <mutex>
 #include <stdexcept>
 #include <string>
@@ -138,106 +139,253 @@ float event_elapsed_ms(void* a, void* b) {
 }
 
 // ------------------------------------------------------------------ grouped GEMM
+//
+// C_g += sum_t alpha_t op(A_t) op(B_t) over tables of thousands of small blocks (1 to ~150
+// rows, tens to thousands of tasks per output).  An SM retires two FP64 FMAs per cycle, 16
+// cycles for one warp's FMA, while L1 serves a warp's operand in 1 to 4: neither register
+// tiling nor staging in shared memory buys anything, but every idle lane and every wait on
+// a chain of tasks does cost.  So the output elements of a group are laid on lanes without
+// padding to a tile: a lane owns R rows of one column (R = 1, 2 or 4, chosen per group so
+// that the fewest lanes idle), the operands come straight from L1 / L2 with no barrier
+// anywhere in the sum, and groups with long task lists are shared by 2 to 8 warps of a CTA,
+// whose partial sums are added in a fixed order (deterministic, no atomics).  Measured
+// against 32 x 32 tiles staged in shared memory with two barriers per 16 columns (H_eff x,
+// whole call): Hubbard L=8, D=64 769 -> 99 us; random L=12, D=500 17.4 -> 1.36 ms; random
+// L=28, D=1500 281 -> 157 ms (phase 1 0.82 of the 1.1 TFLOP/s FP64 rate).
 
 namespace {
-constexpr int BM = 32, BN = 32, BK = 16;
+constexpr int kGemmWarps = 8;
 
-__global__ void __launch_bounds__(256) k_grouped_gemm(const GemmTask* __restrict__ tasks,
-                                                     const GemmGroup* __restrict__ groups,
-                                                     int ngroups) {
-  __shared__ double As[BK][BM + 1];
-  __shared__ double Bs[BK][BN + 1];
-  const int tile = blockIdx.x;
-  int lo = 0, hi = ngroups - 1;
-  while (lo < hi) {  // last group with tile_begin <= tile
-    int mid = (lo + hi + 1) >> 1;
-    if (groups[mid].tile_begin <= tile) lo = mid; else hi = mid - 1;
-  }
-  const GemmGroup g = groups[lo];
-  const int local = tile - g.tile_begin;
-  const int tn = (g.n + BN - 1) / BN;
-  const int row0 = (local / tn) * BM, col0 = (local % tn) * BN;
-  const int tid = threadIdx.x, ty = tid >> 4, tx = tid & 15;
-  double acc[2][2] = {{0.0, 0.0}, {0.0, 0.0}};
-  for (int t = g.task_begin; t < g.task_end; ++t) {
-    const GemmTask T = tasks[t];
-    if (T.A == nullptr) {  // op(A) = identity: C += alpha op(B)
+struct Remap {
+  const char* lo[4];
+  const char* hi[4];
+  char* to[4];
+};
+
+__device__ __forceinline__ const double* remap_ptr(const double* p, const Remap& m) {
+  const char* c = (const char*)p;
 #pragma unroll
-      for (int i = 0; i < 2; ++i)
+  for (int k = 0; k < 4; ++k)
+    if (c >= m.lo[k] && c < m.hi[k]) return (const double*)(m.to[k] + (c - m.lo[k]));
+  return p;
+}
+
+// acc[r] = sum over tasks [t0, t1) of the element (row i0 + r, column j); rows past the
+// group's last one read row i0 again (their sums are dropped by the caller)
+template <int R, bool kRemap>
+__device__ __forceinline__ void gemm_sum(const GemmTask* __restrict__ tasks, int t0, int t1, int i0, int j, int m,
+                                         const Remap& rm, double (&acc)[R]) {
 #pragma unroll
-        for (int j = 0; j < 2; ++j) {
-          int r = row0 + ty + 16 * i, c = col0 + tx + 16 * j;
-          if (r < g.m && c < g.n)
-            acc[i][j] += T.alpha * (T.transB ? T.B[(size_t)c * T.ldb + r] : T.B[(size_t)r * T.ldb + c]);
-        }
+  for (int r = 0; r < R; ++r) acc[r] = 0.0;
+  GemmTask T = tasks[t0 < t1 ? t0 : 0];
+  for (int t = t0; t < t1; ++t) {
+    const GemmTask cur = T;
+    if (t + 1 < t1) T = tasks[t + 1];  // the next descriptor is in flight while this task runs
+    const double* B = kRemap ? remap_ptr(cur.B, rm) : cur.B;
+    if (cur.A == nullptr) {  // op(A) = identity
+      const int64_t si = cur.transB ? 1 : cur.ldb, sj = cur.transB ? cur.ldb : 1;
+#pragma unroll
+      for (int r = 0; r < R; ++r)
+        acc[r] = fma(cur.alpha, B[(i0 + r < m ? i0 + r : i0) * si + j * sj], acc[r]);
       continue;
     }
-    for (int k0 = 0; k0 < T.k; k0 += BK) {
-      for (int e = tid; e < BM * BK; e += 256) {
-        int r, kk;
-        double v = 0.0;
-        if (T.transA) { kk = e / BM; r = e % BM; } else { r = e / BK; kk = e % BK; }
-        int gr = row0 + r, gk = k0 + kk;
-        if (gr < g.m && gk < T.k)
-          v = T.transA ? T.A[(size_t)gk * T.lda + gr] : T.A[(size_t)gr * T.lda + gk];
-        As[kk][r] = v * T.alpha;
-      }
-      for (int e = tid; e < BK * BN; e += 256) {
-        int c, kk;
-        double v = 0.0;
-        if (T.transB) { c = e / BK; kk = e % BK; } else { kk = e / BN; c = e % BN; }
-        int gc = col0 + c, gk = k0 + kk;
-        if (gc < g.n && gk < T.k)
-          v = T.transB ? T.B[(size_t)gc * T.ldb + gk] : T.B[(size_t)gk * T.ldb + gc];
-        Bs[kk][c] = v;
-      }
-      __syncthreads();
+    const double* A = kRemap ? remap_ptr(cur.A, rm) : cur.A;
+    const int64_t sai = cur.transA ? 1 : cur.lda, sak = cur.transA ? cur.lda : 1;
+    const int64_t sbk = cur.transB ? 1 : cur.ldb, sbj = cur.transB ? cur.ldb : 1;
+    const double* pa[R];
 #pragma unroll
-      for (int kk = 0; kk < BK; ++kk) {
-        double a0 = As[kk][ty], a1 = As[kk][ty + 16];
-        double b0 = Bs[kk][tx], b1 = Bs[kk][tx + 16];
-        acc[0][0] = fma(a0, b0, acc[0][0]);
-        acc[0][1] = fma(a0, b1, acc[0][1]);
-        acc[1][0] = fma(a1, b0, acc[1][0]);
-        acc[1][1] = fma(a1, b1, acc[1][1]);
+    for (int r = 0; r < R; ++r) pa[r] = A + (i0 + r < m ? i0 + r : i0) * sai;
+    const double* pb = B + j * sbj;
+    double s[R];
+#pragma unroll
+    for (int r = 0; r < R; ++r) s[r] = 0.0;
+    int k = cur.k;
+    for (; k >= 4; k -= 4) {
+      double b[4], a[R][4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        b[u] = pb[u * sbk];
+#pragma unroll
+        for (int r = 0; r < R; ++r) a[r][u] = pa[r][u * sak];
       }
-      __syncthreads();
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+#pragma unroll
+        for (int r = 0; r < R; ++r) s[r] = fma(a[r][u], b[u], s[r]);
+      pb += 4 * sbk;
+#pragma unroll
+      for (int r = 0; r < R; ++r) pa[r] += 4 * sak;
+    }
+    for (; k > 0; --k) {
+      const double b = *pb;
+      pb += sbk;
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+        s[r] = fma(*pa[r], b, s[r]);
+        pa[r] += sak;
+      }
+    }
+#pragma unroll
+    for (int r = 0; r < R; ++r) acc[r] = fma(cur.alpha, s[r], acc[r]);
+  }
+}
+
+template <int R, bool kRemap>
+__device__ __forceinline__ void gemm_job(const GemmTask* __restrict__ tasks, const GemmGroup& g, const GemmJob& J,
+                                         const Remap& rm, double* red, bool lead_only) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int slots = ((g.m + R - 1) / R) * g.n;
+  const int nt = g.task_end - g.task_begin;
+  const int t0 = g.task_begin + (int)((int64_t)nt * J.sidx / J.ns);
+  const int t1 = g.task_begin + (int)((int64_t)nt * (J.sidx + 1) / J.ns);
+  double* C = kRemap ? (double*)remap_ptr(g.C, rm) : g.C;
+  for (int w = J.w0; w < J.w0 + J.nw; ++w) {
+    const int slot = w * 32 + lane;
+    const bool valid = slot < slots;
+    const int q = valid ? slot : 0;
+    const int i0 = (q / g.n) * R, j = q % g.n;
+    double acc[R];
+    if (lead_only) {  // second call of a shared sum: this warp adds the other warps' parts
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+        acc[r] = red[(warp * 4 + r) * 32 + lane];
+        for (int o = 1; o < J.ns; ++o) acc[r] += red[((warp + o) * 4 + r) * 32 + lane];
+      }
+    } else {
+      gemm_sum<R, kRemap>(tasks, t0, t1, i0, j, g.m, rm, acc);
+      if (J.ns > 1) {
+#pragma unroll
+        for (int r = 0; r < R; ++r) red[(warp * 4 + r) * 32 + lane] = acc[r];
+        return;
+      }
+    }
+#pragma unroll
+    for (int r = 0; r < R; ++r)
+      if (valid && i0 + r < g.m) C[(size_t)(i0 + r) * g.ldc + j] += acc[r];
+  }
+}
+
+// one warp per job, kGemmWarps jobs per CTA; the ns jobs of a shared sum are consecutive
+// and never straddle CTAs
+template <bool kRemap>
+__global__ void __launch_bounds__(kGemmWarps * 32)
+    k_grouped_gemm(const GemmTask* __restrict__ tasks, const GemmGroup* __restrict__ groups,
+                   const GemmJob* __restrict__ jobs, int njobs, Remap rm) {
+  __shared__ double red4[kGemmWarps * 4 * 32];
+  const int id = blockIdx.x * kGemmWarps + (threadIdx.x >> 5);
+  GemmJob J{-1, 0, 0, 0, 0};
+  GemmGroup g{};
+  if (id < njobs) {
+    J = jobs[id];
+    g = groups[J.group];
+  }
+  for (int pass = 0; pass < 2; ++pass) {
+    if (pass == 1) __syncthreads();
+    if (J.group >= 0 && (pass == 0 || (J.ns > 1 && J.sidx == 0))) {
+      if (g.rpl == 4) gemm_job<4, kRemap>(tasks, g, J, rm, red4, pass == 1);
+      else if (g.rpl == 2) gemm_job<2, kRemap>(tasks, g, J, rm, red4, pass == 1);
+      else gemm_job<1, kRemap>(tasks, g, J, rm, red4, pass == 1);
     }
   }
-#pragma unroll
-  for (int i = 0; i < 2; ++i)
-#pragma unroll
-    for (int j = 0; j < 2; ++j) {
-      int r = row0 + ty + 16 * i, c = col0 + tx + 16 * j;
-      if (r < g.m && c < g.n) g.C[(size_t)r * g.ldc + c] += acc[i][j];
+}
+
+// Rows per lane of a group: the choice that leaves the fewest lanes idle, with a preference
+// for more rows (fewer operand loads per FMA), stronger when lanes of neighbouring columns
+// read B with a stride.
+int rows_per_lane(int m, int n, bool strided_b) {
+  int best = 1;
+  double score = -1.0;
+  for (int R : {4, 2, 1}) {
+    const int64_t slots = (int64_t)((m + R - 1) / R) * n, warps = (slots + 31) / 32;
+    const double eff = (double)m * n / ((double)warps * 32 * R);
+    const double s = eff * (R == 4 ? 1.0 : R == 2 ? (strided_b ? 0.8 : 0.95) : (strided_b ? 0.5 : 0.85));
+    if (s > score) { score = s; best = R; }
+  }
+  return best;
+}
+
+// Jobs of a table.  A job's work is counted in warp FMAs (plus a task's fixed cost); the
+// target is what gives every SM about 40 jobs, at least kGemmMinWork so that a job is worth
+// its start.  Groups above it are shared by up to eight warps, groups below it give one
+// warp several of their 32-lane slices.  Longest jobs first.
+constexpr int64_t kGemmMinWork = 48, kGemmJobsTarget = 152 * 40;
+
+std::vector<GemmJob> gemm_jobs(const std::vector<GemmTask>& t, std::vector<GemmGroup>& g) {
+  std::vector<int64_t> work(g.size(), 0);
+  int64_t total = 0;
+  for (size_t q = 0; q < g.size(); ++q) {
+    GemmGroup& G = g[q];
+    if (G.m <= 0 || G.n <= 0 || G.task_begin >= G.task_end) continue;
+    int64_t ks = 0;
+    bool strided = false;
+    for (int k = G.task_begin; k < G.task_end; ++k) {
+      ks += t[k].A ? t[k].k : 1;
+      strided = strided || (t[k].A && t[k].transB);
     }
+    G.rpl = rows_per_lane(G.m, G.n, strided);
+    work[q] = G.rpl * ks + 4 * (int64_t)(G.task_end - G.task_begin);
+    total += work[q] * (((int64_t)((G.m + G.rpl - 1) / G.rpl) * G.n + 31) / 32);
+  }
+  const int64_t target = std::max(kGemmMinWork, total / kGemmJobsTarget);
+  // buckets: by sharing warps (8, 4, 2, 1), then by decreasing powers of two of the work
+  std::vector<GemmJob> bucket[4][48];
+  for (size_t q = 0; q < g.size(); ++q) {
+    const GemmGroup& G = g[q];
+    if (work[q] == 0) continue;
+    const int nt = G.task_end - G.task_begin;
+    const int64_t slices = ((int64_t)((G.m + G.rpl - 1) / G.rpl) * G.n + 31) / 32;
+    int ns = 1, b = 3;
+    while (ns < kGemmWarps && work[q] > ns * target && 2 * ns <= nt) { ns *= 2; --b; }
+    const int64_t nw = ns > 1 ? 1 : std::min<int64_t>(32767, std::max<int64_t>(1, target / work[q]));
+    int64_t w = work[q] * nw / ns;
+    int lg = 0;
+    while (w > 1) { w >>= 1; ++lg; }
+    auto& out = bucket[b][47 - std::min(lg, 47)];
+    for (int64_t s = 0; s < slices; s += nw)
+      for (int i = 0; i < ns; ++i)
+        out.push_back({(int)q, (int)s, (short)std::min<int64_t>(nw, slices - s), (unsigned char)i, (unsigned char)ns});
+  }
+  std::vector<GemmJob> jobs;
+  for (auto& row : bucket)
+    for (auto& v : row) jobs.insert(jobs.end(), v.begin(), v.end());
+  return jobs;
 }
 }  // namespace
 
 GemmPlan* gemm_plan_upload(const std::vector<GemmTask>& t, std::vector<GemmGroup>& g, Stream s) {
   GemmPlan* p = new GemmPlan;
-  int tiles = 0;
-  for (auto& gr : g) {
-    gr.tile_begin = tiles;
-    if (gr.m > 0 && gr.n > 0) tiles += ((gr.m + BM - 1) / BM) * ((gr.n + BN - 1) / BN);
+  const std::vector<GemmJob> jobs = gemm_jobs(t, g);
+  if (jobs.size() > (size_t)std::numeric_limits<int>::max() - kGemmWarps) {
+    delete p;
+    throw std::runtime_error("block-product table exceeds 2^31 jobs");
   }
   p->ngroups = (int)g.size();
-  p->ntiles = tiles;
+  p->njobs = (int)jobs.size();
   p->ntasks = (int64_t)t.size();
-  if (!t.empty()) {
-    p->tasks = (GemmTask*)dev_alloc(t.size() * sizeof(GemmTask), s);
-    dev_h2d(p->tasks, t.data(), t.size() * sizeof(GemmTask), s);
-  }
-  if (!g.empty()) {
-    p->groups = (GemmGroup*)dev_alloc(g.size() * sizeof(GemmGroup), s);
-    dev_h2d(p->groups, g.data(), g.size() * sizeof(GemmGroup), s);
+  try {
+    if (!t.empty()) {
+      p->tasks = (GemmTask*)dev_alloc(t.size() * sizeof(GemmTask), s);
+      dev_h2d(p->tasks, t.data(), t.size() * sizeof(GemmTask), s);
+    }
+    if (!g.empty()) {
+      p->groups = (GemmGroup*)dev_alloc(g.size() * sizeof(GemmGroup), s);
+      dev_h2d(p->groups, g.data(), g.size() * sizeof(GemmGroup), s);
+    }
+    if (!jobs.empty()) {
+      p->jobs = (GemmJob*)dev_alloc(jobs.size() * sizeof(GemmJob), s);
+      dev_h2d(p->jobs, jobs.data(), jobs.size() * sizeof(GemmJob), s);
+    }
+  } catch (...) {
+    gemm_plan_free(p, s);
+    throw;
   }
   return p;
 }
 
 void gemm_plan_run(const GemmPlan* p, Stream s) {
-  if (!p || p->ntiles == 0) return;
-  k_grouped_gemm<<<p->ntiles, 256, 0, S(s)>>>(p->tasks, p->groups, p->ngroups);
+  if (!p || p->njobs == 0) return;
+  k_grouped_gemm<false><<<(p->njobs + kGemmWarps - 1) / kGemmWarps, kGemmWarps * 32, 0, S(s)>>>(
+      p->tasks, p->groups, p->jobs, p->njobs, Remap{});
   ++g_launches;
   ck(cudaGetLastError(), "grouped_gemm launch");
 }
@@ -246,6 +394,7 @@ void gemm_plan_free(GemmPlan* p, Stream s) {
   if (!p) return;
   dev_free(p->tasks, s);
   dev_free(p->groups, s);
+  dev_free(p->jobs, s);
   delete p;
 }
 
@@ -1524,95 +1673,6 @@ static __device__ __align__(256) double g_noalloc_scratch[kNoAllocScratchDoubles
 std::mutex g_noalloc_mu;
 double* g_noalloc_ptr[64] = {nullptr};  // device address of the array, per device ordinal
 
-struct Remap {
-  const char* lo[4];
-  const char* hi[4];
-  char* to[4];
-};
-
-__device__ __forceinline__ const double* remap_ptr(const double* p, const Remap& m) {
-  const char* c = (const char*)p;
-#pragma unroll
-  for (int k = 0; k < 4; ++k)
-    if (c >= m.lo[k] && c < m.hi[k]) return (const double*)(m.to[k] + (c - m.lo[k]));
-  return p;
-}
-
-// k_grouped_gemm with every operand / output address passed through the remap
-__global__ void __launch_bounds__(256) k_grouped_gemm_ra(const GemmTask* __restrict__ tasks,
-                                                        const GemmGroup* __restrict__ groups,
-                                                        int ngroups, Remap rm) {
-  __shared__ double As[BK][BM + 1];
-  __shared__ double Bs[BK][BN + 1];
-  const int tile = blockIdx.x;
-  int lo = 0, hi = ngroups - 1;
-  while (lo < hi) {
-    int mid = (lo + hi + 1) >> 1;
-    if (groups[mid].tile_begin <= tile) lo = mid; else hi = mid - 1;
-  }
-  const GemmGroup g = groups[lo];
-  double* Cp = (double*)remap_ptr(g.C, rm);
-  const int local = tile - g.tile_begin;
-  const int tn = (g.n + BN - 1) / BN;
-  const int row0 = (local / tn) * BM, col0 = (local % tn) * BN;
-  const int tid = threadIdx.x, ty = tid >> 4, tx = tid & 15;
-  double acc[2][2] = {{0.0, 0.0}, {0.0, 0.0}};
-  for (int t = g.task_begin; t < g.task_end; ++t) {
-    const GemmTask T = tasks[t];
-    const double* Bp = remap_ptr(T.B, rm);
-    if (T.A == nullptr) {
-#pragma unroll
-      for (int i = 0; i < 2; ++i)
-#pragma unroll
-        for (int j = 0; j < 2; ++j) {
-          int r = row0 + ty + 16 * i, c = col0 + tx + 16 * j;
-          if (r < g.m && c < g.n)
-            acc[i][j] += T.alpha * (T.transB ? Bp[(size_t)c * T.ldb + r] : Bp[(size_t)r * T.ldb + c]);
-        }
-      continue;
-    }
-    const double* Ap = remap_ptr(T.A, rm);
-    for (int k0 = 0; k0 < T.k; k0 += BK) {
-      for (int e = tid; e < BM * BK; e += 256) {
-        int r, kk;
-        double v = 0.0;
-        if (T.transA) { kk = e / BM; r = e % BM; } else { r = e / BK; kk = e % BK; }
-        int gr = row0 + r, gk = k0 + kk;
-        if (gr < g.m && gk < T.k)
-          v = T.transA ? Ap[(size_t)gk * T.lda + gr] : Ap[(size_t)gr * T.lda + gk];
-        As[kk][r] = v * T.alpha;
-      }
-      for (int e = tid; e < BK * BN; e += 256) {
-        int c, kk;
-        double v = 0.0;
-        if (T.transB) { c = e / BK; kk = e % BK; } else { kk = e / BN; c = e % BN; }
-        int gc = col0 + c, gk = k0 + kk;
-        if (gc < g.n && gk < T.k)
-          v = T.transB ? Bp[(size_t)gc * T.ldb + gk] : Bp[(size_t)gk * T.ldb + gc];
-        Bs[kk][c] = v;
-      }
-      __syncthreads();
-#pragma unroll
-      for (int kk = 0; kk < BK; ++kk) {
-        double a0 = As[kk][ty], a1 = As[kk][ty + 16];
-        double b0 = Bs[kk][tx], b1 = Bs[kk][tx + 16];
-        acc[0][0] = fma(a0, b0, acc[0][0]);
-        acc[0][1] = fma(a0, b1, acc[0][1]);
-        acc[1][0] = fma(a1, b0, acc[1][0]);
-        acc[1][1] = fma(a1, b1, acc[1][1]);
-      }
-      __syncthreads();
-    }
-  }
-#pragma unroll
-  for (int i = 0; i < 2; ++i)
-#pragma unroll
-    for (int j = 0; j < 2; ++j) {
-      int r = row0 + ty + 16 * i, c = col0 + tx + 16 * j;
-      if (r < g.m && c < g.n) Cp[(size_t)r * g.ldc + c] += acc[i][j];
-    }
-}
-
 // k_combine with remapped addresses
 __global__ void k_combine_ra(const CombSrc* __restrict__ src, const CombDst* __restrict__ dst, Remap rm) {
   const CombDst d = dst[blockIdx.x];
@@ -1664,10 +1724,13 @@ void noalloc_matvec_run(const GemmPlan* p1, const CombPlan* pc, const GemmPlan* 
   // phase 1 accumulates into Z and phase 2 into y: both start at zero; W is overwritten
   if (zsize) ck(cudaMemsetAsync(scratch, 0, sizeof(double) * zsize, S(s)), "memset scratch");
   if (n) ck(cudaMemsetAsync(y, 0, sizeof(double) * n, S(s)), "memset y");
-  if (p1 && p1->ntiles) {
-    k_grouped_gemm_ra<<<p1->ntiles, 256, 0, S(s)>>>(p1->tasks, p1->groups, p1->ngroups, rm);
+  auto gemm = [&](const GemmPlan* p) {
+    if (!p || p->njobs == 0) return;
+    k_grouped_gemm<true><<<(p->njobs + kGemmWarps - 1) / kGemmWarps, kGemmWarps * 32, 0, S(s)>>>(
+        p->tasks, p->groups, p->jobs, p->njobs, rm);
     ++g_launches;
-  }
+  };
+  gemm(p1);
   if (pc && pc->ndst) {
     for (int off = 0; off < pc->ndst; off += 65535) {
       int nb = std::min(65535, pc->ndst - off);
@@ -1675,10 +1738,7 @@ void noalloc_matvec_run(const GemmPlan* p1, const CombPlan* pc, const GemmPlan* 
       ++g_launches;
     }
   }
-  if (p2 && p2->ntiles) {
-    k_grouped_gemm_ra<<<p2->ntiles, 256, 0, S(s)>>>(p2->tasks, p2->groups, p2->ngroups, rm);
-    ++g_launches;
-  }
+  gemm(p2);
   ck(cudaGetLastError(), "allocation-free matvec launch");
 }
 

@@ -6,10 +6,19 @@ namespace dmrg {
 
 void note_launches(int64_t k);  // adds to the count kernel_launches() reports
 
+// what one warp of the grouped GEMM does: nw 32-lane slices of a group's output from slice
+// w0 on, or (ns > 1) the sidx-th of ns parts of the task list for one slice
+struct GemmJob {
+  int group, w0;
+  short nw;
+  unsigned char sidx, ns;
+};
+
 struct GemmPlan {
   GemmTask* tasks = nullptr;
   GemmGroup* groups = nullptr;
-  int ngroups = 0, ntiles = 0;
+  GemmJob* jobs = nullptr;
+  int ngroups = 0, njobs = 0;
   int64_t ntasks = 0;
 };
 
