@@ -51,8 +51,15 @@ struct GemmGroup {
   int rpl;            // rows of one column that a lane sums (1, 2 or 4; filled by the uploader)
 };
 struct GemmPlan;  // device copy of a task/group table
-GemmPlan* gemm_plan_upload(const std::vector<GemmTask>& t, std::vector<GemmGroup>& g, Stream s);
-void gemm_plan_run(const GemmPlan* p, Stream s);
+// How elements are summed.  GEMM_ORDERED: one chain of FMAs in table order, so that the
+// bits do not depend on how the work is split (what steers a Davidson run, which amplifies a
+// rounding difference about a hundredfold per iteration until it converges).  GEMM_SHARED:
+// long task lists are shared by several warps, whose partial sums are added in a fixed order
+// (shorter chains, other rounding).  A plan carries a job table for each kind it is run with.
+enum { GEMM_ORDERED = 1, GEMM_SHARED = 2 };
+GemmPlan* gemm_plan_upload(const std::vector<GemmTask>& t, std::vector<GemmGroup>& g, Stream s,
+                           int sums = GEMM_ORDERED);
+void gemm_plan_run(const GemmPlan* p, Stream s, int sums = GEMM_ORDERED);
 void gemm_plan_free(GemmPlan* p, Stream s);
 int64_t gemm_plan_tasks(const GemmPlan* p);
 

@@ -1243,10 +1243,10 @@ Engine::MatvecPlan* Engine::plan_matvec(int i, bool rdm) {
   P->tall_off = std::move(tall_off);
   P->tall_rows = std::move(tall_rows);
   P->sec_dim = br.dim;
-  P->p1 = gemm_plan_upload(t1, g1, stream_);
+  P->p1 = gemm_plan_upload(t1, g1, stream_, rdm ? GEMM_SHARED : GEMM_ORDERED | GEMM_SHARED);
   P->pc = comb_plan_upload(cs, cd, stream_);
   if (!rdm) {
-    P->p2 = gemm_plan_upload(t2, g2, stream_);
+    P->p2 = gemm_plan_upload(t2, g2, stream_, GEMM_ORDERED | GEMM_SHARED);
     DiagPlan* pd = diag_plan_upload(dt, dov, stream_);
     diag_plan_run(pd, stream_);
     diag_plan_free(pd, stream_);
@@ -1534,7 +1534,8 @@ uint64_t Engine::tc_serial(int i) const {
   return (cached_ && cached_site_ == i && cached_->tc) ? cached_->serial : 0;
 }
 
-void Engine::run_matvec(MatvecPlan* p, const double* x, double* y, bool tc) {
+// sums: how the FP64 products are summed (GEMM_ORDERED inside Davidson)
+void Engine::run_matvec(MatvecPlan* p, const double* x, double* y, bool tc, int sums) {
   if (tc) {
     flush_events();
     if (!ev_[0]) for (auto& e : ev_) e = event_create();
@@ -1569,10 +1570,10 @@ void Engine::run_matvec(MatvecPlan* p, const double* x, double* y, bool tc) {
   flush_events();
   if (!ev_[0]) for (auto& e : ev_) e = event_create();
   event_record(ev_[0], stream_);
-  gemm_plan_run(p->p1, stream_);
+  gemm_plan_run(p->p1, stream_, sums);
   comb_plan_run(p->pc, stream_);
   event_record(ev_[1], stream_);
-  gemm_plan_run(p->p2, stream_);
+  gemm_plan_run(p->p2, stream_, sums);
   event_record(ev_[2], stream_);
   ev_pending_ = true;
   ev_tc_ = false;
@@ -1678,9 +1679,9 @@ void Engine::build_rq(MatvecPlan* P) {
     }
   }
   try {
-    P->rq1 = gemm_plan_upload(t1, g1, stream_);
+    P->rq1 = gemm_plan_upload(t1, g1, stream_, GEMM_SHARED);
     P->rqc = comb_plan_upload(cs, cd, stream_);
-    P->rq2 = gemm_plan_upload(t2, g2, stream_);
+    P->rq2 = gemm_plan_upload(t2, g2, stream_, GEMM_SHARED);
   } catch (...) {
     gemm_plan_free(P->rq1, stream_);
     comb_plan_free(P->rqc, stream_);
@@ -1702,10 +1703,10 @@ void Engine::run_rq(MatvecPlan* P) {
   flush_events();
   if (!ev_[0]) for (auto& e : ev_) e = event_create();
   event_record(ev_[0], stream_);
-  gemm_plan_run(P->rq1, stream_);
+  gemm_plan_run(P->rq1, stream_, GEMM_SHARED);
   comb_plan_run(P->rqc, stream_);
   event_record(ev_[1], stream_);
-  gemm_plan_run(P->rq2, stream_);
+  gemm_plan_run(P->rq2, stream_, GEMM_SHARED);
   event_record(ev_[2], stream_);
   ev_pending_ = true;
   ev_tc_ = false;
@@ -1720,7 +1721,7 @@ void Engine::matvec(int i, const double* x, double* y) {
   check_ready();
   if (i < 0 || i > L_ - 2) throw std::out_of_range("site out of range");
   MatvecPlan* p = plan_for(i);
-  run_matvec(p, x, y, precision_ == 1);
+  run_matvec(p, x, y, precision_ == 1, GEMM_SHARED);
   if (precision_ == 1 && tc_error_flag(stream_)) throw std::runtime_error("cuda: tensor-core wait timed out");
 }
 
@@ -1915,7 +1916,7 @@ double Engine::davidson_core(MatvecPlan* P, double* x, double tol, int maxit, bo
   dev_d2d(V, x, sizeof(double) * n, stream_);
   vec_multidot(V, n, 1, V, n, dots, sc, stream_);
   vec_normalize(V, dots, n, stream_);
-  run_matvec(P, V, AV, tc);
+  run_matvec(P, V, AV, tc, GEMM_ORDERED);
   vec_multidot(V, n, 1, AV, n, G, sc, stream_);
   int m = 1;
   for (; it < maxit; ++it) {
@@ -1987,7 +1988,7 @@ double Engine::davidson_core(MatvecPlan* P, double* x, double tol, int maxit, bo
       m = nkeep;
     }
     dev_d2d(V + (size_t)m * n, t, sizeof(double) * n, stream_);
-    run_matvec(P, V + (size_t)m * n, AV + (size_t)m * n, tc);
+    run_matvec(P, V + (size_t)m * n, AV + (size_t)m * n, tc, GEMM_ORDERED);
     // row m of the Rayleigh matrix (lower triangle is what small_eig reads)
     vec_multidot(V, n, m + 1, AV + (size_t)m * n, n, G + (size_t)m * mmax, sc, stream_);
     ++m;
@@ -2559,7 +2560,7 @@ void Engine::rdm_site(MatvecPlan* P, int i, double* dg, bool last) {
   const double n2 = 1.0;
   // W = sum coef Z (phases 1 and the combine of the FP64 matvec)
   if (P->zsize) dev_zero(P->Z, sizeof(double) * P->zsize, stream_);
-  gemm_plan_run(P->p1, stream_);
+  gemm_plan_run(P->p1, stream_, GEMM_SHARED);
   comb_plan_run(P->pc, stream_);
   const size_t nw = P->witems.size();
   std::vector<int64_t> woff(nw);
@@ -2615,8 +2616,8 @@ void Engine::rdm_site(MatvecPlan* P, int i, double* dg, bool last) {
   dev_zero(Gb, sizeof(double) * std::max<int64_t>(gsize, 1), stream_);
   for (size_t q = 0; q < gg.size(); ++q) gg[q].C = Gb + goff[q];
   {
-    GemmPlan* p = gemm_plan_upload(gt, gg, stream_);
-    gemm_plan_run(p, stream_);
+    GemmPlan* p = gemm_plan_upload(gt, gg, stream_, GEMM_SHARED);
+    gemm_plan_run(p, stream_, GEMM_SHARED);
     gemm_plan_free(p, stream_);
   }
   double flops = P->flops1;
@@ -2672,8 +2673,8 @@ void Engine::rdm_site(MatvecPlan* P, int i, double* dg, bool last) {
         }
       }
     }
-    GemmPlan* p = gemm_plan_upload(ut, ug, stream_);
-    gemm_plan_run(p, stream_);
+    GemmPlan* p = gemm_plan_upload(ut, ug, stream_, GEMM_SHARED);
+    gemm_plan_run(p, stream_, GEMM_SHARED);
     gemm_plan_free(p, stream_);
     for (size_t q = 0; q < ug.size(); ++q)
       if (ut[q].A) flops += 2.0 * ug[q].m * ug[q].n * ut[q].k;

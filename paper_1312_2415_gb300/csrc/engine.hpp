@@ -215,7 +215,7 @@ class Engine {
   void build_rq(MatvecPlan* p);    // tables of the symmetric quadratic form (energy)
   void run_rq(MatvecPlan* p);
   MatvecPlan* plan_for(int i);
-  void run_matvec(MatvecPlan* p, const double* x, double* y, bool tc = false);
+  void run_matvec(MatvecPlan* p, const double* x, double* y, bool tc, int sums);
   double davidson_core(MatvecPlan* P, double* x, double tol, int maxit, bool tc, int* iters,
                        bool* converged);
   void update_left_from(int i, std::vector<CombOp>& comb);

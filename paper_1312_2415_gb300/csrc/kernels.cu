@@ -171,12 +171,28 @@ __device__ __forceinline__ const double* remap_ptr(const double* p, const Remap&
 }
 
 // acc[r] = sum over tasks [t0, t1) of the element (row i0 + r, column j); rows past the
-// group's last one read row i0 again (their sums are dropped by the caller)
-template <int R, bool kRemap>
+// group's last one read row i0 again (their sums are dropped by the caller).
+//
+// kOrdered: one chain of FMAs per element over the tasks and columns in table order with
+// alpha multiplied into A first, whatever the job table: the products that steer a Davidson
+// run (an unconverged one amplifies a rounding difference about a hundredfold per
+// iteration) keep their bits when the work split changes.  alpha = +-1 needs no multiply;
+// otherwise the warp scales each distinct element of A once, four columns at a time,
+// through buf (its 128 doubles of shared memory), instead of once per lane that reads it.
+// Otherwise each task is summed on its own and alpha applied to the sum.
+template <int R, bool kRemap, bool kOrdered>
 __device__ __forceinline__ void gemm_sum(const GemmTask* __restrict__ tasks, int t0, int t1, int i0, int j, int m,
-                                         const Remap& rm, double (&acc)[R]) {
+                                         const Remap& rm, double* buf, double (&acc)[R]) {
+  const int lane = threadIdx.x & 31;
+  // rows the warp's lanes read: first row, count, and this lane's rows among them
+  const int row0 = __reduce_min_sync(0xffffffffu, i0);
+  const int nrow = kOrdered ? min(__reduce_max_sync(0xffffffffu, i0) + R, m) - row0 : 0;
+  int ro[R];
 #pragma unroll
-  for (int r = 0; r < R; ++r) acc[r] = 0.0;
+  for (int r = 0; r < R; ++r) {
+    ro[r] = i0 + r < m ? i0 + r : i0;
+    acc[r] = 0.0;
+  }
   GemmTask T = tasks[t0 < t1 ? t0 : 0];
   for (int t = t0; t < t1; ++t) {
     const GemmTask cur = T;
@@ -185,28 +201,65 @@ __device__ __forceinline__ void gemm_sum(const GemmTask* __restrict__ tasks, int
     if (cur.A == nullptr) {  // op(A) = identity
       const int64_t si = cur.transB ? 1 : cur.ldb, sj = cur.transB ? cur.ldb : 1;
 #pragma unroll
-      for (int r = 0; r < R; ++r)
-        acc[r] = fma(cur.alpha, B[(i0 + r < m ? i0 + r : i0) * si + j * sj], acc[r]);
+      for (int r = 0; r < R; ++r) acc[r] = fma(cur.alpha, B[ro[r] * si + j * sj], acc[r]);
       continue;
     }
     const double* A = kRemap ? remap_ptr(cur.A, rm) : cur.A;
     const int64_t sai = cur.transA ? 1 : cur.lda, sak = cur.transA ? cur.lda : 1;
     const int64_t sbk = cur.transB ? 1 : cur.ldb, sbj = cur.transB ? cur.ldb : 1;
-    const double* pa[R];
-#pragma unroll
-    for (int r = 0; r < R; ++r) pa[r] = A + (i0 + r < m ? i0 + r : i0) * sai;
     const double* pb = B + j * sbj;
+    const bool unit = fabs(cur.alpha) == 1.0;
+    if (kOrdered && !unit && nrow * 4 <= 128) {
+      const int per = nrow > 0 ? nrow : 1;
+      int k = cur.k;
+      for (; k > 0; k -= 4) {
+        double b[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) b[u] = u < k ? pb[u * sbk] : 0.0;
+        __syncwarp();
+        for (int e = lane; e < nrow * 4; e += 32) {
+          const int u = cur.transA ? e / per : e & 3, r = cur.transA ? e - u * per : e >> 2;
+          if (u < k) buf[r * 4 + u] = A[(row0 + r) * sai + u * sak] * cur.alpha;
+        }
+        __syncwarp();
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+          if (u < k) {
+#pragma unroll
+            for (int r = 0; r < R; ++r) acc[r] = fma(buf[(ro[r] - row0) * 4 + u], b[u], acc[r]);
+          }
+        pb += 4 * sbk;
+        A += 4 * sak;
+      }
+      continue;
+    }
+    const double* pa[R];
     double s[R];
 #pragma unroll
-    for (int r = 0; r < R; ++r) s[r] = 0.0;
+    for (int r = 0; r < R; ++r) {
+      pa[r] = A + ro[r] * sai;
+      s[r] = kOrdered ? acc[r] : 0.0;
+    }
+    // what multiplies an element of A (ordered sums): alpha, or its sign moved to B
+    const double fa = kOrdered && !unit ? cur.alpha : 1.0;
+    const double fb = kOrdered && unit && cur.alpha < 0.0 ? -0.0 : 0.0;
+    auto flip = [&](double v) {
+      return __longlong_as_double(__double_as_longlong(v) ^ __double_as_longlong(fb));
+    };
     int k = cur.k;
     for (; k >= 4; k -= 4) {
       double b[4], a[R][4];
 #pragma unroll
       for (int u = 0; u < 4; ++u) {
-        b[u] = pb[u * sbk];
+        b[u] = kOrdered ? flip(pb[u * sbk]) : pb[u * sbk];
 #pragma unroll
         for (int r = 0; r < R; ++r) a[r][u] = pa[r][u * sak];
+      }
+      if (kOrdered && fa != 1.0) {
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+#pragma unroll
+          for (int r = 0; r < R; ++r) a[r][u] *= fa;
       }
 #pragma unroll
       for (int u = 0; u < 4; ++u)
@@ -217,20 +270,21 @@ __device__ __forceinline__ void gemm_sum(const GemmTask* __restrict__ tasks, int
       for (int r = 0; r < R; ++r) pa[r] += 4 * sak;
     }
     for (; k > 0; --k) {
-      const double b = *pb;
+      const double b = kOrdered ? flip(*pb) : *pb;
       pb += sbk;
 #pragma unroll
       for (int r = 0; r < R; ++r) {
-        s[r] = fma(*pa[r], b, s[r]);
+        const double a = kOrdered && fa != 1.0 ? __dmul_rn(*pa[r], fa) : *pa[r];
+        s[r] = fma(a, b, s[r]);
         pa[r] += sak;
       }
     }
 #pragma unroll
-    for (int r = 0; r < R; ++r) acc[r] = fma(cur.alpha, s[r], acc[r]);
+    for (int r = 0; r < R; ++r) acc[r] = kOrdered ? s[r] : fma(cur.alpha, s[r], acc[r]);
   }
 }
 
-template <int R, bool kRemap>
+template <int R, bool kRemap, bool kOrdered>
 __device__ __forceinline__ void gemm_job(const GemmTask* __restrict__ tasks, const GemmGroup& g, const GemmJob& J,
                                          const Remap& rm, double* red, bool lead_only) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -242,7 +296,7 @@ __device__ __forceinline__ void gemm_job(const GemmTask* __restrict__ tasks, con
   for (int w = J.w0; w < J.w0 + J.nw; ++w) {
     const int slot = w * 32 + lane;
     const bool valid = slot < slots;
-    const int q = valid ? slot : 0;
+    const int q = valid ? slot : slots - 1;
     const int i0 = (q / g.n) * R, j = q % g.n;
     double acc[R];
     if (lead_only) {  // second call of a shared sum: this warp adds the other warps' parts
@@ -252,8 +306,8 @@ __device__ __forceinline__ void gemm_job(const GemmTask* __restrict__ tasks, con
         for (int o = 1; o < J.ns; ++o) acc[r] += red[((warp + o) * 4 + r) * 32 + lane];
       }
     } else {
-      gemm_sum<R, kRemap>(tasks, t0, t1, i0, j, g.m, rm, acc);
-      if (J.ns > 1) {
+      gemm_sum<R, kRemap, kOrdered>(tasks, t0, t1, i0, j, g.m, rm, red + warp * 128, acc);
+      if (!kOrdered && J.ns > 1) {
 #pragma unroll
         for (int r = 0; r < R; ++r) red[(warp * 4 + r) * 32 + lane] = acc[r];
         return;
@@ -266,8 +320,8 @@ __device__ __forceinline__ void gemm_job(const GemmTask* __restrict__ tasks, con
 }
 
 // one warp per job, kGemmWarps jobs per CTA; the ns jobs of a shared sum are consecutive
-// and never straddle CTAs
-template <bool kRemap>
+// and never straddle CTAs (ordered sums are never shared)
+template <bool kRemap, bool kOrdered>
 __global__ void __launch_bounds__(kGemmWarps * 32)
     k_grouped_gemm(const GemmTask* __restrict__ tasks, const GemmGroup* __restrict__ groups,
                    const GemmJob* __restrict__ jobs, int njobs, Remap rm) {
@@ -279,12 +333,12 @@ __global__ void __launch_bounds__(kGemmWarps * 32)
     J = jobs[id];
     g = groups[J.group];
   }
-  for (int pass = 0; pass < 2; ++pass) {
+  for (int pass = 0; pass < (kOrdered ? 1 : 2); ++pass) {
     if (pass == 1) __syncthreads();
     if (J.group >= 0 && (pass == 0 || (J.ns > 1 && J.sidx == 0))) {
-      if (g.rpl == 4) gemm_job<4, kRemap>(tasks, g, J, rm, red4, pass == 1);
-      else if (g.rpl == 2) gemm_job<2, kRemap>(tasks, g, J, rm, red4, pass == 1);
-      else gemm_job<1, kRemap>(tasks, g, J, rm, red4, pass == 1);
+      if (g.rpl == 4) gemm_job<4, kRemap, kOrdered>(tasks, g, J, rm, red4, pass == 1);
+      else if (g.rpl == 2) gemm_job<2, kRemap, kOrdered>(tasks, g, J, rm, red4, pass == 1);
+      else gemm_job<1, kRemap, kOrdered>(tasks, g, J, rm, red4, pass == 1);
     }
   }
 }
@@ -310,7 +364,7 @@ int rows_per_lane(int m, int n, bool strided_b) {
 // warp several of their 32-lane slices.  Longest jobs first.
 constexpr int64_t kGemmMinWork = 48, kGemmJobsTarget = 152 * 40;
 
-std::vector<GemmJob> gemm_jobs(const std::vector<GemmTask>& t, std::vector<GemmGroup>& g) {
+std::vector<GemmJob> gemm_jobs(const std::vector<GemmTask>& t, std::vector<GemmGroup>& g, bool ordered) {
   std::vector<int64_t> work(g.size(), 0);
   int64_t total = 0;
   for (size_t q = 0; q < g.size(); ++q) {
@@ -335,7 +389,7 @@ std::vector<GemmJob> gemm_jobs(const std::vector<GemmTask>& t, std::vector<GemmG
     const int nt = G.task_end - G.task_begin;
     const int64_t slices = ((int64_t)((G.m + G.rpl - 1) / G.rpl) * G.n + 31) / 32;
     int ns = 1, b = 3;
-    while (ns < kGemmWarps && work[q] > ns * target && 2 * ns <= nt) { ns *= 2; --b; }
+    while (!ordered && ns < kGemmWarps && work[q] > ns * target && 2 * ns <= nt) { ns *= 2; --b; }
     const int64_t nw = ns > 1 ? 1 : std::min<int64_t>(32767, std::max<int64_t>(1, target / work[q]));
     int64_t w = work[q] * nw / ns;
     int lg = 0;
@@ -352,17 +406,20 @@ std::vector<GemmJob> gemm_jobs(const std::vector<GemmTask>& t, std::vector<GemmG
 }
 }  // namespace
 
-GemmPlan* gemm_plan_upload(const std::vector<GemmTask>& t, std::vector<GemmGroup>& g, Stream s) {
+GemmPlan* gemm_plan_upload(const std::vector<GemmTask>& t, std::vector<GemmGroup>& g, Stream s, int sums) {
   GemmPlan* p = new GemmPlan;
-  const std::vector<GemmJob> jobs = gemm_jobs(t, g);
-  if (jobs.size() > (size_t)std::numeric_limits<int>::max() - kGemmWarps) {
-    delete p;
-    throw std::runtime_error("block-product table exceeds 2^31 jobs");
-  }
-  p->ngroups = (int)g.size();
-  p->njobs = (int)jobs.size();
   p->ntasks = (int64_t)t.size();
   try {
+    for (int kind = 0; kind < 2; ++kind) {
+      if (!(sums & (kind == 0 ? GEMM_ORDERED : GEMM_SHARED))) continue;
+      const std::vector<GemmJob> jobs = gemm_jobs(t, g, kind == 0);  // also sets the groups' rpl
+      if (jobs.size() > (size_t)std::numeric_limits<int>::max() - kGemmWarps)
+        throw std::runtime_error("block-product table exceeds 2^31 jobs");
+      p->njobs[kind] = (int)jobs.size();
+      if (jobs.empty()) continue;
+      p->jobs[kind] = (GemmJob*)dev_alloc(jobs.size() * sizeof(GemmJob), s);
+      dev_h2d(p->jobs[kind], jobs.data(), jobs.size() * sizeof(GemmJob), s);
+    }
     if (!t.empty()) {
       p->tasks = (GemmTask*)dev_alloc(t.size() * sizeof(GemmTask), s);
       dev_h2d(p->tasks, t.data(), t.size() * sizeof(GemmTask), s);
@@ -371,10 +428,6 @@ GemmPlan* gemm_plan_upload(const std::vector<GemmTask>& t, std::vector<GemmGroup
       p->groups = (GemmGroup*)dev_alloc(g.size() * sizeof(GemmGroup), s);
       dev_h2d(p->groups, g.data(), g.size() * sizeof(GemmGroup), s);
     }
-    if (!jobs.empty()) {
-      p->jobs = (GemmJob*)dev_alloc(jobs.size() * sizeof(GemmJob), s);
-      dev_h2d(p->jobs, jobs.data(), jobs.size() * sizeof(GemmJob), s);
-    }
   } catch (...) {
     gemm_plan_free(p, s);
     throw;
@@ -382,19 +435,27 @@ GemmPlan* gemm_plan_upload(const std::vector<GemmTask>& t, std::vector<GemmGroup
   return p;
 }
 
-void gemm_plan_run(const GemmPlan* p, Stream s) {
-  if (!p || p->njobs == 0) return;
-  k_grouped_gemm<false><<<(p->njobs + kGemmWarps - 1) / kGemmWarps, kGemmWarps * 32, 0, S(s)>>>(
-      p->tasks, p->groups, p->jobs, p->njobs, Remap{});
+namespace {
+template <bool kRemap>
+void gemm_launch(const GemmPlan* p, const Remap& rm, int sums, Stream s) {
+  const int kind = sums == GEMM_ORDERED ? 0 : 1;
+  if (!p || p->njobs[kind] == 0) return;
+  const int n = p->njobs[kind], grid = (n + kGemmWarps - 1) / kGemmWarps;
+  if (kind == 0) k_grouped_gemm<kRemap, true><<<grid, kGemmWarps * 32, 0, S(s)>>>(p->tasks, p->groups, p->jobs[0], n, rm);
+  else k_grouped_gemm<kRemap, false><<<grid, kGemmWarps * 32, 0, S(s)>>>(p->tasks, p->groups, p->jobs[1], n, rm);
   ++g_launches;
   ck(cudaGetLastError(), "grouped_gemm launch");
 }
+}  // namespace
+
+void gemm_plan_run(const GemmPlan* p, Stream s, int sums) { gemm_launch<false>(p, Remap{}, sums, s); }
 
 void gemm_plan_free(GemmPlan* p, Stream s) {
   if (!p) return;
   dev_free(p->tasks, s);
   dev_free(p->groups, s);
-  dev_free(p->jobs, s);
+  dev_free(p->jobs[0], s);
+  dev_free(p->jobs[1], s);
   delete p;
 }
 
@@ -1724,13 +1785,7 @@ void noalloc_matvec_run(const GemmPlan* p1, const CombPlan* pc, const GemmPlan* 
   // phase 1 accumulates into Z and phase 2 into y: both start at zero; W is overwritten
   if (zsize) ck(cudaMemsetAsync(scratch, 0, sizeof(double) * zsize, S(s)), "memset scratch");
   if (n) ck(cudaMemsetAsync(y, 0, sizeof(double) * n, S(s)), "memset y");
-  auto gemm = [&](const GemmPlan* p) {
-    if (!p || p->njobs == 0) return;
-    k_grouped_gemm<true><<<(p->njobs + kGemmWarps - 1) / kGemmWarps, kGemmWarps * 32, 0, S(s)>>>(
-        p->tasks, p->groups, p->jobs, p->njobs, rm);
-    ++g_launches;
-  };
-  gemm(p1);
+  gemm_launch<true>(p1, rm, GEMM_SHARED, s);
   if (pc && pc->ndst) {
     for (int off = 0; off < pc->ndst; off += 65535) {
       int nb = std::min(65535, pc->ndst - off);
@@ -1738,7 +1793,7 @@ void noalloc_matvec_run(const GemmPlan* p1, const CombPlan* pc, const GemmPlan* 
       ++g_launches;
     }
   }
-  gemm(p2);
+  gemm_launch<true>(p2, rm, GEMM_SHARED, s);
   ck(cudaGetLastError(), "allocation-free matvec launch");
 }
 

@@ -17,8 +17,8 @@ struct GemmJob {
 struct GemmPlan {
   GemmTask* tasks = nullptr;
   GemmGroup* groups = nullptr;
-  GemmJob* jobs = nullptr;
-  int ngroups = 0, njobs = 0;
+  GemmJob* jobs[2] = {nullptr, nullptr};  // ordered sums, shared sums
+  int njobs[2] = {0, 0};
   int64_t ntasks = 0;
 };
 
