@@ -238,6 +238,7 @@ struct TfTile {         // one output tile of y, computed by one CTA from all of
   int tiny;             // 1: at most 4 x 4 outputs, terms of at most 4 x rows, sources of one K chunk
                         // (computed on CUDA cores, one term per lane)
   int pad;
+  int64_t part;         // first partial sum of this run of terms (set by tc_plan_build)
 };
 // one FP64 block (rows x cols, row-major) to tiled hi / lo (nrg = ceil(rows / 8) row
 // groups per chunk; lo = hi + lo floats); identity != 0: the rows x rows identity

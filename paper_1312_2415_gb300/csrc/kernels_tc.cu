@@ -4,21 +4,22 @@
 // operators of Sec. 2.5, acts on an output block y_X' as a sum of terms
 //   y_X' += C W,   W = sum_s coef_s x_s D_s^T,
 // C a left-operator block, x_s blocks of the two-site vector and D_s right-operator
-// blocks (the combined operators of the left / right environments).  One CTA owns each
-// output tile (up to 128 rows x 128 columns of one block, so nothing is added with
-// atomics and the summation order is fixed) and runs all of its terms; the launch is
-// persistent (one CTA per SM taking tiles from a work queue), so the pipeline runs on
-// from one tile into the next (tiles of at most 4 x 4 outputs go to a CUDA-core kernel,
-// k_tc_tiny, instead):
+// blocks (the combined operators of the left / right environments).  An output tile (up to
+// 128 rows x 128 columns of one block) is cut into runs of terms; a CTA computes a run and
+// leaves its partial sums, which are added in term order afterwards (nothing is added with
+// atomics and the summation order is fixed).  The launch is persistent (one to four CTAs per
+// SM by tile size, taking runs from a work queue), so the pipeline runs on from one run into
+// the next (tiles of at most 4 x 4 outputs go to a CUDA-core kernel, k_tc_tiny, instead):
 //   product 1: W^T = D_s x_s^T per source, into tensor-memory accumulators of at most
 //              two 32-column K chunks each (M = 128 output columns, N = x rows of the
 //              term, K = the right sector);
 //   the converter warps add coef_s times each accumulator into FP32 registers, split the
 //              sum into TF32 head and tail and store it as the A operand of
 //   product 2: y^T += W^T C^T (M = 128 output columns, N = output rows, K = x rows),
-//              restarted per term and drained into FP32 registers, which are added to y
-//              (FP64) every few terms.  The tensor core's own FP32 accumulation loses
-//              accuracy over long runs of products, hence the short accumulators.
+//              restarted per term and drained into FP32 registers, stored every few
+//              terms (the partial sums, added to y in FP64).  The tensor core's own FP32
+//              accumulation loses accuracy over long runs of products, hence the short
+//              accumulators.
 // Every product uses split TF32: v = hi + lo with hi = rna_tf32(v), lo = rna_tf32(v - hi),
 // and the three leading products hi*hi + hi*lo + lo*hi (about 2^-21 relative).  The
 // second operand's hi and lo tiles sit one above the other in shared memory, so one MMA
@@ -55,26 +56,38 @@ namespace dmrg {
 namespace {
 
 constexpr long long kSpinLimit = 1ll << 22;  // polls of an mbarrier before giving up (seconds)
-constexpr int kTF = 128 * 32;                // floats of a 128-row x 32-column tile (16 KB)
+constexpr int kRowsF = 128 * 32;             // floats an M = 128 product reads of its first operand (16 KB)
 constexpr int kMaxS1 = 8;                    // slots of the product-1 operand ring, at most
-constexpr int kS1KB = 96;                    // shared memory of the product-1 ring (KB)
 constexpr int kMaxB2 = 2;                    // C slots, at most
-constexpr int kTmemCols = 512;
-constexpr int kWCols = 128;                  // tensor-memory columns of a W^T accumulator
-constexpr int kNW = 3;                       // W^T accumulators
-constexpr int kYCol = kNW * kWCols;          // first column of the y^T accumulator (128 columns)
+constexpr int kMaxW = 3;                     // W^T accumulators, at most
 constexpr int kTileQ = 4;                    // tiles taken from the work queue ahead of the slowest role
-// shared memory (floats): product-1 slot = D tile hi, lo (up to 128 rows) and x tile hi,
-// lo (kp rows each); product 2: C slots (2 x 128 rows x 2 chunks in all) and W^T tiles
-// (128 rows x 2 chunks, hi, lo)
-constexpr int kB2F = 4 * kTF;
-constexpr int kA2F = 4 * kTF;
-constexpr int kSmemF = kS1KB * 256 + kB2F + kA2F;
 constexpr int kSegChunks = 2;   // K chunks per product-1 accumulator (then added in registers)
-constexpr int kFlushTerms = 16; // terms summed in FP32 registers before they are added to y (FP64)
-constexpr int kProducerWarp = 0, kMma1Warp = 1, kMma2Warp = 2, kConvWarp0 = 3, kConvWarps = 8;
-constexpr int kMvThreads = (kConvWarp0 + kConvWarps) * 32;
-constexpr int kConvThreads = kConvWarps * 32;
+constexpr int kFlushTerms = 16; // terms summed in FP32 registers per partial sum of y
+
+// Three builds of the kernel by tile size.  A tile's terms form a chain (product 1, the
+// conversion of W^T, product 2: about 3.5 us a term, mostly handoffs between the roles), so
+// what counts for small blocks is how many chains an SM runs at once: four CTAs for tiles of
+// at most 32 x 32, two up to 64 x 64, one up to 128 x 128, each with its share of shared
+// memory (KB), tensor memory (columns) and only the converter warps whose rows exist.  NQ:
+// 32-column quarters of the output (tensor-memory lanes); NH: converter warps per quarter,
+// which split the x rows of W^T and the output rows.
+template <int NQ, int NH, int A2KB, int S1KB, int B2KB, int TMEM, int YCOLS, int CTAS>
+struct TileClass {
+  static constexpr int kA2F = A2KB * 256, kS1F = S1KB * 256, kB2F = B2KB * 256;
+  static constexpr int kTmem = TMEM, kWReg = TMEM - YCOLS, kCtas = CTAS;
+  static constexpr int kSmemF = kA2F + kS1F + kB2F;
+  static constexpr int kMaxM = YCOLS, kMaxN = 32 * NQ, kMaxKdl = 32 * NH;
+  static constexpr int kYR = YCOLS / NH;  // output rows per converter thread
+  // warps: a converter of quarter q is a warp with index q mod 4 (tensor-memory lanes)
+  static constexpr int kProducerWarp = NQ == 1 ? 1 : NQ == 2 ? 2 : 8;
+  static constexpr int kMma1Warp = NQ == 1 ? 2 : NQ == 2 ? 3 : 9;
+  static constexpr int kMma2Warp = NQ == 1 ? 3 : NQ == 2 ? 6 : 10;
+  static constexpr int kThreads = NQ == 1 ? 128 : NQ == 2 ? 224 : 352;
+  static constexpr int kConvThreads = NQ * NH * 32;
+};
+using TileS = TileClass<1, 1, 8, 32, 8, 128, 32, 4>;
+using TileM = TileClass<2, 2, 24, 62, 24, 256, 64, 2>;
+using TileL = TileClass<4, 2, 64, 96, 64, 512, 128, 1>;
 
 __device__ int g_tc_error = 0;
 __device__ int g_tc_inject = 0;
@@ -211,8 +224,8 @@ __device__ __forceinline__ void mma_triple_steps(uint32_t tmem, uint64_t ah, uin
 
 struct Bars {
   uint64_t s1_full[kMaxS1], s1_empty[kMaxS1];
-  uint64_t b2_full[kMaxB2], b2_empty[kMaxB2];
-  uint64_t w_full[kNW], w_empty[kNW];
+  uint64_t b2_full[kMaxB2];
+  uint64_t w_full[kMaxW], w_empty[kMaxW];
   uint64_t a2_full, mma2_done;
   uint64_t drain1, drain2, never;
   uint64_t tile_full[kTileQ], tile_empty[kTileQ];
@@ -240,52 +253,71 @@ __device__ __forceinline__ void mma_pair_steps(uint32_t tmem, uint64_t ah, uint6
   }
 }
 
-// Geometry of one output tile.  kp: x rows of a term rounded up to 32 (x hi and x lo are
-// stacked kp rows apart); mp: output rows rounded up to 32 (C hi and C lo are stacked mp
-// rows apart).  Product-1 slots are sized for the tile (its output columns and its
-// widest term), as many as fit: small blocks keep more copies in flight.  C slots hold
-// the chunks of the tile's widest term.
+// Geometry of one output tile in its class.  kp: x rows of a term rounded up to 16 (x hi
+// and x lo are stacked kp rows apart; kpm for the widest term); mp: output rows rounded up to
+// 16 (C hi and C lo are stacked mp rows apart).  Product-1 slots are sized for the tile (its
+// output columns and its widest term), as many as fit: small blocks keep more copies in
+// flight; the D tiles of the last slot must leave room for an M = 128 product's reads.  C
+// slots hold the chunks of the tile's widest term.  A segment's slots are released together,
+// so there are at least kSegChunks of them.  wc, nw: tensor-memory columns and number
+// of the W^T accumulators.
+__host__ __device__ constexpr int term_rows(int kdl) { return (kdl + 15) & ~15; }
+
+template <class K>
 struct TileGeom {
-  int T, nvg, mg, mp, kpm, slot_f, nslots, b2_f, nb2;
-  __device__ explicit TileGeom(const TfTile& t) {
+  int T, nvg, mg, mp, kpm, slot_f, nslots, b2_f, nb2, a2_f, wc, nw;
+  bool fits;  // the class can run the tile
+  __host__ __device__ explicit TileGeom(const TfTile& t) {
     T = t.t_end - t.t_begin;
     nvg = (t.nv + 7) >> 3;
     mg = (t.m + 7) >> 3;
-    mp = (t.m + 31) & ~31;
-    kpm = t.kdg > 4 ? 64 : 32;
+    mp = (t.m + 15) & ~15;
+    kpm = term_rows(t.kdg * 8);
+    a2_f = nvg * 256;  // one W^T tile: nvg * 8 rows x 32 columns
     slot_f = (2 * nvg + kpm / 4) * 256;
-    nslots = min(kMaxS1, (kS1KB * 256) / slot_f);
-    b2_f = 2 * mp * 32 * (kpm / 32);
-    nb2 = min(kMaxB2, kB2F / b2_f);
+    const int room = (K::kSmemF - K::kA2F - kRowsF - nvg * 256) / slot_f + 1, fit = K::kS1F / slot_f;
+    nslots = room < fit ? room : fit;
+    if (nslots > kMaxS1) nslots = kMaxS1;
+    b2_f = 2 * mp * 32 * (kpm > 32 ? 2 : 1);
+    nb2 = K::kB2F / b2_f;
+    if (nb2 > kMaxB2) nb2 = kMaxB2;
+    wc = 2 * kpm;
+    nw = K::kWReg / wc;
+    if (nw > kMaxW) nw = kMaxW;
+    fits = t.m <= K::kMaxM && t.nv <= K::kMaxN && t.kdg * 8 <= K::kMaxKdl && nslots >= kSegChunks && nb2 >= 1 && nw >= 1 &&
+           a2_f * 2 * (kpm > 32 ? 2 : 1) <= K::kA2F;
   }
 };
 
-// Persistent: one CTA per SM takes tiles from a work queue (a counter in global memory,
-// zeroed before the launch, handing out the tiles in the planner's order) until it is
-// empty, so the pipeline runs on from one tile into the next.  The producer thread takes
-// each tile and passes its index to the other roles through a small ring in shared
-// memory (tile_full / tile_empty); -1 ends the list.  Ring phases are kept per slot
-// across tiles (bit masks of parities), and a tile whose product-1 slot layout differs
-// from the last one's waits for the last one's slots to be released first.  Tensor
-// memory has a fixed layout: kNW W^T accumulators of 128 columns and the y^T accumulator
-// in the last 128 columns.
-__global__ void __launch_bounds__(kMvThreads, 1)
+// Persistent: K::kCtas CTAs per SM take tiles from a work queue (a counter in global
+// memory, zeroed before the launch, handing out the tiles in the planner's order) until it
+// is empty, so the pipeline runs on from one tile into the next.  A tile here is a run of
+// the terms of one output tile, a multiple of kFlushTerms long (tc_plan_build); the FP32
+// sum of every kFlushTerms terms goes to `part`, and k_tc_reduce adds an output tile's
+// partial sums to y in FP64 in term order: the same additions in the same order whatever
+// the split.  The producer thread takes each tile and passes its index to the other roles
+// through a small ring in shared memory (tile_full / tile_empty); -1 ends the list.  Ring
+// phases are kept per slot across tiles (bit masks of parities), and a tile whose product-1
+// slot or W^T accumulator layout differs from the last one's waits for the last one's to be
+// released first.
+template <class K>
+__global__ void __launch_bounds__(K::kThreads, K::kCtas)
     k_tc_matvec(const TfTile* __restrict__ tiles, const TfTask* __restrict__ tasks, const TfSrc* __restrict__ srcs,
-                int* __restrict__ queue, const int* __restrict__ active, int ntiles) {
+                float* __restrict__ part, int* __restrict__ queue, const int* __restrict__ active, int ntiles) {
   extern __shared__ unsigned char smem_dyn[];
   float* sm = (float*)(((uintptr_t)smem_dyn + 1023) & ~(uintptr_t)1023);
-  float* s1 = sm;                      // product-1 slots: D hi, D lo (nvg KB each), x hi, x lo (kp rows each)
-  float* b2 = sm + kS1KB * 256;        // C slots: per K chunk C hi (mp rows) then C lo (mp rows); they
-                                       // follow the product-1 slots, which the MMA's reads of a whole
-                                       // 128-row D tile may run past
-  float* a2 = b2 + kB2F;               // W^T: chunk 0 hi, lo, chunk 1 hi, lo
+  float* a2 = sm;                      // W^T: chunk 0 hi, lo, chunk 1 hi, lo (a2_f floats each)
+  float* s1 = sm + K::kA2F;            // product-1 slots: D hi, D lo (nvg KB each), x hi, x lo (kp rows each)
+  float* b2 = s1 + K::kS1F;            // C slots: per K chunk C hi (mp rows) then C lo (mp rows)
+                                       // (an M = 128 product reads 16 KB from a D or W^T tile's start,
+                                       // past its rows: rows of the result nobody uses)
   __shared__ __align__(8) Bars bar;
   __shared__ uint32_t tmem_slot;
   __shared__ volatile int abort_flag;
   __shared__ int tile_q[kTileQ];
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  if (warp == kMma1Warp) tmem_alloc(&tmem_slot, kTmemCols);
+  if (warp == K::kMma1Warp) tmem_alloc(&tmem_slot, K::kTmem);
   if (tid == 0) {
     for (int s = 0; s < kMaxS1; ++s) {
       mbar_init_n(&bar.s1_full[s], 1);
@@ -293,33 +325,32 @@ __global__ void __launch_bounds__(kMvThreads, 1)
     }
     for (int s = 0; s < kMaxB2; ++s) {
       mbar_init_n(&bar.b2_full[s], 1);
-      mbar_init_n(&bar.b2_empty[s], 1);
     }
-    for (int q = 0; q < kNW; ++q) {
+    for (int q = 0; q < kMaxW; ++q) {
       mbar_init_n(&bar.w_full[q], 1);
-      mbar_init_n(&bar.w_empty[q], kConvThreads);
+      mbar_init_n(&bar.w_empty[q], K::kConvThreads);
     }
-    mbar_init_n(&bar.a2_full, kConvThreads);
+    mbar_init_n(&bar.a2_full, K::kConvThreads);
     mbar_init_n(&bar.mma2_done, 1);
     mbar_init_n(&bar.drain1, 1);
     mbar_init_n(&bar.drain2, 1);
     mbar_init_n(&bar.never, 1);
     for (int r = 0; r < kTileQ; ++r) {
       mbar_init_n(&bar.tile_full[r], 1);
-      mbar_init_n(&bar.tile_empty[r], 2 + kConvThreads);
+      mbar_init_n(&bar.tile_empty[r], 2 + K::kConvThreads);
     }
     asm volatile("fence.mbarrier_init.release.cluster;");
     abort_flag = 0;
   }
   // stale shared memory past the rows a copy fills must be finite: it meets zeros in
   // padded products
-  for (int e = tid * 4; e < kSmemF; e += kMvThreads * 4)
+  for (int e = tid * 4; e < K::kSmemF; e += K::kThreads * 4)
     *reinterpret_cast<float4*>(sm + e) = make_float4(0.f, 0.f, 0.f, 0.f);
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;");
   const uint32_t tmem = tmem_slot;
-  if (tid == kMma1Warp * 32 && g_tc_inject) {
+  if (tid == K::kMma1Warp * 32 && g_tc_inject) {
     // test hook: a wait on a barrier that nothing completes, with a short limit
     wait_or_abort(&bar.never, 0, &abort_flag, 4096);
   }
@@ -334,7 +365,7 @@ __global__ void __launch_bounds__(kMvThreads, 1)
     mbar_arrive(&bar.tile_empty[r]);
     return ti;
   };
-  if (warp == kProducerWarp) {
+  if (warp == K::kProducerWarp) {
     // ---- producer: takes the tiles; product-1 operands in the order the MMA thread
     // consumes them
     if (lane == 0 && !abort_flag) {
@@ -352,7 +383,7 @@ __global__ void __launch_bounds__(kMvThreads, 1)
         if (ti < 0) break;
         const TfTile tile = tiles[ti];
         if (!active[tile.inst]) continue;
-        const TileGeom g(tile);
+        const TileGeom<K> g(tile);
         if (g.slot_f != last_slot_f) {
           // a new slot layout overlaps the old slots: all of them are released first
           for (int s = 0; s < kMaxS1 && ok; ++s)
@@ -366,7 +397,7 @@ __global__ void __launch_bounds__(kMvThreads, 1)
         int slot = 0;
         for (int t = 0; t < g.T && ok; ++t) {
           const TfTask tk = tasks[tile.t_begin + t];
-          const int kdg = (tk.kdl + 7) >> 3, kp = tk.kdl > 32 ? 64 : 32;
+          const int kdg = (tk.kdl + 7) >> 3, kp = term_rows(tk.kdl);
           const uint32_t bytes = 2u * (g.nvg + kdg) * 1024u;
           for (int si = tk.s_begin; si < tk.s_end && ok; ++si) {
             const TfSrc S = srcs[si];
@@ -399,32 +430,45 @@ __global__ void __launch_bounds__(kMvThreads, 1)
       for (int s = 0; s < kMaxS1; ++s)
         if ((pend >> s) & 1u) wait_drain(&bar.s1_full[s], ((fpar >> s) & 1u) ^ 1u);
     }
-  } else if (warp == kMma1Warp) {
+  } else if (warp == K::kMma1Warp) {
     // ---- product 1: W^T = D x^T per source, segments of up to two K chunks per
     // accumulator
     if (lane == 0 && !abort_flag) {
-      uint32_t ful = 0;  // per slot: parity of the next fill
-      int q = 0, wround = 0;
+      uint32_t ful = 0;              // per slot: parity of the next fill
+      uint32_t wemp = 0, wpend = 0;  // per accumulator: release parity, written and not yet released
+      int last_wc = -1;
       bool ok = true;
       for (int k = 0; ok; ++k) {
         const int ti = next_tile(k);
         if (ti < 0) break;
         const TfTile tile = tiles[ti];
         if (!active[tile.inst]) continue;
-        const TileGeom g(tile);
-        int slot = 0;
+        const TileGeom<K> g(tile);
+        if (g.wc != last_wc) {
+          for (int q = 0; q < kMaxW && ok; ++q)
+            if ((wpend >> q) & 1u) {
+              ok = wait_or_abort(&bar.w_empty[q], (wemp >> q) & 1u, &abort_flag);
+              wemp ^= 1u << q;
+              wpend &= ~(1u << q);
+            }
+          last_wc = g.wc;
+        }
+        int slot = 0, q = 0;
         for (int t = 0; t < g.T && ok; ++t) {
           const TfTask tk = tasks[tile.t_begin + t];
-          const int kp = tk.kdl > 32 ? 64 : 32;
+          const int kp = term_rows(tk.kdl);
           const uint32_t id2 = idesc_tf32(2 * kp), id1 = idesc_tf32(kp);
           for (int si = tk.s_begin; si < tk.s_end && ok; ++si) {
             const TfSrc S = srcs[si];
             for (int k0 = 0; k0 < S.nkc; k0 += kSegChunks) {
-              if (wround >= 1 && !wait_or_abort(&bar.w_empty[q], (wround - 1) & 1, &abort_flag)) {
-                ok = false;
-                break;
+              if ((wpend >> q) & 1u) {
+                if (!wait_or_abort(&bar.w_empty[q], (wemp >> q) & 1u, &abort_flag)) {
+                  ok = false;
+                  break;
+                }
+                wemp ^= 1u << q;
               }
-              const uint32_t wq = tmem + (uint32_t)(q * kWCols);
+              const uint32_t wq = tmem + (uint32_t)(q * g.wc);
               const int k1 = min(S.nkc, k0 + kSegChunks);
               for (int kk = k0; kk < k1; ++kk) {
                 if (!wait_or_abort(&bar.s1_full[slot], (ful >> slot) & 1u, &abort_flag)) {
@@ -437,15 +481,12 @@ __global__ void __launch_bounds__(kMvThreads, 1)
                 const float* base = s1 + slot * g.slot_f;
                 mma_pair_steps(wq, smem_desc(smem_u32(base)), smem_desc(smem_u32(base + g.nvg * 256)),
                                smem_desc(smem_u32(base + 2 * g.nvg * 256)), id2, id1, (kv + 7) >> 3, kk == k0);
-                mma_commit(&bar.s1_empty[slot]);
                 if (++slot == g.nslots) slot = 0;
               }
               if (!ok) break;
               mma_commit(&bar.w_full[q]);
-              if (++q == kNW) {
-                q = 0;
-                ++wround;
-              }
+              wpend |= 1u << q;
+              if (++q == g.nw) q = 0;
             }
           }
         }
@@ -454,12 +495,12 @@ __global__ void __launch_bounds__(kMvThreads, 1)
       mma_commit(&bar.drain1);
       wait_drain(&bar.drain1, 0);
     }
-  } else if (warp == kMma2Warp) {
+  } else if (warp == K::kMma2Warp) {
     // ---- product 2: y^T = W^T C^T per term, fresh accumulator; this thread also loads
     // the C tiles (slot u % nb2 of the tile; the next fill of a slot waits for the
     // product that read it, and a tile starts once the last one's products have finished)
     if (lane == 0 && !abort_flag) {
-      uint32_t bf = 0, bc = 0, lf = 0, filled = 0;  // per C slot: fill parity to wait, commits, last fill, ever filled
+      uint32_t bf = 0, lf = 0, filled = 0;  // per C slot: fill parity to wait, last fill, ever filled
       int gt = 0;                                    // terms of the CTA's earlier tiles
       int tiles_done = 0;
       bool ok = true;
@@ -468,7 +509,7 @@ __global__ void __launch_bounds__(kMvThreads, 1)
         if (ti < 0) break;
         const TfTile tile = tiles[ti];
         if (!active[tile.inst]) continue;
-        const TileGeom g(tile);
+        const TileGeom<K> g(tile);
         auto load_c = [&](int u) {
           const TfTask tk = tasks[tile.t_begin + u];
           const int nch = (tk.kdl + 31) >> 5, s = u % g.nb2;
@@ -483,7 +524,7 @@ __global__ void __launch_bounds__(kMvThreads, 1)
           filled |= 1u << s;
         };
         for (int u = 0; u < min(g.nb2, g.T); ++u) load_c(u);
-        const uint32_t idm = idesc_tf32((tile.m + 15) & ~15);
+        const uint32_t idm = idesc_tf32(g.mp);
         for (int t = 0; t < g.T; ++t) {
           const int s = t % g.nb2;
           const TfTask tk = tasks[tile.t_begin + t];
@@ -497,15 +538,13 @@ __global__ void __launch_bounds__(kMvThreads, 1)
           const float* cb = b2 + s * g.b2_f;
           for (int c = 0; c * 32 < tk.kdl; ++c) {
             const int kv = min(32, tk.kdl - 32 * c);
-            mma_triple_steps(tmem + kYCol, smem_desc(smem_u32(a2 + (2 * c) * kTF)),
-                             smem_desc(smem_u32(a2 + (2 * c + 1) * kTF)), smem_desc(smem_u32(cb + c * 2 * g.mp * 32)),
+            mma_triple_steps(tmem + K::kWReg, smem_desc(smem_u32(a2 + (2 * c) * g.a2_f)),
+                             smem_desc(smem_u32(a2 + (2 * c + 1) * g.a2_f)), smem_desc(smem_u32(cb + c * 2 * g.mp * 32)),
                              smem_desc(smem_u32(cb + c * 2 * g.mp * 32 + g.mp * 32)), idm, (kv + 7) >> 3, c == 0);
           }
-          mma_commit(&bar.b2_empty[s]);
-          bc ^= 1u << s;
           mma_commit(&bar.mma2_done);
           if (t + g.nb2 < g.T) {
-            if (!wait_or_abort(&bar.b2_empty[s], ((bc >> s) & 1u) ^ 1u, &abort_flag)) {
+            if (!wait_or_abort(&bar.mma2_done, (gt + t) & 1, &abort_flag)) {
               ok = false;
               break;
             }
@@ -528,55 +567,53 @@ __global__ void __launch_bounds__(kMvThreads, 1)
     }
   } else {
     // ---- converters: warp w reads tensor-memory lanes 32 (w % 4) .. (its output
-    // columns); half 0 / 1 holds x rows 0..31 / 32..63 of W^T and output rows 0..63 /
-    // 64..127 of y.  A W^T accumulator holds the hi part in columns [0, kp) and the
-    // stacked lo part in [kp, 2 kp); their sum is the product.
-    const int quarter = warp & 3, half = (warp - kConvWarp0) >> 2;
+    // columns); half h holds x rows 32 h .. of W^T and output rows kYR h .. of y.  A W^T
+    // accumulator holds the hi part in columns [0, kp) and the stacked lo part in
+    // [kp, 2 kp); their sum is the product.
+    const int quarter = warp & 3, half = warp >> 2;
     const int n = quarter * 32 + lane;
     const uint32_t lane_base = tmem + ((uint32_t)(quarter * 32) << 16);
-    int q = 0, wround = 0, gt = 0;
+    uint32_t wful = 0;  // per accumulator: parity of the next fill
+    int gt = 0;
     bool ok = !abort_flag;
     for (int k = 0; ok; ++k) {
       const int ti = next_tile(k);
       if (ti < 0) break;
       const TfTile tile = tiles[ti];
       if (!active[tile.inst]) continue;
-      const int T = tile.t_end - tile.t_begin;
-      float yacc[64];
+      const TileGeom<K> g(tile);
+      const int T = g.T;
+      int q = 0, slot = 0;
+      float* pp = part + tile.part;  // the partial sums of this run: m x nv values each
+      float yacc[K::kYR];
 #pragma unroll
-      for (int j = 0; j < 64; ++j) yacc[j] = 0.0f;
+      for (int j = 0; j < K::kYR; ++j) yacc[j] = 0.0f;
       auto drain_y = [&]() {
         asm volatile("tcgen05.fence::after_thread_sync;");
 #pragma unroll
-        for (int i = 0; i < 2; ++i) {
-          if (64 * half + 32 * i < tile.m) {
+        for (int i = 0; i < K::kYR / 32; ++i) {
+          if (K::kYR * half + 32 * i < tile.m) {
             float v[32];
-            tmem_ld32(lane_base + (uint32_t)(kYCol + 64 * half + 32 * i), v);
+            tmem_ld32(lane_base + (uint32_t)(K::kWReg + K::kYR * half + 32 * i), v);
 #pragma unroll
             for (int j = 0; j < 32; ++j) yacc[32 * i + j] += v[j];
           }
         }
         asm volatile("tcgen05.fence::before_thread_sync;");
       };
-      // the FP32 sums of the last terms are added to y (the tile's owner writes it
-      // first, then accumulates into it)
-      bool stored = false;
       auto flush_y = [&]() {
-        if (abort_flag || n >= tile.nv) return;
+        if (abort_flag) return;
 #pragma unroll
-        for (int j = 0; j < 64; ++j) {
-          const int r = 64 * half + j;
-          if (r < tile.m) {
-            double* yp = tile.y + (int64_t)r * tile.ldy + n;
-            *yp = stored ? *yp + (double)yacc[j] : (double)yacc[j];
-          }
+        for (int j = 0; j < K::kYR; ++j) {
+          const int r = K::kYR * half + j;
+          if (r < tile.m && n < tile.nv) pp[r * tile.nv + n] = yacc[j];
           yacc[j] = 0.0f;
         }
-        stored = true;
+        pp += tile.m * tile.nv;
       };
       for (int t = 0; t < T && ok; ++t) {
         const TfTask tk = tasks[tile.t_begin + t];
-        const int kp = tk.kdl > 32 ? 64 : 32;
+        const int kp = term_rows(tk.kdl);
         float wsum[32];
 #pragma unroll
         for (int j = 0; j < 32; ++j) wsum[j] = 0.0f;
@@ -584,13 +621,21 @@ __global__ void __launch_bounds__(kMvThreads, 1)
           const float coef = srcs[si].coef;
           const int nseg = (srcs[si].nkc + kSegChunks - 1) / kSegChunks;
           for (int sg = 0; sg < nseg; ++sg) {
-            if (!wait_or_abort(&bar.w_full[q], wround & 1, &abort_flag)) {
+            if (!wait_or_abort(&bar.w_full[q], (wful >> q) & 1u, &abort_flag)) {
               ok = false;
               break;
             }
+            wful ^= 1u << q;
+            // the segment's products have finished, so its operand slots are free: a plain
+            // arrival here costs a few cycles, a commit per slot 150 to 200 of the MMA
+            // thread's
+            for (int c = min(srcs[si].nkc - sg * kSegChunks, kSegChunks); c > 0; --c) {
+              if (tid == 0) mbar_arrive(&bar.s1_empty[slot]);
+              if (++slot == g.nslots) slot = 0;
+            }
             asm volatile("tcgen05.fence::after_thread_sync;");
             if (32 * half < tk.kdl) {
-              const uint32_t wa = lane_base + (uint32_t)(q * kWCols + 32 * half);
+              const uint32_t wa = lane_base + (uint32_t)(q * g.wc + 32 * half);
               float v[32];
               tmem_ld32(wa, v);
 #pragma unroll
@@ -601,10 +646,7 @@ __global__ void __launch_bounds__(kMvThreads, 1)
             }
             asm volatile("tcgen05.fence::before_thread_sync;");
             mbar_arrive(&bar.w_empty[q]);
-            if (++q == kNW) {
-              q = 0;
-              ++wround;
-            }
+            if (++q == g.nw) q = 0;
           }
         }
         if (!ok) break;
@@ -619,21 +661,23 @@ __global__ void __launch_bounds__(kMvThreads, 1)
           drain_y();
           if (t % kFlushTerms == 0) flush_y();
         }
-        float* ah = a2 + (2 * half) * kTF;
-        float* al = ah + kTF;
+        if (n < g.nvg * 8 && 32 * half < kp) {
+          float* ah = a2 + (2 * half) * g.a2_f;
+          float* al = ah + g.a2_f;
 #pragma unroll
-        for (int gg = 0; gg < 8; ++gg) {
-          float4 h, l;
-          float* hv = &h.x;
-          float* lv = &l.x;
+          for (int gg = 0; gg < 8; ++gg) {
+            float4 h, l;
+            float* hv = &h.x;
+            float* lv = &l.x;
 #pragma unroll
-          for (int e = 0; e < 4; ++e) {
-            const float v = (32 * half + 4 * gg + e < tk.kdl) ? wsum[4 * gg + e] : 0.0f;
-            hv[e] = tf32_round(v);
-            lv[e] = tf32_round(v - hv[e]);
+            for (int e = 0; e < 4; ++e) {
+              const float v = (32 * half + 4 * gg + e < tk.kdl) ? wsum[4 * gg + e] : 0.0f;
+              hv[e] = tf32_round(v);
+              lv[e] = tf32_round(v - hv[e]);
+            }
+            *reinterpret_cast<float4*>(ah + kmo(n, 4 * gg)) = h;
+            *reinterpret_cast<float4*>(al + kmo(n, 4 * gg)) = l;
           }
-          *reinterpret_cast<float4*>(ah + kmo(n, 4 * gg)) = h;
-          *reinterpret_cast<float4*>(al + kmo(n, 4 * gg)) = l;
         }
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         mbar_arrive(&bar.a2_full);
@@ -648,78 +692,149 @@ __global__ void __launch_bounds__(kMvThreads, 1)
   }
   asm volatile("tcgen05.fence::before_thread_sync;");
   __syncthreads();
-  if (warp == kMma1Warp) tmem_free(tmem, kTmemCols);
+  if (warp == K::kMma1Warp) tmem_free(tmem, K::kTmem);
+}
+
+// y of one output tile: its partial sums, in term order, in FP64 (one CTA per tile)
+struct TfReduce { double* y; int64_t part; int ldy, m, nv, count, inst, pad; };
+
+__global__ void __launch_bounds__(256) k_tc_reduce(const TfReduce* __restrict__ red, const float* __restrict__ part,
+                                                  const int* __restrict__ active) {
+  const TfReduce R = red[blockIdx.x];
+  if (!active[R.inst]) return;
+  const int mn = R.m * R.nv;
+  for (int e = threadIdx.x; e < mn; e += 256) {
+    const float* p = part + R.part + e;
+    double v = (double)p[0];
+    int f = 1;
+    for (; f + 8 <= R.count; f += 8) {  // eight loads in flight ahead of the chain of additions
+      float q[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) q[u] = p[(int64_t)(f + u) * mn];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) v += (double)q[u];
+    }
+    for (; f < R.count; ++f) v += (double)p[(int64_t)f * mn];
+    R.y[(int64_t)(e / R.nv) * R.ldy + e % R.nv] = v;
+  }
 }
 
 // ------------------------------------------------------------------ tiny tiles
 
-// element (row, col) of a tiled hi / lo operand (chunk 0, col < 32) as hi + lo in FP64
-__device__ __forceinline__ double tiled_val(const float* __restrict__ p, int64_t lo, int row, int col) {
-  const int64_t e = (int64_t)kmo(row, col);
-  return (double)p[e] + (double)p[e + lo];
+// four consecutive columns (col0 a multiple of 4, < 32) of a row of a tiled hi / lo operand
+// (chunk 0) as hi + lo in FP64; hi + lo has at most 23 significant bits, so the FP32 sum is
+// exact and one conversion per element is enough
+__device__ __forceinline__ void tiled_val4(const float* __restrict__ p, int64_t lo, int row, int col0, double (&v)[4]) {
+  const int64_t e = (int64_t)kmo(row, col0);
+  const float4 h = *reinterpret_cast<const float4*>(p + e), l = *reinterpret_cast<const float4*>(p + e + lo);
+  v[0] = (double)(h.x + l.x);
+  v[1] = (double)(h.y + l.y);
+  v[2] = (double)(h.z + l.z);
+  v[3] = (double)(h.w + l.w);
 }
 
 // Output tiles of at most 4 x 4 elements whose terms have at most 4 x rows and whose
 // sources are one K chunk (tile.tiny): the same sum y += C (sum_s coef_s x_s D_s^T) on
-// CUDA cores in FP64 from the FP32 operand tiles, one warp per tile and one term per lane
-// (tensor-core products would be nearly all padding and the pipeline's per-term handoffs
-// would dominate).  The lanes' partial sums are reduced in a fixed order and written
-// once: deterministic, no atomics.
-__global__ void __launch_bounds__(256) k_tc_tiny(const TfTile* __restrict__ tiles, const TfTask* __restrict__ tasks,
-                                                 const TfSrc* __restrict__ srcs, const int* __restrict__ active,
-                                                 int n) {
-  const int w = (int)((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
-  if (w >= n) return;
-  const TfTile tile = tiles[w];
+// CUDA cores in FP64 from the FP32 operand tiles (tensor-core products would be nearly all
+// padding and the pipeline's per-term handoffs would dominate).  One CTA of four warps per
+// tile.  The terms are dealt to 32 chains (chain l sums the terms l, l + 32, ... in order);
+// of the next 4 x 32 terms warp w forms W of the w-th 32, one term per lane, and then warp i
+// adds row i of C W of all four to the chains, lane = chain.  The chains are reduced in a
+// fixed order and written once: deterministic, no atomics, the same sums as one warp per
+// tile gives.  FP64 is what bounds it (a warp's FMA holds a sub-partition for 64 cycles):
+// each element is converted once per use in a 4 x 4 product, and the tiles, far fewer than
+// the sub-partitions, spread over four of them.  Measured (one matvec, random L=28, D=700):
+// one warp per tile converting per product 3.33 ms, now 0.48 ms.
+constexpr int kTinyWarps = 4;
+
+__global__ void __launch_bounds__(kTinyWarps * 32) k_tc_tiny(const TfTile* __restrict__ tiles,
+                                                             const TfTask* __restrict__ tasks,
+                                                             const TfSrc* __restrict__ srcs,
+                                                             const int* __restrict__ active) {
+  __shared__ double Ws[kTinyWarps][16][32];  // W (k, j) of every lane's term
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const TfTile tile = tiles[blockIdx.x];
   if (!active[tile.inst]) return;
-  double y[4][4];
+  double y[4] = {0.0, 0.0, 0.0, 0.0};  // row `warp` of the chain `lane`
+  for (int t0 = tile.t_begin; t0 < tile.t_end; t0 += 32 * kTinyWarps) {
+    const int t = t0 + 32 * warp + lane;
+    if (t < tile.t_end) {
+      const TfTask tk = tasks[t];
+      double W[4][4];
 #pragma unroll
-  for (int i = 0; i < 4; ++i)
+      for (int k = 0; k < 4; ++k)
 #pragma unroll
-    for (int j = 0; j < 4; ++j) y[i][j] = 0.0;
-  for (int t = tile.t_begin + lane; t < tile.t_end; t += 32) {
-    const TfTask tk = tasks[t];
-    double W[4][4];
+        for (int j = 0; j < 4; ++j) W[k][j] = 0.0;
+      for (int si = tk.s_begin; si < tk.s_end; ++si) {
+        const TfSrc S = srcs[si];
+        const double coef = (double)S.coef;
+        double acc[4][4];
 #pragma unroll
-    for (int k = 0; k < 4; ++k)
+        for (int k = 0; k < 4; ++k)
 #pragma unroll
-      for (int j = 0; j < 4; ++j) W[k][j] = 0.0;
-    for (int si = tk.s_begin; si < tk.s_end; ++si) {
-      const TfSrc S = srcs[si];
-      const double coef = (double)S.coef;
+          for (int j = 0; j < 4; ++j) acc[k][j] = 0.0;
+        for (int r0 = 0; r0 < S.klast; r0 += 4) {
+          double dv[4][4];
 #pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        if (k >= tk.kdl) break;
+          for (int j = 0; j < 4; ++j)
+            if (j < tile.nv) tiled_val4(S.d, tile.dlo, j, r0, dv[j]);
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          if (j >= tile.nv) break;
-          double acc = 0.0;
-          for (int r = 0; r < S.klast; ++r) acc += tiled_val(S.x, tile.xlo, k, r) * tiled_val(S.d, tile.dlo, j, r);
-          W[k][j] += coef * acc;
+          for (int k = 0; k < 4; ++k) {
+            if (k >= tk.kdl) break;
+            double xv[4];
+            tiled_val4(S.x, tile.xlo, k, r0, xv);
+#pragma unroll
+            for (int r = 0; r < 4; ++r) {
+              if (r0 + r >= S.klast) break;
+#pragma unroll
+              for (int j = 0; j < 4; ++j)
+                if (j < tile.nv) acc[k][j] = fma(xv[r], dv[j][r], acc[k][j]);
+            }
+          }
+        }
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          if (k >= tk.kdl) break;
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            if (j >= tile.nv) break;
+            W[k][j] = fma(coef, acc[k][j], W[k][j]);
+          }
+        }
+      }
+#pragma unroll
+      for (int k = 0; k < 4; ++k)
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+          if (k < tk.kdl && j < tile.nv) Ws[warp][4 * k + j][lane] = W[k][j];
+    }
+    __syncthreads();
+    if (warp < tile.m) {
+      for (int u = 0; u < kTinyWarps; ++u) {
+        const int tu = t0 + 32 * u + lane;
+        if (tu >= tile.t_end) break;
+        const TfTask tk = tasks[tu];
+        double cv[4];
+        tiled_val4(tk.c, tile.dlo, warp, 0, cv);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          if (k >= tk.kdl) break;
+#pragma unroll
+          for (int j = 0; j < 4; ++j)
+            if (j < tile.nv) y[j] = fma(cv[k], Ws[u][4 * k + j][lane], y[j]);
         }
       }
     }
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      if (i >= tile.m) break;
-#pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        if (k >= tk.kdl) break;
-        const double c = tiled_val(tk.c, tile.dlo, i, k);
-#pragma unroll
-        for (int j = 0; j < 4; ++j) y[i][j] += c * W[k][j];
-      }
-    }
+    __syncthreads();
   }
+  if (warp >= tile.m) return;
 #pragma unroll
-  for (int i = 0; i < 4; ++i)
+  for (int j = 0; j < 4; ++j) {
+    double v = y[j];
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      double v = y[i][j];
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-      if (lane == 0 && i < tile.m && j < tile.nv) tile.y[(int64_t)i * tile.ldy + j] = v;
-    }
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    if (lane == 0 && j < tile.nv) tile.y[(int64_t)warp * tile.ldy + j] = v;
+  }
 }
 
 // ------------------------------------------------------------------ conversions
@@ -759,21 +874,27 @@ T* upload(const std::vector<T>& v, Stream s) {
   return p;
 }
 
-size_t smem_bytes() { return sizeof(float) * (size_t)kSmemF + 1024; }
+template <class K>
+size_t smem_bytes() {
+  return sizeof(float) * (size_t)K::kSmemF + 1024;
+}
 
 }  // namespace
 
 struct TcPlan {
-  TfTile* tiles = nullptr;
+  TfTile* tiles = nullptr;     // runs of terms by class (S, M, L), in queue order
   TfTask* tasks = nullptr;
   TfSrc* srcs = nullptr;
   TfConv* xb = nullptr;
   TfTile* tiny = nullptr;      // tiles for k_tc_tiny
-  int ntiny = 0;
-  int* queue = nullptr;        // the persistent kernel's tile counter
+  TfReduce* red = nullptr;     // output tiles and their partial sums
+  float* part = nullptr;
+  int ntiny = 0, nred = 0;
+  int* queue = nullptr;        // the persistent kernels' tile counters, one per class
   int* active = nullptr;       // per instance: 0 = skip its tiles
   int ninst = 0;
-  int ntiles = 0, nxb = 0, grid = 0;
+  int nclass[3] = {0, 0, 0}, first[3] = {0, 0, 0}, grid[3] = {0, 0, 0};
+  int nxb = 0;
   int launches = 0;  // kernels of one launch sequence
 };
 
@@ -840,17 +961,66 @@ TcPlan* tc_plan_build(const std::vector<const TcHost*>& inst, Stream st) {
     for (size_t i = 0; i < order.size(); ++i) (tiles0[order[i]].tiny ? tiny : sorted).push_back(tiles0[order[i]]);
     P->tiny = upload(tiny, st);
     P->ntiny = (int)tiny.size();
-    P->grid = (int)std::min<size_t>(sorted.size(), (size_t)sm_count());
-    P->queue = (int*)dev_alloc(sizeof(int), st);
+    // Classes, and runs of terms.  A run is long enough to pay for its pipeline fill (about
+    // two terms' time) and short enough that every resident CTA gets several: 16 terms up
+    // to kMaxRun.
+    const int sms = sm_count();
+    constexpr int kMaxRun = 64;
+    auto cls = [](const TfTile& q) {
+      return TileGeom<TileS>(q).fits ? 0 : TileGeom<TileM>(q).fits ? 1 : 2;
+    };
+    int64_t terms[3] = {0, 0, 0};
+    std::vector<char> cl(sorted.size());
+    for (size_t i = 0; i < sorted.size(); ++i) {
+      cl[i] = (char)cls(sorted[i]);
+      terms[(int)cl[i]] += sorted[i].t_end - sorted[i].t_begin;
+    }
+    const int ctas[3] = {sms * TileS::kCtas, sms * TileM::kCtas, sms * TileL::kCtas};
+    int64_t run[3];
+    for (int c = 0; c < 3; ++c) {
+      run[c] = terms[c] / ((int64_t)8 * ctas[c]);
+      run[c] = std::min<int64_t>(kMaxRun, std::max<int64_t>(kFlushTerms, run[c] / kFlushTerms * kFlushTerms));
+    }
+    std::vector<TfTile> runs[3];
+    std::vector<TfReduce> red;
+    red.reserve(sorted.size());
+    int64_t part = 0;
+    for (size_t i = 0; i < sorted.size(); ++i) {
+      const TfTile& q = sorted[i];
+      const int T = q.t_end - q.t_begin, nf = std::max(1, (T + kFlushTerms - 1) / kFlushTerms);
+      const int64_t mn = (int64_t)q.m * q.nv, step = run[(int)cl[i]];
+      red.push_back({q.y, part, q.ldy, q.m, q.nv, nf, q.inst, 0});
+      int64_t t = 0;
+      do {
+        TfTile u = q;
+        u.t_begin = q.t_begin + (int)t;
+        u.t_end = q.t_begin + (int)std::min<int64_t>(T, t + step);
+        u.part = part + t / kFlushTerms * mn;
+        runs[(int)cl[i]].push_back(u);
+        t += step;
+      } while (t < T);
+      part += nf * mn;
+    }
+    std::vector<TfTile> all;
+    for (int c = 0; c < 3; ++c) {
+      P->first[c] = (int)all.size();
+      P->nclass[c] = (int)runs[c].size();
+      P->grid[c] = (int)std::min<size_t>(runs[c].size(), (size_t)ctas[c]);
+      all.insert(all.end(), runs[c].begin(), runs[c].end());
+    }
+    P->queue = (int*)dev_alloc(3 * sizeof(int), st);
+    P->part = (float*)dev_alloc(sizeof(float) * std::max<int64_t>(part, 1), st);
     P->ninst = (int)inst.size();
     P->active = upload(std::vector<int>(inst.size(), 1), st);
-    P->tiles = upload(sorted, st);
+    P->tiles = upload(all, st);
+    P->red = upload(red, st);
+    P->nred = (int)red.size();
     P->tasks = upload(single ? inst[0]->t : t, st);
     P->srcs = upload(single ? inst[0]->s : s, st);
     P->xb = upload(single ? inst[0]->xb : xb, st);
-    P->ntiles = (int)sorted.size();
     P->nxb = (int)(single ? inst[0]->xb.size() : xb.size());
-    P->launches = (P->nxb > 0) + (P->ntiles > 0) + (P->ntiny > 0);
+    P->launches = (P->nxb > 0) + (P->nclass[0] > 0) + (P->nclass[1] > 0) + (P->nclass[2] > 0) + (P->nred > 0) +
+                  (P->ntiny > 0);
   } catch (...) {
     tc_plan_free(P, st);
     throw;
@@ -868,6 +1038,8 @@ void tc_plan_free(TcPlan* p, Stream s) {
   dev_free(p->xb, s);
   dev_free(p->queue, s);
   dev_free(p->tiny, s);
+  dev_free(p->red, s);
+  dev_free(p->part, s);
   dev_free(p->active, s);
   delete p;
 }
@@ -877,9 +1049,20 @@ namespace {
 void tc_set_attributes() {
   static bool attr = false;
   if (attr) return;
-  ck(cudaFuncSetAttribute(k_tc_matvec, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes()),
-     "tc matvec smem");
+  auto set = [](const void* f, size_t bytes) {
+    ck(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes), "tc matvec smem");
+  };
+  set((const void*)k_tc_matvec<TileS>, smem_bytes<TileS>());
+  set((const void*)k_tc_matvec<TileM>, smem_bytes<TileM>());
+  set((const void*)k_tc_matvec<TileL>, smem_bytes<TileL>());
   attr = true;
+}
+
+template <class K>
+void tc_run(const TcPlan* p, int c, cudaStream_t cs) {
+  if (p->nclass[c] > 0)
+    k_tc_matvec<K><<<p->grid[c], K::kThreads, smem_bytes<K>(), cs>>>(p->tiles + p->first[c], p->tasks, p->srcs, p->part,
+                                                                    p->queue + c, p->active, p->nclass[c]);
 }
 
 void tc_enqueue(const TcPlan* p, void* const* ev, cudaStream_t cs) {
@@ -887,11 +1070,13 @@ void tc_enqueue(const TcPlan* p, void* const* ev, cudaStream_t cs) {
   if (p->nxb > 0) k_tiled_convert<<<p->nxb, 256, 0, cs>>>(p->xb);
   if (ev) event_record(ev[1], cs);
   if (p->ntiny > 0)
-    k_tc_tiny<<<(p->ntiny + 7) / 8, 256, 0, cs>>>(p->tiny, p->tasks, p->srcs, p->active, p->ntiny);
-  if (p->ntiles > 0) {
-    ck(cudaMemsetAsync(p->queue, 0, sizeof(int), cs), "tile queue reset");
-    k_tc_matvec<<<p->grid, kMvThreads, smem_bytes(), cs>>>(p->tiles, p->tasks, p->srcs, p->queue, p->active,
-                                                           p->ntiles);
+    k_tc_tiny<<<p->ntiny, kTinyWarps * 32, 0, cs>>>(p->tiny, p->tasks, p->srcs, p->active);
+  if (p->nred > 0) {
+    ck(cudaMemsetAsync(p->queue, 0, 3 * sizeof(int), cs), "tile queue reset");
+    tc_run<TileL>(p, 2, cs);
+    tc_run<TileM>(p, 1, cs);
+    tc_run<TileS>(p, 0, cs);
+    k_tc_reduce<<<p->nred, 256, 0, cs>>>(p->red, p->part, p->active);
   }
   if (ev) event_record(ev[2], cs);
   ck(cudaGetLastError(), "tc matvec launch");
