@@ -420,7 +420,7 @@ int dmrg_truncate(dmrg_ctx* c, int site, int dir, int D, double noise, const dou
     if (stream) dmrg::dev_d2d(dx.p, x, sizeof(double) * n, s);
     else dmrg::dev_h2d(dx.p, x, sizeof(double) * n, s);
     if (noise > 0) dmrg::vec_add_noise(dx.p, n, noise, 0x7a11u + (uint64_t)site, s);
-    double w = c->eng->truncate(site, dir, D, dx.p, noise);
+    double w = c->eng->truncate(site, dir, D, dx.p, true);
     dmrg::dev_sync(s);
     if (w_disc) *w_disc = w;
     return DMRG_OK;

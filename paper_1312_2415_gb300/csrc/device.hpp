@@ -180,6 +180,14 @@ struct EigJob {
   int n;
 };
 void eig_batched(const std::vector<EigJob>& jobs, Stream s);
+// the same for Gram matrices A = op(M)^T op(M), by FP32 Jacobi passes refined with FP64
+// products of M (other rounding; A is only read where a job is not handed to eig_batched):
+// op(M) is M^T (trans = 1) or M, inner x n
+struct EigSource {
+  const double* M;
+  int ld, inner, trans;
+};
+void eig_refined(const std::vector<EigJob>& jobs, const std::vector<EigSource>& src, Stream s);
 
 // ---- global selection of the D largest values (ties: earlier group, lower index) ----
 // vals: concatenated eigenvalues (lambda^2) of groups with offsets goff (size G+1);

@@ -2023,7 +2023,10 @@ namespace dmrg {
 // its side (M M^T for U, M^T M for V); the other factor is the projection of M onto
 // them (kappa V = U^T M / |M|, U kappa = M V^T / |M|), with no division by lambda.
 // Returns the discarded weight sum over dropped (2jM+1) kappa^2 (Eq. 15).
-double Engine::truncate(int i, int dir, int D, const double* x, double /*unused*/) {
+// refined: decompose by eig_refined (the call on its own).  A sweep step keeps the Jacobi
+// solver, bit for bit: its Davidson may have stopped at the iteration cap, where a difference
+// of 1e-15 in the state grows a hundredfold per iteration of the next step.
+double Engine::truncate(int i, int dir, int D, const double* x, bool refined) {
   check_ready();
   if (i < 0 || i > L_ - 2) throw std::out_of_range("site out of range");
   Timer tm;
@@ -2147,7 +2150,13 @@ double Engine::truncate(int i, int dir, int D, const double* x, double /*unused*
   }
   std::vector<EigJob> jobs;
   for (auto& g : gs) jobs.push_back({Gm + g.goff, Q + g.goff, W + g.woff, g.n});
-  eig_batched(jobs, stream_);
+  if (refined) {
+    std::vector<EigSource> src;  // dir > 0: the Gram matrix is M M^T, otherwise M^T M
+    for (auto& g : gs) src.push_back({M + g.moff, g.C, dir > 0 ? g.C : g.R, dir > 0 ? 1 : 0});
+    eig_refined(jobs, src, stream_);
+  } else {
+    eig_batched(jobs, stream_);
+  }
   std::vector<int> goff(1, 0), wgt;
   for (auto& g : gs) { goff.push_back(goff.back() + g.n); wgt.push_back(g.s.tj + 1); }
   std::vector<int> kept;
@@ -3092,7 +3101,7 @@ double Engine::sweep_step(int i, int dir, int D, double gamma, double* w_disc, i
   double w;
   bool keep = false;
   try {
-    w = truncate(i, dir, D, x, 0.0);
+    w = truncate(i, dir, D, x, false);
     half_wmax_ = std::max(half_wmax_, w);
     launch_rq();  // after the decomposition, whose kernels would otherwise queue behind it
     if (dir > 0) update_left_from(i, P->cl);

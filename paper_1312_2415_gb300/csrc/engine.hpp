@@ -144,7 +144,7 @@ class Engine {
   // quotient of the tensor-core Ritz vector): with defer set the FP64 matvec is queued on
   // a side stream and the energy is collected by finish_rq()
   double davidson_ex(int i, double* x_dev, int* iters, bool* converged, bool defer);
-  double truncate(int i, int dir, int D, const double* x_dev, double noise);
+  double truncate(int i, int dir, int D, const double* x_dev, bool refined);
   double solve(double* e_last);
   // one micro-iteration of a sweep at sites (i, i+1): Eq. 25, Davidson, noise,
   // Eqs. 26-28 and the operator update in the sweep direction

@@ -1191,6 +1191,73 @@ __global__ void __launch_bounds__(NT) k_eig_batched(const EigJob* __restrict__ j
 // ------------------------------------------------------------------ parallel block Jacobi
 
 namespace {
+// round-robin pairing of np (even) indices: pair r of a step
+__device__ __forceinline__ void rr_pair(int r, int step, int np, int& p, int& q) {
+  const int b = np - 1 - r;
+  p = r == 0 ? 0 : 1 + (r - 1 + step) % (np - 1);
+  q = 1 + (b - 1 + step) % (np - 1);
+  if (p > q) { const int t = p; p = q; q = t; }
+}
+
+// Cyclic Jacobi in FP32 on the np x np matrix A (np even, at most 64, row stride ld) in
+// shared memory, the rotations accumulated into Q, by a CTA of 256 threads: at most `sweeps`
+// sweeps, ended by one without an off-diagonal above floor_abs (pairs are rotated from a
+// tenth of that on).  A step has two barriers: one warp computes the
+// rotations, then every thread updates whole 2 x 2 blocks J_r^T A J_u (lane = pair u, warps
+// stride over r, four blocks' loads in flight) and columns of Q.
+__device__ void jacobi_f32(float* A, float* Q, int np, int ld, int sweeps, float floor_abs, float* cs, float* sn, int* pp,
+                           int* qq, int* flag) {
+  const int tid = threadIdx.x, nr = np / 2, lane = tid & 31, warp = tid >> 5;
+  for (int sweep = 0; sweep < sweeps; ++sweep) {
+    if (tid == 0) *flag = 0;
+    __syncthreads();
+    for (int step = 0; step < np - 1; ++step) {
+      if (tid < nr) {
+        int p, q;
+        rr_pair(tid, step, np, p, q);
+        const float app = A[p * ld + p], aqq = A[q * ld + q], apq = A[p * ld + q];
+        float c = 1.0f, s = 0.0f;
+        if (fabsf(apq) > 0.1f * floor_abs) {
+          const float th = __fdividef(aqq - app, 2.0f * apq), at = fabsf(th);
+          const float t = copysignf(at < 1e18f ? __fdividef(1.0f, at + sqrtf(fmaf(at, at, 1.0f))) : 0.0f, th);
+          c = rsqrtf(fmaf(t, t, 1.0f));
+          s = t * c;
+          if (fabsf(apq) > floor_abs) *flag = 1;
+        }
+        cs[tid] = c; sn[tid] = s; pp[tid] = p; qq[tid] = q;
+      }
+      __syncthreads();
+      if (lane < nr) {
+        const float cu = cs[lane], su = sn[lane];
+        const int v = pp[lane], w = qq[lane];
+#pragma unroll 4
+        for (int r = warp; r < nr; r += 8) {
+          const float cr = cs[r], sr = sn[r];
+          const int p = pp[r] * ld, q = qq[r] * ld;
+          const float a0 = A[p + v], a1 = A[p + w], b0 = A[q + v], b1 = A[q + w];
+          const float x0 = cr * a0 - sr * b0, x1 = cr * a1 - sr * b1, y0 = sr * a0 + cr * b0, y1 = sr * a1 + cr * b1;
+          A[p + v] = cu * x0 - su * x1;
+          A[p + w] = r == lane ? 0.0f : su * x0 + cu * x1;
+          A[q + v] = r == lane ? 0.0f : cu * y0 - su * y1;
+          A[q + w] = su * y0 + cu * y1;
+        }
+#pragma unroll 8
+        for (int i = warp; i < np; i += 8) {  // columns of Q
+          float* row = Q + i * ld;
+          const float a0 = row[v], a1 = row[w];
+          row[v] = cu * a0 - su * a1;
+          row[w] = su * a0 + cu * a1;
+        }
+      }
+      __syncthreads();
+    }
+    if (!*flag) break;
+    __syncthreads();
+  }
+}
+}  // namespace
+
+namespace {
 // Symmetric eigensolver for the large Gram blocks (n above the shared-memory limit): a
 // two-sided block Jacobi.  Rows and columns are grouped in blocks of 32; each step of
 // a round-robin tournament pairs the blocks, and for every pair (I, J) the 64 x 64
@@ -1204,9 +1271,10 @@ constexpr int kOB = 32;   // rows per block
 constexpr int kOP = 64;   // rows per pair
 constexpr int kOL = 65;   // shared-memory row stride (doubles)
 
+template <class T>
 struct BjJob {
-  double* A;      // n x n symmetric (the Gram matrix), diagonalised in place
-  double* Q;      // n x n accumulated rotations (eigenvectors as columns)
+  T* A;           // n x n symmetric (the Gram matrix), diagonalised in place
+  T* Q;           // n x n accumulated rotations (eigenvectors as columns)
   double* w;      // n eigenvalues (output, descending)
   int n, nb;      // nb = number of row blocks, even
   int pair_begin; // first CTA of this job in a step launch
@@ -1274,15 +1342,15 @@ __device__ void cta_jacobi64(double* A, double* V, double* cs, double* sn, int* 
 
 // out(64 x 64 tile) = op(X) op(Y) with a 4 x 4 register tile per thread; X, Y in shared
 // memory with stride kOL; tx / ty: transpose flags
-template <bool TX, bool TY>
-__device__ __forceinline__ void tile64(const double* X, const double* Y, double (&acc)[4][4]) {
+template <bool TX, bool TY, class T>
+__device__ __forceinline__ void tile64(const T* X, const T* Y, T (&acc)[4][4]) {
   const int ti = threadIdx.x >> 4, tj = threadIdx.x & 15;
 #pragma unroll
   for (int u = 0; u < 4; ++u)
 #pragma unroll
-    for (int v = 0; v < 4; ++v) acc[u][v] = 0.0;
+    for (int v = 0; v < 4; ++v) acc[u][v] = T(0);
   for (int k = 0; k < kOP; ++k) {
-    double x[4], y[4];
+    T x[4], y[4];
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
       x[u] = TX ? X[k * kOL + ti * 4 + u] : X[(ti * 4 + u) * kOL + k];
@@ -1295,7 +1363,8 @@ __device__ __forceinline__ void tile64(const double* X, const double* Y, double 
   }
 }
 
-__device__ __forceinline__ int find_job(const BjJob* jobs, int njobs) {
+template <class T>
+__device__ __forceinline__ int find_job(const BjJob<T>* jobs, int njobs) {
   int lo = 0, hi = njobs - 1;
   while (lo < hi) {
     const int mid = (lo + hi + 1) >> 1;
@@ -1304,7 +1373,8 @@ __device__ __forceinline__ int find_job(const BjJob* jobs, int njobs) {
   return lo;
 }
 
-__device__ __forceinline__ void pair_rows(const BjJob& J, int r, int step, int* idx) {
+template <class T>
+__device__ __forceinline__ void pair_rows(const BjJob<T>& J, int r, int step, int* idx) {
   const int a = r, b = J.nb - 1 - r;
   const int p = a == 0 ? 0 : 1 + (a - 1 + step) % (J.nb - 1);
   const int q = b == 0 ? 0 : 1 + (b - 1 + step) % (J.nb - 1);
@@ -1315,8 +1385,8 @@ __device__ __forceinline__ void pair_rows(const BjJob& J, int r, int step, int* 
 }
 
 // Q = identity, and the largest |diagonal| of A per job (the noise scale eps |G|)
-__global__ void k_bj_prep(const BjJob* __restrict__ jobs, double* __restrict__ gmax) {
-  const BjJob J = jobs[blockIdx.x];
+__global__ void k_bj_prep(const BjJob<double>* __restrict__ jobs, double* __restrict__ gmax) {
+  const BjJob<double> J = jobs[blockIdx.x];
   const int n = J.n;
   for (int64_t e = threadIdx.x; e < (int64_t)n * n; e += blockDim.x) J.Q[e] = (e / n == e % n) ? 1.0 : 0.0;
   double best = 0.0;
@@ -1331,18 +1401,43 @@ __global__ void k_bj_prep(const BjJob* __restrict__ jobs, double* __restrict__ g
   if (threadIdx.x == 0) gmax[blockIdx.x] = red[0];
 }
 
+// What the two element types ask of a pair: an off-diagonal above rel sqrt|g_ii g_jj| +
+// abs |G| sends it to the inner solver (|G| = the largest diagonal entry).  FP64: below that
+// it is rounding noise of the rotations (~eps sqrt(64) |G|) and moves the eigenvalues only at
+// second order; the absolute part must stay above the inner solver's floor, or pairs of
+// null-space directions would be sent back to it forever.  FP32 (passes whose result is
+// refined): the pass's floor alone.
+template <class T>
+struct BjTol;
+template <>
+struct BjTol<double> {
+  static constexpr double rel = 1e-14, abs = 1e-14;
+};
+template <>
+struct BjTol<float> {
+  static constexpr double rel = 0.0, abs = 1.0;  // gmax carries the pass's floor
+};
+
+__device__ __forceinline__ void bj_inner(double* S, double* V, double* cs, double* sn, int* pq, int* nrot, double gmax) {
+  cta_jacobi64(S, V, cs, sn, pq, nrot, 1e-16 * gmax);  // floor below the outer one
+}
+__device__ __forceinline__ void bj_inner(float* S, float* V, float* cs, float* sn, int* pq, int* nrot, double gmax) {
+  jacobi_f32(S, V, kOP, kOL, 1, (float)(BjTol<float>::abs * gmax), cs, sn, pq, pq + kOP / 2, nrot);
+}
+
 // step, part 1: V of every pair from its diagonal sub-block (one CTA per pair)
-__global__ void __launch_bounds__(256) k_bj_rows(const BjJob* __restrict__ jobs, int njobs, int step,
-                                                 const double* __restrict__ gmax, double* __restrict__ vbuf,
+template <class T>
+__global__ void __launch_bounds__(256) k_bj_rows(const BjJob<T>* __restrict__ jobs, int njobs, int step,
+                                                 const double* __restrict__ gmax, T* __restrict__ vbuf,
                                                  int* __restrict__ flag, int* __restrict__ nrot) {
   extern __shared__ double bsm[];
-  double* S = bsm;              // sub-block, then diagonalised
-  double* V = S + kOP * kOL;    // its eigenvectors
-  __shared__ double cs[kOP / 2], sn[kOP / 2];
+  T* S = reinterpret_cast<T*>(bsm);  // sub-block, then diagonalised
+  T* V = S + kOP * kOL;              // its eigenvectors
+  __shared__ T cs[kOP / 2], sn[kOP / 2];
   __shared__ int pq[kOP], idx[kOP];
   __shared__ int inner_rot, need;
   const int lo = find_job(jobs, njobs);
-  const BjJob J = jobs[lo];
+  const BjJob<T> J = jobs[lo];
   const int r = blockIdx.x - J.pair_begin, tid = threadIdx.x, n = J.n;
   if (r >= J.nb / 2 || step >= J.nb - 1) {
     if (tid == 0) flag[blockIdx.x] = 0;
@@ -1351,33 +1446,29 @@ __global__ void __launch_bounds__(256) k_bj_rows(const BjJob* __restrict__ jobs,
   pair_rows(J, r, step, idx);
   if (tid == 0) need = 0;
   __syncthreads();
-  // Rotate while an off-diagonal exceeds 1e-14 sqrt|g_ii g_jj| + 1e-14 |G| (|G| = the
-  // largest diagonal entry): below that it is rounding noise of the rotations (~eps
-  // sqrt(64) |G|), and it moves the eigenvalues only at second order.  The absolute part
-  // must stay above the inner solver's floor, or pairs of null-space directions would
-  // be sent back to it forever.
-  const double fl = 1e-14 * gmax[lo];
+  const T rel = (T)BjTol<T>::rel, fl = (T)(BjTol<T>::abs * gmax[lo]);
   for (int e = tid; e < kOP * kOP; e += 256) {
     const int i = e >> 6, j = e & 63;
-    S[i * kOL + j] = (idx[i] >= 0 && idx[j] >= 0) ? J.A[(size_t)idx[i] * n + idx[j]] : 0.0;
+    S[i * kOL + j] = (idx[i] >= 0 && idx[j] >= 0) ? J.A[(size_t)idx[i] * n + idx[j]] : T(0);
   }
   __syncthreads();
   for (int e = tid; e < kOP * kOP; e += 256) {
     const int i = e >> 6, j = e & 63;
-    if (i < j && fabs(S[i * kOL + j]) > 1e-14 * sqrt(fabs(S[i * kOL + i] * S[j * kOL + j])) + fl) need = 1;
+    if (i < j && fabs(S[i * kOL + j]) > rel * sqrt(fabs(S[i * kOL + i] * S[j * kOL + j])) + fl) need = 1;
   }
   __syncthreads();
   if (!need) {
     if (tid == 0) flag[blockIdx.x] = 0;
     return;
   }
-  for (int e = tid; e < kOP * kOL; e += 256) V[e] = ((e / kOL) == (e % kOL)) ? 1.0 : 0.0;
+  for (int e = tid; e < kOP * kOL; e += 256) V[e] = ((e / kOL) == (e % kOL)) ? T(1) : T(0);
   __syncthreads();
-  cta_jacobi64(S, V, cs, sn, pq, &inner_rot, 1e-16 * gmax[lo]);  // floor below the outer one
+  bj_inner(S, V, cs, sn, pq, &inner_rot, gmax[lo]);
+  __syncthreads();
   // one Newton-Schulz step V <- V (3 I - V^T V) / 2 against the rounding of the rotations
   {
-    double acc[4][4];
-    tile64<true, false>(V, V, acc);  // V^T V
+    T acc[4][4];
+    tile64<true, false, T>(V, V, acc);  // V^T V
     __syncthreads();
     const int ti = tid >> 4, tj = tid & 15;
 #pragma unroll
@@ -1385,10 +1476,10 @@ __global__ void __launch_bounds__(256) k_bj_rows(const BjJob* __restrict__ jobs,
 #pragma unroll
       for (int v = 0; v < 4; ++v) {
         const int i = ti * 4 + u, j = tj * 4 + v;
-        S[i * kOL + j] = (i == j ? 1.5 : 0.0) - 0.5 * acc[u][v];
+        S[i * kOL + j] = (i == j ? T(1.5) : T(0)) - T(0.5) * acc[u][v];
       }
     __syncthreads();
-    tile64<false, false>(V, S, acc);
+    tile64<false, false, T>(V, S, acc);
     __syncthreads();
 #pragma unroll
     for (int u = 0; u < 4; ++u)
@@ -1396,7 +1487,7 @@ __global__ void __launch_bounds__(256) k_bj_rows(const BjJob* __restrict__ jobs,
       for (int v = 0; v < 4; ++v) V[(ti * 4 + u) * kOL + tj * 4 + v] = acc[u][v];
     __syncthreads();
   }
-  double* vg = vbuf + (size_t)blockIdx.x * kOP * kOP;
+  T* vg = vbuf + (size_t)blockIdx.x * kOP * kOP;
   for (int e = tid; e < kOP * kOP; e += 256) vg[e] = V[(e >> 6) * kOL + (e & 63)];
   if (tid == 0) {
     flag[blockIdx.x] = 1;
@@ -1405,29 +1496,30 @@ __global__ void __launch_bounds__(256) k_bj_rows(const BjJob* __restrict__ jobs,
 }
 
 // step, part 2: rows I+J of A <- V^T rows I+J, one 64-column chunk per CTA (grid.y)
-__global__ void __launch_bounds__(256) k_bj_rowapply(const BjJob* __restrict__ jobs, int njobs, int step,
-                                                     const double* __restrict__ vbuf, const int* __restrict__ flag) {
+template <class T>
+__global__ void __launch_bounds__(256) k_bj_rowapply(const BjJob<T>* __restrict__ jobs, int njobs, int step,
+                                                     const T* __restrict__ vbuf, const int* __restrict__ flag) {
   extern __shared__ double bsm[];
-  double* V = bsm;
-  double* buf = V + kOP * kOL;
+  T* V = reinterpret_cast<T*>(bsm);
+  T* buf = V + kOP * kOL;
   __shared__ int idx[kOP];
   if (!flag[blockIdx.x]) return;
   const int lo = find_job(jobs, njobs);
-  const BjJob J = jobs[lo];
+  const BjJob<T> J = jobs[lo];
   const int r = blockIdx.x - J.pair_begin, tid = threadIdx.x, n = J.n;
   const int c0 = blockIdx.y * kOP;
   if (c0 >= n) return;
   pair_rows(J, r, step, idx);
-  const double* vg = vbuf + (size_t)blockIdx.x * kOP * kOP;
+  const T* vg = vbuf + (size_t)blockIdx.x * kOP * kOP;
   for (int e = tid; e < kOP * kOP; e += 256) V[(e >> 6) * kOL + (e & 63)] = vg[e];
   __syncthreads();
   for (int e = tid; e < kOP * kOP; e += 256) {
     const int i = e >> 6, k = e & 63;
-    buf[i * kOL + k] = (idx[i] >= 0 && c0 + k < n) ? J.A[(size_t)idx[i] * n + c0 + k] : 0.0;
+    buf[i * kOL + k] = (idx[i] >= 0 && c0 + k < n) ? J.A[(size_t)idx[i] * n + c0 + k] : T(0);
   }
   __syncthreads();
-  double acc[4][4];
-  tile64<true, false>(V, buf, acc);
+  T acc[4][4];
+  tile64<true, false, T>(V, buf, acc);
   const int ti = tid >> 4, tj = tid & 15;
 #pragma unroll
   for (int u = 0; u < 4; ++u) {
@@ -1441,31 +1533,32 @@ __global__ void __launch_bounds__(256) k_bj_rowapply(const BjJob* __restrict__ j
 
 // step, part 3: columns I+J of A (grid.z = 0) and of Q (grid.z = 1) <- columns times V,
 // one 64-row chunk per CTA (grid.y)
-__global__ void __launch_bounds__(256) k_bj_cols(const BjJob* __restrict__ jobs, int njobs, int step,
-                                                 const double* __restrict__ vbuf, const int* __restrict__ flag) {
+template <class T>
+__global__ void __launch_bounds__(256) k_bj_cols(const BjJob<T>* __restrict__ jobs, int njobs, int step,
+                                                 const T* __restrict__ vbuf, const int* __restrict__ flag) {
   extern __shared__ double bsm[];
-  double* V = bsm;
-  double* buf = V + kOP * kOL;
+  T* V = reinterpret_cast<T*>(bsm);
+  T* buf = V + kOP * kOL;
   __shared__ int idx[kOP];
   if (!flag[blockIdx.x]) return;
   const int lo = find_job(jobs, njobs);
-  const BjJob J = jobs[lo];
+  const BjJob<T> J = jobs[lo];
   const int r = blockIdx.x - J.pair_begin, tid = threadIdx.x, n = J.n;
   pair_rows(J, r, step, idx);
-  const double* vg = vbuf + (size_t)blockIdx.x * kOP * kOP;
+  const T* vg = vbuf + (size_t)blockIdx.x * kOP * kOP;
   for (int e = tid; e < kOP * kOP; e += 256) V[(e >> 6) * kOL + (e & 63)] = vg[e];
   __syncthreads();
   const int ti = tid >> 4, tj = tid & 15;
-  double* M = blockIdx.z == 0 ? J.A : J.Q;
+  T* M = blockIdx.z == 0 ? J.A : J.Q;
   const int r0 = blockIdx.y * kOP;
   if (r0 >= n) return;
   for (int e = tid; e < kOP * kOP; e += 256) {
     const int rr = e >> 6, k = e & 63;
-    buf[rr * kOL + k] = (idx[k] >= 0 && r0 + rr < n) ? M[(size_t)(r0 + rr) * n + idx[k]] : 0.0;
+    buf[rr * kOL + k] = (idx[k] >= 0 && r0 + rr < n) ? M[(size_t)(r0 + rr) * n + idx[k]] : T(0);
   }
   __syncthreads();
-  double acc[4][4];
-  tile64<false, false>(buf, V, acc);
+  T acc[4][4];
+  tile64<false, false, T>(buf, V, acc);
 #pragma unroll
   for (int u = 0; u < 4; ++u) {
     const int rr = r0 + ti * 4 + u;
@@ -1480,8 +1573,8 @@ __global__ void __launch_bounds__(256) k_bj_cols(const BjJob* __restrict__ jobs,
 
 // eigenvalues = diagonal of the rotated A, sorted descending (ties by index) with the
 // normalised columns of Q; A is scratch for the unsorted eigenvectors
-__global__ void k_bj_finish(const BjJob* __restrict__ jobs) {
-  const BjJob J = jobs[blockIdx.x];
+__global__ void k_bj_finish(const BjJob<double>* __restrict__ jobs) {
+  const BjJob<double> J = jobs[blockIdx.x];
   const int n = J.n, tid = threadIdx.x;
   extern __shared__ double wn[];
   double* qn = wn + n;
@@ -1506,45 +1599,42 @@ __global__ void k_bj_finish(const BjJob* __restrict__ jobs) {
   }
 }
 
-}  // namespace
-
-static void eig_block_jacobi(const std::vector<EigJob>& jobs, Stream s) {
-  if (jobs.empty()) return;
-  std::vector<BjJob> bj;
+// Block-Jacobi sweeps over the jobs (A and Q in place) until no pair needs one, at most
+// `sweeps`; gmax: the largest diagonal entry of every job (device).
+template <class T>
+void bj_sweeps(std::vector<BjJob<T>>& bj, const double* gmax, int sweeps, Stream s) {
+  if (bj.empty()) return;
   int pairs = 0, nbmax = 0, nmax = 0;
-  for (const EigJob& j : jobs) {
-    int nb = (j.n + kOB - 1) / kOB;
-    nb += nb & 1;
-    bj.push_back({j.A, j.Q, j.w, j.n, nb, pairs, 0});
-    pairs += nb / 2;
-    nbmax = std::max(nbmax, nb);
+  for (auto& j : bj) {
+    j.nb = (j.n + kOB - 1) / kOB;
+    j.nb += j.nb & 1;
+    j.pair_begin = pairs;
+    pairs += j.nb / 2;
+    nbmax = std::max(nbmax, j.nb);
     nmax = std::max(nmax, j.n);
   }
   const int nj = (int)bj.size();
   const int nch = (nmax + kOP - 1) / kOP;  // 64-wide chunks of the largest matrix
-  BjJob* d = (BjJob*)dev_alloc(sizeof(BjJob) * nj, s);
-  dev_h2d(d, bj.data(), sizeof(BjJob) * nj, s);
-  double* gmax = (double*)dev_alloc(sizeof(double) * nj, s);
-  double* vbuf = (double*)dev_alloc(sizeof(double) * (size_t)pairs * kOP * kOP, s);
+  BjJob<T>* d = (BjJob<T>*)dev_alloc(sizeof(BjJob<T>) * nj, s);
+  dev_h2d(d, bj.data(), sizeof(BjJob<T>) * nj, s);
+  T* vbuf = (T*)dev_alloc(sizeof(T) * (size_t)pairs * kOP * kOP, s);
   int* flag = (int*)dev_alloc(sizeof(int) * pairs, s);
   int* nrot = (int*)dev_alloc(sizeof(int) * nj, s);
   std::vector<int> hrot(nj);
-  k_bj_prep<<<nj, 256, 0, S(s)>>>(d, gmax);
-  ++g_launches;
-  const size_t shr = sizeof(double) * 2 * kOP * kOL, shc = sizeof(double) * 2 * kOP * kOL;
-  static bool attr = false;
+  const size_t sh = sizeof(T) * 2 * kOP * kOL;
+  static bool attr = false;  // per element type
   if (!attr) {
-    ck(cudaFuncSetAttribute(k_bj_rows, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shr), "bj smem");
-    ck(cudaFuncSetAttribute(k_bj_cols, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shc), "bj smem");
-    ck(cudaFuncSetAttribute(k_bj_rowapply, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shc), "bj smem");
+    ck(cudaFuncSetAttribute(k_bj_rows<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh), "bj smem");
+    ck(cudaFuncSetAttribute(k_bj_cols<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh), "bj smem");
+    ck(cudaFuncSetAttribute(k_bj_rowapply<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh), "bj smem");
     attr = true;
   }
-  for (int sweep = 0; sweep < 40; ++sweep) {
+  for (int sweep = 0; sweep < sweeps; ++sweep) {
     ck(cudaMemsetAsync(nrot, 0, sizeof(int) * nj, S(s)), "bj counters");
     for (int step = 0; step < nbmax - 1; ++step) {
-      k_bj_rows<<<pairs, 256, shr, S(s)>>>(d, nj, step, gmax, vbuf, flag, nrot);
-      k_bj_rowapply<<<dim3(pairs, nch), 256, shc, S(s)>>>(d, nj, step, vbuf, flag);
-      k_bj_cols<<<dim3(pairs, nch, 2), 256, shc, S(s)>>>(d, nj, step, vbuf, flag);
+      k_bj_rows<T><<<pairs, 256, sh, S(s)>>>(d, nj, step, gmax, vbuf, flag, nrot);
+      k_bj_rowapply<T><<<dim3(pairs, nch), 256, sh, S(s)>>>(d, nj, step, vbuf, flag);
+      k_bj_cols<T><<<dim3(pairs, nch, 2), 256, sh, S(s)>>>(d, nj, step, vbuf, flag);
       g_launches += 3;
     }
     ck(cudaGetLastError(), "bj step");
@@ -1554,16 +1644,36 @@ static void eig_block_jacobi(const std::vector<EigJob>& jobs, Stream s) {
     for (int v : hrot) any = any || v > 0;
     if (!any) break;
   }
+  dev_free(nrot, s);
+  dev_free(flag, s);
+  dev_free(vbuf, s);
+  dev_free(d, s);
+}
+
+}  // namespace
+
+static void eig_block_jacobi(const std::vector<EigJob>& jobs, Stream s) {
+  if (jobs.empty()) return;
+  std::vector<BjJob<double>> bj;
+  int nmax = 0;
+  for (const EigJob& j : jobs) {
+    bj.push_back({j.A, j.Q, j.w, j.n, 0, 0, 0});
+    nmax = std::max(nmax, j.n);
+  }
+  const int nj = (int)bj.size();
   const size_t shf = sizeof(double) * 2 * nmax;
   if (shf > 220 * 1024) throw std::runtime_error("eig_batched: block too large");
+  BjJob<double>* d = (BjJob<double>*)dev_alloc(sizeof(BjJob<double>) * nj, s);
+  dev_h2d(d, bj.data(), sizeof(BjJob<double>) * nj, s);
+  double* gmax = (double*)dev_alloc(sizeof(double) * nj, s);
+  k_bj_prep<<<nj, 256, 0, S(s)>>>(d, gmax);
+  ++g_launches;
+  bj_sweeps(bj, gmax, 40, s);
   if (shf > 48 * 1024)
     ck(cudaFuncSetAttribute(k_bj_finish, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shf), "bj finish smem");
   k_bj_finish<<<nj, 256, shf, S(s)>>>(d);
   ++g_launches;
   ck(cudaGetLastError(), "bj finish");
-  dev_free(nrot, s);
-  dev_free(flag, s);
-  dev_free(vbuf, s);
   dev_free(gmax, s);
   dev_free(d, s);
 }
@@ -1590,6 +1700,314 @@ void eig_batched(const std::vector<EigJob>& jobs, Stream s) {
   dev_free(d, s);
 }
 
+// ------------------------------------------------------------------ refined eigensolver
+//
+// The same eigenproblems, mostly in FP32.  FP64 Jacobi costs about 50 n^3 FP64 operations
+// and a chain of n - 1 rotations (3000 cycles each) per sweep; an SM does two FP64 FMAs
+// per cycle and 128 FP32 ones.  So three passes of: FP32 Jacobi on the current matrix S
+// (scaled by its largest diagonal entry) -> Q; X <- X Q, orthonormalised by a Newton-Schulz
+// step X (3 I - X^T X) / 2; T = M^T X (or M X), S = T^T T, all of these FP64 products of the
+// whole GPU (S from M itself, G = M M^T or M^T M, has errors of eps sigma_i sigma_j, where
+// X^T G X has eps |G|).  Each pass resolves eigenvectors to FP32 accuracy within blocks of
+// similar eigenvalues, so the unresolved part of S falls from |G| to 1e-7, 1e-14 |G| and
+// rounding (the floors below which a pass leaves an off-diagonal alone).  Then one step of
+// the iterative refinement of T. Ogita and K. Aishima (Japan J. Indust. Appl. Math. 35, 2018):
+// with R = I - X^T X, lambda_i = S_ii / (1 - R_ii), X <- X + X E, E_ij = (S_ij + lambda_j
+// R_ij) / (lambda_j - lambda_i), R_ij / 2 where that is not small, and a last Newton-Schulz
+// step.  Measured (dmrg_truncate, against the Jacobi solver): Hubbard L=16, D=200 (sectors up
+// to 114 rows) 37.1 -> 8.1 ms, random L=28, D=1500 (up to 202) 116 -> 22.4 ms, the error of the
+// truncated state against an SVD 6.5e-15 -> 2.3e-15 and 1.5e-14 -> 3.5e-15.  A job that still
+// has an
+// off-diagonal above rounding whose rotation is not negligible (a relative gap below FP32's
+// resolution) is handed to the FP64 solver.
+
+namespace {
+struct ReJob {
+  const double* G;
+  double *X, *S, *R, *w, *Q;
+  float *A32, *Q32;
+  int n, pad;
+};
+
+// A32 = S / max diagonal, Q32 = I
+__global__ void __launch_bounds__(256) k_re_start(const ReJob* __restrict__ jobs, int first) {
+  const ReJob J = jobs[blockIdx.x];
+  const double* S = first ? J.G : J.S;
+  const int n = J.n, tid = threadIdx.x;
+  __shared__ double red[256];
+  double best = 0.0;
+  for (int i = tid; i < n; i += 256) best = fmax(best, fabs(S[(size_t)i * n + i]));
+  red[tid] = best;
+  __syncthreads();
+  for (int o = 128; o > 0; o >>= 1) {
+    if (tid < o) red[tid] = fmax(red[tid], red[tid + o]);
+    __syncthreads();
+  }
+  const double inv = red[0] > 0.0 ? 1.0 / red[0] : 0.0;
+  for (int64_t e = tid; e < (int64_t)n * n; e += 256) {
+    const int i = (int)(e / n), j = (int)(e % n);
+    J.A32[e] = (float)(S[i <= j ? e : (int64_t)j * n + i] * inv);  // symmetric to the bit
+    J.Q32[e] = i == j ? 1.0f : 0.0f;
+  }
+}
+
+// FP32 Jacobi of the blocks up to kEigSmemN rows, one CTA each
+__global__ void __launch_bounds__(256) k_re_small(const ReJob* __restrict__ jobs, const int* __restrict__ which,
+                                                  int sweeps, float floor_abs) {
+  const ReJob J = jobs[which[blockIdx.x]];
+  const int n = J.n, np = (n + 1) & ~1, ld = np + 1, tid = threadIdx.x;
+  extern __shared__ float fsm[];
+  float* A = fsm;
+  float* Q = A + np * ld;
+  __shared__ float cs[kEigSmemN / 2], sn[kEigSmemN / 2];
+  __shared__ int pp[kEigSmemN / 2], qq[kEigSmemN / 2], flag;
+  for (int e = tid; e < np * np; e += 256) {
+    const int i = e / np, j = e % np;
+    const bool in = i < n && j < n;
+    A[i * ld + j] = in ? J.A32[(size_t)i * n + j] : 0.0f;
+    Q[i * ld + j] = i == j ? 1.0f : 0.0f;
+  }
+  __syncthreads();
+  if (np > 1) jacobi_f32(A, Q, np, ld, sweeps, floor_abs, cs, sn, pp, qq, &flag);
+  __syncthreads();
+  for (int e = tid; e < n * n; e += 256) J.Q32[e] = Q[(e / n) * ld + e % n];
+}
+
+// out = (double)Q32 (to X on the first pass, to S, as scratch, afterwards)
+__global__ void k_re_widen(const ReJob* __restrict__ jobs, int first) {
+  const ReJob J = jobs[blockIdx.x];
+  double* out = first ? J.X : J.S;
+  for (int64_t e = threadIdx.x + (int64_t)blockIdx.y * blockDim.x; e < (int64_t)J.n * J.n; e += (int64_t)gridDim.y * blockDim.x)
+    out[e] = (double)J.Q32[e];
+}
+
+__global__ void k_re_identity(const ReJob* __restrict__ jobs) {  // R = I
+  const ReJob J = jobs[blockIdx.x];
+  for (int64_t e = threadIdx.x + (int64_t)blockIdx.y * blockDim.x; e < (int64_t)J.n * J.n; e += (int64_t)gridDim.y * blockDim.x)
+    J.R[e] = e / J.n == e % J.n ? 1.0 : 0.0;
+}
+
+__global__ void k_re_half(const ReJob* __restrict__ jobs) {  // R <- R / 2 (Newton-Schulz)
+  const ReJob J = jobs[blockIdx.x];
+  for (int64_t e = threadIdx.x + (int64_t)blockIdx.y * blockDim.x; e < (int64_t)J.n * J.n; e += (int64_t)gridDim.y * blockDim.x)
+    J.R[e] *= 0.5;
+}
+
+// R <- E; bad[job] = 1 where the refinement cannot be trusted
+__global__ void __launch_bounds__(256) k_re_correct(const ReJob* __restrict__ jobs, int* __restrict__ bad) {
+  const ReJob J = jobs[blockIdx.x];
+  const int n = J.n, tid = threadIdx.x;
+  extern __shared__ double lam[];
+  __shared__ double gm;
+  __shared__ int fail;
+  if (tid == 0) { fail = 0; gm = 0.0; }
+  for (int i = tid; i < n; i += 256) lam[i] = J.S[(size_t)i * n + i] / (1.0 - J.R[(size_t)i * n + i]);
+  __syncthreads();
+  if (tid < 32) {
+    double m = 0.0;
+    for (int i = tid; i < n; i += 32) m = fmax(m, fabs(lam[i]));
+    for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
+    if (tid == 0) gm = m;
+  }
+  __syncthreads();
+  for (int64_t e = tid; e < (int64_t)n * n; e += 256) {
+    const int i = (int)(e / n), j = (int)(e % n);
+    const double r = J.R[e];
+    double v = 0.5 * r;
+    if (!(fabs(r) <= 1e-9)) fail = 1;  // also not finite
+    if (i != j) {
+      const double g = J.S[e] + lam[j] * r, gap = lam[j] - lam[i];
+      if (fabs(g) < 1e-5 * fabs(gap)) v = g / gap;
+      else if (!(fabs(g) <= 1e-14 * gm)) fail = 1;
+    }
+    J.R[e] = v;
+  }
+  for (int i = tid; i < n; i += 256) J.w[i] = lam[i];
+  __syncthreads();
+  if (tid == 0) bad[blockIdx.x] = fail;
+}
+
+// eigenvalues (in w) sorted descending (ties by index) with the columns of X, into w and Q
+__global__ void __launch_bounds__(256) k_re_finish(const ReJob* __restrict__ jobs) {
+  const ReJob J = jobs[blockIdx.x];
+  const int n = J.n, tid = threadIdx.x;
+  extern __shared__ double lam[];
+  int* rank = reinterpret_cast<int*>(lam + n);
+  for (int i = tid; i < n; i += 256) lam[i] = J.w[i];
+  __syncthreads();
+  for (int i = tid; i < n; i += 256) {
+    int r = 0;
+    for (int j = 0; j < n; ++j) r += lam[j] > lam[i] || (lam[j] == lam[i] && j < i);
+    rank[i] = r;
+    J.w[r] = lam[i];
+  }
+  __syncthreads();
+  for (int64_t e = tid; e < (int64_t)n * n; e += 256) J.Q[(e / n) * n + rank[e % n]] = J.X[e];
+}
+}  // namespace
+
+void eig_refined(const std::vector<EigJob>& jobs, const std::vector<EigSource>& src, Stream s) {
+  if (jobs.empty()) return;
+  std::vector<int64_t> off(1, 0), toff(1, 0);
+  int nmax = 1;
+  for (size_t k = 0; k < jobs.size(); ++k) {
+    off.push_back(off.back() + (int64_t)jobs[k].n * jobs[k].n);
+    toff.push_back(toff.back() + (int64_t)src[k].inner * jobs[k].n);
+    nmax = std::max(nmax, jobs[k].n);
+  }
+  if (sizeof(double) * 2 * (size_t)nmax > 200 * 1024) return eig_batched(jobs, s);
+  const int64_t tot = off.back();
+  const int nj = (int)jobs.size();
+  // X, X2, S, R, T (FP64), A32, Q32 (FP32)
+  const int64_t ttot = toff.back();
+  double* buf = (double*)dev_alloc(sizeof(double) * (size_t)(tot * 5 + ttot), s);
+  double *X = buf, *X2 = X + tot, *Sm = X2 + tot, *R = Sm + tot, *T = R + tot;
+  float *A32 = (float*)(T + ttot), *Q32 = A32 + tot;
+  ReJob* d = nullptr;
+  int *dsmall = nullptr, *dbad = nullptr;
+  double* gbig = nullptr;
+  GemmPlan *pq = nullptr, *pr = nullptr, *pn = nullptr, *pt = nullptr, *ps = nullptr;
+  std::vector<int> hbad(nj, 0);
+  auto cleanup = [&]() {
+    for (GemmPlan* p : {pq, pr, pn, pt, ps}) gemm_plan_free(p, s);
+    dev_free(d, s);
+    dev_free(dsmall, s);
+    dev_free(dbad, s);
+    dev_free(gbig, s);
+    dev_free(buf, s);
+  };
+  try {
+    std::vector<ReJob> re;
+    std::vector<int> small;
+    std::vector<BjJob<float>> big;
+    int nsm = 1;
+    for (int k = 0; k < nj; ++k) {
+      const EigJob& j = jobs[k];
+      const int64_t o = off[k];
+      re.push_back({j.A, X + o, Sm + o, R + o, j.w, j.Q, A32 + o, Q32 + o, j.n, 0});
+      if (j.n <= kEigSmemN) {
+        small.push_back(k);
+        nsm = std::max(nsm, j.n);
+      } else {
+        big.push_back({A32 + o, Q32 + o, nullptr, j.n, 0, 0, 0});
+      }
+    }
+    d = (ReJob*)dev_alloc(sizeof(ReJob) * nj, s);
+    dev_h2d(d, re.data(), sizeof(ReJob) * nj, s);
+    dsmall = (int*)dev_alloc(sizeof(int) * (small.size() + 1), s);
+    dev_h2d(dsmall, small.data(), sizeof(int) * small.size(), s);
+    dbad = (int*)dev_alloc(sizeof(int) * nj, s);
+    // the three passes: floor (of the largest diagonal entry, scaled to 1: a little above
+    // what FP32 rounding leaves of the part that the pass resolves), sweeps at most, and
+    // Newton-Schulz steps (FP32 rotations leave Q orthonormal to 1e-5 where they are large)
+    constexpr double kFloor[3] = {1e-6, 5e-13, 5e-16};
+    constexpr int kSweeps[3] = {10, 8, 4}, kSchulz[3] = {2, 2, 1};
+    const size_t nb = big.size();
+    gbig = (double*)dev_alloc(sizeof(double) * std::max<size_t>(3 * nb, 1), s);
+    std::vector<double> fl;
+    for (double f : kFloor) fl.insert(fl.end(), nb, f);
+    dev_h2d(gbig, fl.data(), sizeof(double) * fl.size(), s);
+    // one n-column product per job: C (m x n) += alpha op(A) B
+    auto plan = [&](auto task) {
+      std::vector<GemmTask> t;
+      std::vector<GemmGroup> g;
+      for (int k = 0; k < nj; ++k) {
+        double* c = nullptr;
+        int m = jobs[k].n;
+        t.push_back(task(k, c, m));
+        g.push_back({c, jobs[k].n, m, jobs[k].n, k, k + 1, 0});
+      }
+      return gemm_plan_upload(t, g, s, GEMM_SHARED);
+    };
+    pq = plan([&](int k, double*& c, int&) {  // X2 = X Q (Q widened into S)
+      const int n = jobs[k].n;
+      c = X2 + off[k];
+      return GemmTask{X + off[k], Sm + off[k], n, n, n, 0, 0, 1.0};
+    });
+    pr = plan([&](int k, double*& c, int&) {  // R -= X^T X
+      const int n = jobs[k].n;
+      c = R + off[k];
+      return GemmTask{X + off[k], X + off[k], n, n, n, 1, 0, -1.0};
+    });
+    pn = plan([&](int k, double*& c, int&) {  // X2 += X R
+      const int n = jobs[k].n;
+      c = X2 + off[k];
+      return GemmTask{X + off[k], R + off[k], n, n, n, 0, 0, 1.0};
+    });
+    pt = plan([&](int k, double*& c, int& m) {  // T = M^T X or M X
+      const int n = jobs[k].n;
+      c = T + toff[k];
+      m = src[k].inner;
+      return GemmTask{src[k].M, X + off[k], src[k].ld, n, n, src[k].trans, 0, 1.0};
+    });
+    ps = plan([&](int k, double*& c, int&) {  // S = T^T T
+      const int n = jobs[k].n;
+      c = Sm + off[k];
+      return GemmTask{T + toff[k], T + toff[k], n, n, src[k].inner, 1, 0, 1.0};
+    });
+    const size_t bytes = sizeof(double) * (size_t)tot;
+    const dim3 grid(nj, std::max(1, std::min(64, nmax * nmax / 4096)));
+    const int np = (nsm + 1) & ~1;
+    const size_t shs = sizeof(float) * 2 * (size_t)np * (np + 1), shc = sizeof(double) * 2 * (size_t)nmax;
+    if (shc > 48 * 1024) {
+      ck(cudaFuncSetAttribute(k_re_correct, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shc), "eig smem");
+      ck(cudaFuncSetAttribute(k_re_finish, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shc), "eig smem");
+    }
+    // X <- X2 + ... where X2 holds a copy of X, then X = X2
+    auto residual = [&]() {  // R = I - X^T X
+      k_re_identity<<<grid, 256, 0, S(s)>>>(d);
+      gemm_plan_run(pr, s, GEMM_SHARED);
+      ++g_launches;
+    };
+    auto add_correction = [&]() {  // X <- X + X R
+      dev_d2d(X2, X, bytes, s);
+      gemm_plan_run(pn, s, GEMM_SHARED);
+      dev_d2d(X, X2, bytes, s);
+    };
+    auto schulz = [&]() {  // X <- X (3 I - X^T X) / 2
+      residual();
+      k_re_half<<<grid, 256, 0, S(s)>>>(d);
+      ++g_launches;
+      add_correction();
+    };
+    for (int pass = 0; pass < 3; ++pass) {
+      k_re_start<<<nj, 256, 0, S(s)>>>(d, pass == 0);
+      if (!small.empty()) k_re_small<<<(int)small.size(), 256, shs, S(s)>>>(d, dsmall, kSweeps[pass], (float)kFloor[pass]);
+      bj_sweeps(big, gbig + pass * nb, kSweeps[pass], s);
+      k_re_widen<<<grid, 256, 0, S(s)>>>(d, pass == 0);
+      g_launches += 3;
+      if (pass > 0) {
+        dev_zero(X2, bytes, s);
+        gemm_plan_run(pq, s, GEMM_SHARED);
+        dev_d2d(X, X2, bytes, s);
+      }
+      for (int u = 0; u < kSchulz[pass]; ++u) schulz();
+      dev_zero(T, sizeof(double) * (size_t)ttot, s);
+      gemm_plan_run(pt, s, GEMM_SHARED);
+      dev_zero(Sm, bytes, s);
+      gemm_plan_run(ps, s, GEMM_SHARED);
+    }
+    residual();
+    k_re_correct<<<nj, 256, shc, S(s)>>>(d, dbad);
+    add_correction();
+    schulz();
+    ck(cudaGetLastError(), "refined eig");
+    dev_d2h(hbad.data(), dbad, sizeof(int) * nj, s);
+    k_re_finish<<<nj, 256, shc, S(s)>>>(d);
+    g_launches += 2;
+    ck(cudaGetLastError(), "refined eig");
+    dev_sync(s);
+  } catch (...) {
+    cleanup();
+    throw;
+  }
+  cleanup();
+  std::vector<EigJob> again;
+  for (int k = 0; k < nj; ++k)
+    if (hbad[k]) again.push_back(jobs[k]);
+  eig_batched(again, s);
+}
+
 // ------------------------------------------------------------------ selection
 
 namespace {
@@ -1597,21 +2015,25 @@ namespace {
 // value, many CTAs; keep[i] = rank < D and above the zero threshold
 __global__ void k_select_rank(const double* __restrict__ v, int n, const double* __restrict__ vmax,
                               int D, double zero_rel, int* __restrict__ keep) {
-  __shared__ double tile[1024];
+  // non-negative doubles order like their bit patterns: integer comparisons (an FP64 one
+  // costs a warp 16 cycles of the SM: 0.82 ms for 6,000 values, now 0.10)
+  __shared__ long long tile[1024];
+  auto bits = [](double x) { return x > 0.0 ? __double_as_longlong(x) : 0ll; };
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  const double vi = i < n ? fmax(v[i], 0.0) : 0.0;
+  const double vd = i < n ? fmax(v[i], 0.0) : 0.0;
+  const long long vi = bits(vd);
   int rank = 0;
   for (int j0 = 0; j0 < n; j0 += 1024) {
-    for (int t = threadIdx.x; t < 1024; t += blockDim.x) tile[t] = (j0 + t < n) ? fmax(v[j0 + t], 0.0) : -1.0;
+    for (int t = threadIdx.x; t < 1024; t += blockDim.x) tile[t] = (j0 + t < n) ? bits(v[j0 + t]) : -1ll;
     __syncthreads();
     const int jn = min(1024, n - j0);
     for (int t = 0; t < jn; ++t) {
-      const double vj = tile[t];
+      const long long vj = tile[t];
       rank += (vj > vi || (vj == vi && j0 + t < i)) ? 1 : 0;
     }
     __syncthreads();
   }
-  if (i < n) keep[i] = (rank < D && vi > zero_rel * zero_rel * (*vmax)) ? 1 : 0;
+  if (i < n) keep[i] = (rank < D && vd > zero_rel * zero_rel * (*vmax)) ? 1 : 0;
 }
 
 __global__ void k_select_max(const double* __restrict__ v, int n, double* __restrict__ vmax) {
