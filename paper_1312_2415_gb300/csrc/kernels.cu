@@ -150,11 +150,14 @@ float event_elapsed_ms(void* a, void* b) {
 // anywhere in the sum, and groups with long task lists are shared by 2 to 8 warps of a CTA,
 // whose partial sums are added in a fixed order (deterministic, no atomics).  Measured
 // against 32 x 32 tiles staged in shared memory with two barriers per 16 columns (H_eff x,
-// whole call): Hubbard L=8, D=64 769 -> 99 us; random L=12, D=500 17.4 -> 1.36 ms; random
-// L=28, D=1500 281 -> 157 ms (phase 1 0.82 of the 1.1 TFLOP/s FP64 rate).
+// whole call): Hubbard L=8, D=64 769 -> 98 us; random L=12, D=500 17.4 -> 1.2 ms; random
+// L=28, D=1500 281 -> 128 ms (0.90 TFLOP/s; cuBLAS DGEMM reaches 1.10 on large squares).  Four
+// CTAs of 64 registers per SM against two of 128: phase 1 95 -> 83 ms, phase 2 39 -> 43 ms
+// there.  The last one to three columns of a task are loaded together, not one at a time:
+// phase 2 50 -> 39 ms.
 
 namespace {
-constexpr int kGemmWarps = 8;
+constexpr int kGemmWarps = 8, kGemmMinCtas = 4;
 
 struct Remap {
   const char* lo[4];
@@ -269,30 +272,149 @@ __device__ __forceinline__ void gemm_sum(const GemmTask* __restrict__ tasks, int
 #pragma unroll
       for (int r = 0; r < R; ++r) pa[r] += 4 * sak;
     }
-    for (; k > 0; --k) {
-      const double b = kOrdered ? flip(*pb) : *pb;
-      pb += sbk;
+    if (k > 0) {  // the last one to three columns, their loads in flight together
+      double b[3], a[R][3];
 #pragma unroll
-      for (int r = 0; r < R; ++r) {
-        const double a = kOrdered && fa != 1.0 ? __dmul_rn(*pa[r], fa) : *pa[r];
-        s[r] = fma(a, b, s[r]);
-        pa[r] += sak;
-      }
+      for (int u = 0; u < 3; ++u)
+        if (!kOrdered || u < k) {
+          const int o = kOrdered || u < k ? u : 0;  // shared sums: a repeated load for a branch
+          b[u] = kOrdered ? flip(pb[o * sbk]) : pb[o * sbk];
+#pragma unroll
+          for (int r = 0; r < R; ++r) a[r][u] = pa[r][o * sak];
+        }
+#pragma unroll
+      for (int u = 0; u < 3; ++u)
+        if (u < k) {
+#pragma unroll
+          for (int r = 0; r < R; ++r) s[r] = fma(kOrdered && fa != 1.0 ? __dmul_rn(a[r][u], fa) : a[r][u], b[u], s[r]);
+        }
     }
 #pragma unroll
     for (int r = 0; r < R; ++r) acc[r] = kOrdered ? s[r] : fma(cur.alpha, s[r], acc[r]);
   }
 }
 
-template <int R, bool kRemap, bool kOrdered>
+// A warp's shared memory: a ring of operand chunks (up to four columns of A and rows of B:
+// a[u * 32 + row], b[u * 32 + lane]) and the descriptors of two batches of 32 tasks.
+constexpr int kGemmDepth = 4;
+struct GemmWarpBuf {
+  double a[kGemmDepth][128], b[kGemmDepth][128];
+  GemmTask desc[2][32];
+};
+
+__device__ __forceinline__ void cp_async8(double* dst, const double* src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src));
+}
+
+// The same ordered sum for tables too small to fill the GPU, one row per lane (the warp's
+// lanes read at most 32 rows).  The chunks of all tasks form one stream: kGemmDepth - 1 of them are in
+// flight (cp.async) while one is summed, so that a chain of small tasks costs its FMAs (66
+// cycles each) and its instructions, not several trips to L2 per task.  Measured (phase 2 of
+// Hubbard L=8, D=64, ordered lists of up to 137 tasks of 4 columns): loads when a task starts
+// 236 us, the stream 165 us.  Tables that fill the GPU keep the direct loads: the FP64 pipe
+// is busy anyway, and the rings' shared memory takes away L1 (phase 1 of random L=28, D=1500:
+// direct 104 ms, stream 134 ms); so do shared sums, whose warps have few tasks each (phase 2
+// of random L=12, D=350: 54 / 86 us).
+template <bool kRemap>
+__device__ __forceinline__ void gemm_stream(const GemmTask* __restrict__ tasks, int t0, int t1, int i0, int j,
+                                         const Remap& rm, GemmWarpBuf& wb, double (&acc)[1]) {
+
+  const int lane = threadIdx.x & 31, nt = t1 - t0;
+  // rows the warp's lanes read, and this lane's among them
+  const int row0 = __reduce_min_sync(0xffffffffu, i0);
+  const int nrow = __reduce_max_sync(0xffffffffu, i0) + 1 - row0, lr = i0 - row0;
+  double s = 0.0;
+  int it = 0, ik = 0;  // next chunk to load
+  auto issue = [&](int slot) {
+    if (it < nt) {
+      if (ik == 0 && (it & 31) == 0) {  // the descriptors of the next 32 tasks
+        __syncwarp();
+        if (it + lane < nt) wb.desc[(it >> 5) & 1][lane] = tasks[t0 + it + lane];
+        __syncwarp();
+      }
+      const GemmTask& T = wb.desc[(it >> 5) & 1][it & 31];
+      const double* B = kRemap ? remap_ptr(T.B, rm) : T.B;
+      const int64_t ldb = T.ldb;
+      int k;
+      if (T.A == nullptr) {  // op(A) = identity: the elements of op(B) themselves
+        k = 1;
+        const int64_t si = T.transB ? 1 : ldb, sj = T.transB ? ldb : 1;
+        cp_async8(&wb.b[slot][lane], B + i0 * si + j * sj);
+      } else {
+        k = T.k;
+        const double* A = kRemap ? remap_ptr(T.A, rm) : T.A;
+        const int64_t lda = T.lda, sai = T.transA ? 1 : lda, sak = T.transA ? lda : 1;
+        const int64_t sbk = T.transB ? 1 : ldb, sbj = T.transB ? ldb : 1;
+        const double* pa = A + (row0 + lane) * sai + ik * sak;
+        const double* pb = B + j * sbj + ik * sbk;
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+          if (ik + u < k) {
+            if (lane < nrow) cp_async8(&wb.a[slot][u * 32 + lane], pa + u * sak);
+            cp_async8(&wb.b[slot][u * 32 + lane], pb + u * sbk);
+          }
+      }
+      ik += 4;
+      if (ik >= k) {
+        ik = 0;
+        ++it;
+      }
+    }
+    asm volatile("cp.async.commit_group;");
+  };
+#pragma unroll
+  for (int d = 0; d < kGemmDepth - 1; ++d) issue(d);
+  int slot = 0;
+  for (int ct = 0; ct < nt; ++ct) {
+    int K = 1, ck = 0;
+    do {
+      issue((slot + kGemmDepth - 1) % kGemmDepth);
+      asm volatile("cp.async.wait_group %0;" ::"n"(kGemmDepth - 1));
+      __syncwarp();
+      const GemmTask& T = wb.desc[(ct >> 5) & 1][ct & 31];
+      const double alpha = T.alpha;
+      double* a = wb.a[slot];
+      const double* b = wb.b[slot];
+      if (T.A == nullptr) {
+        s = fma(alpha, b[lane], s);
+      } else {
+        K = T.k;
+        const bool unit = fabs(alpha) == 1.0;
+        if (!unit) {
+#pragma unroll
+          for (int u = 0; u < 4; ++u)
+            if (ck + u < K && lane < nrow) a[u * 32 + lane] = __dmul_rn(a[u * 32 + lane], alpha);
+          __syncwarp();
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+          if (ck + u < K) {
+            double bv = b[u * 32 + lane];
+            if (unit && alpha < 0.0) bv = -bv;
+            s = fma(a[u * 32 + lr], bv, s);
+          }
+      }
+      __syncwarp();  // the slot may be refilled
+      slot = (slot + 1) % kGemmDepth;
+      ck += 4;
+    } while (ck < K);
+  }
+  acc[0] = s;
+}
+
+// kStream: the streamed sum (R = 1, ordered); buf: 128 doubles per warp (kGemmWarps of them),
+// or the warps' rings
+template <int R, bool kRemap, bool kOrdered, bool kStream>
 __device__ __forceinline__ void gemm_job(const GemmTask* __restrict__ tasks, const GemmGroup& g, const GemmJob& J,
-                                         const Remap& rm, double* red, bool lead_only) {
+                                         const Remap& rm, void* buf, bool lead_only) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int slots = ((g.m + R - 1) / R) * g.n;
   const int nt = g.task_end - g.task_begin;
   const int t0 = g.task_begin + (int)((int64_t)nt * J.sidx / J.ns);
   const int t1 = g.task_begin + (int)((int64_t)nt * (J.sidx + 1) / J.ns);
   double* C = kRemap ? (double*)remap_ptr(g.C, rm) : g.C;
+  // a shared sum's partial sums: R x 32 of every warp
+  auto part = [&](int w) { return (double*)buf + w * 128; };
   for (int w = J.w0; w < J.w0 + J.nw; ++w) {
     const int slot = w * 32 + lane;
     const bool valid = slot < slots;
@@ -302,14 +424,15 @@ __device__ __forceinline__ void gemm_job(const GemmTask* __restrict__ tasks, con
     if (lead_only) {  // second call of a shared sum: this warp adds the other warps' parts
 #pragma unroll
       for (int r = 0; r < R; ++r) {
-        acc[r] = red[(warp * 4 + r) * 32 + lane];
-        for (int o = 1; o < J.ns; ++o) acc[r] += red[((warp + o) * 4 + r) * 32 + lane];
+        acc[r] = part(warp)[r * 32 + lane];
+        for (int o = 1; o < J.ns; ++o) acc[r] += part(warp + o)[r * 32 + lane];
       }
     } else {
-      gemm_sum<R, kRemap, kOrdered>(tasks, t0, t1, i0, j, g.m, rm, red + warp * 128, acc);
+      if constexpr (kStream) gemm_stream<kRemap>(tasks, t0, t1, i0, j, rm, ((GemmWarpBuf*)buf)[warp], acc);
+      else gemm_sum<R, kRemap, kOrdered>(tasks, t0, t1, i0, j, g.m, rm, (double*)buf + warp * 128, acc);
       if (!kOrdered && J.ns > 1) {
 #pragma unroll
-        for (int r = 0; r < R; ++r) red[(warp * 4 + r) * 32 + lane] = acc[r];
+        for (int r = 0; r < R; ++r) part(warp)[r * 32 + lane] = acc[r];
         return;
       }
     }
@@ -319,14 +442,14 @@ __device__ __forceinline__ void gemm_job(const GemmTask* __restrict__ tasks, con
   }
 }
 
-// one warp per job, kGemmWarps jobs per CTA; the ns jobs of a shared sum are consecutive
-// and never straddle CTAs (ordered sums are never shared)
-template <bool kRemap, bool kOrdered>
-__global__ void __launch_bounds__(kGemmWarps * 32)
+// one warp per job, up to kGemmWarps jobs per CTA; the ns jobs of a shared sum are
+// consecutive and never straddle CTAs (kGemmWarps warps then; ordered sums are never shared)
+template <bool kRemap, bool kOrdered, bool kStream>
+__global__ void __launch_bounds__(kGemmWarps * 32, kGemmMinCtas)
     k_grouped_gemm(const GemmTask* __restrict__ tasks, const GemmGroup* __restrict__ groups,
                    const GemmJob* __restrict__ jobs, int njobs, Remap rm) {
-  __shared__ double red4[kGemmWarps * 4 * 32];
-  const int id = blockIdx.x * kGemmWarps + (threadIdx.x >> 5);
+  extern __shared__ __align__(16) unsigned char gemm_smem[];
+  const int id = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   GemmJob J{-1, 0, 0, 0, 0};
   GemmGroup g{};
   if (id < njobs) {
@@ -336,9 +459,13 @@ __global__ void __launch_bounds__(kGemmWarps * 32)
   for (int pass = 0; pass < (kOrdered ? 1 : 2); ++pass) {
     if (pass == 1) __syncthreads();
     if (J.group >= 0 && (pass == 0 || (J.ns > 1 && J.sidx == 0))) {
-      if (g.rpl == 4) gemm_job<4, kRemap, kOrdered>(tasks, g, J, rm, red4, pass == 1);
-      else if (g.rpl == 2) gemm_job<2, kRemap, kOrdered>(tasks, g, J, rm, red4, pass == 1);
-      else gemm_job<1, kRemap, kOrdered>(tasks, g, J, rm, red4, pass == 1);
+      if constexpr (kStream) {
+        gemm_job<1, kRemap, kOrdered, true>(tasks, g, J, rm, gemm_smem, pass == 1);
+      } else {
+        if (g.rpl == 4) gemm_job<4, kRemap, kOrdered, false>(tasks, g, J, rm, gemm_smem, pass == 1);
+        else if (g.rpl == 2) gemm_job<2, kRemap, kOrdered, false>(tasks, g, J, rm, gemm_smem, pass == 1);
+        else gemm_job<1, kRemap, kOrdered, false>(tasks, g, J, rm, gemm_smem, pass == 1);
+      }
     }
   }
 }
@@ -362,23 +489,18 @@ int rows_per_lane(int m, int n, bool strided_b) {
 // target is what gives every SM about 40 jobs, at least kGemmMinWork so that a job is worth
 // its start.  Groups above it are shared by up to eight warps, groups below it give one
 // warp several of their 32-lane slices.  Longest jobs first.
-constexpr int64_t kGemmMinWork = 48, kGemmJobsTarget = 152 * 40;
+constexpr int64_t kGemmMinWork = 48, kGemmJobsTarget = 152 * 40, kGemmFewSlices = 8;
 
-std::vector<GemmJob> gemm_jobs(const std::vector<GemmTask>& t, std::vector<GemmGroup>& g, bool ordered) {
+// ks: columns of a group's tasks in all; rpl: its rows per lane.
+std::vector<GemmJob> gemm_jobs(const std::vector<GemmGroup>& g, const std::vector<int64_t>& ks, const std::vector<int>& rpl,
+                               bool ordered) {
   std::vector<int64_t> work(g.size(), 0);
   int64_t total = 0;
   for (size_t q = 0; q < g.size(); ++q) {
-    GemmGroup& G = g[q];
-    if (G.m <= 0 || G.n <= 0 || G.task_begin >= G.task_end) continue;
-    int64_t ks = 0;
-    bool strided = false;
-    for (int k = G.task_begin; k < G.task_end; ++k) {
-      ks += t[k].A ? t[k].k : 1;
-      strided = strided || (t[k].A && t[k].transB);
-    }
-    G.rpl = rows_per_lane(G.m, G.n, strided);
-    work[q] = G.rpl * ks + 4 * (int64_t)(G.task_end - G.task_begin);
-    total += work[q] * (((int64_t)((G.m + G.rpl - 1) / G.rpl) * G.n + 31) / 32);
+    const GemmGroup& G = g[q];
+    if (ks[q] == 0) continue;
+    work[q] = rpl[q] * ks[q] + 4 * (int64_t)(G.task_end - G.task_begin);
+    total += work[q] * (((int64_t)((G.m + rpl[q] - 1) / rpl[q]) * G.n + 31) / 32);
   }
   const int64_t target = std::max(kGemmMinWork, total / kGemmJobsTarget);
   // buckets: by sharing warps (8, 4, 2, 1), then by decreasing powers of two of the work
@@ -387,7 +509,7 @@ std::vector<GemmJob> gemm_jobs(const std::vector<GemmTask>& t, std::vector<GemmG
     const GemmGroup& G = g[q];
     if (work[q] == 0) continue;
     const int nt = G.task_end - G.task_begin;
-    const int64_t slices = ((int64_t)((G.m + G.rpl - 1) / G.rpl) * G.n + 31) / 32;
+    const int64_t slices = ((int64_t)((G.m + rpl[q] - 1) / rpl[q]) * G.n + 31) / 32;
     int ns = 1, b = 3;
     while (!ordered && ns < kGemmWarps && work[q] > ns * target && 2 * ns <= nt) { ns *= 2; --b; }
     const int64_t nw = ns > 1 ? 1 : std::min<int64_t>(32767, std::max<int64_t>(1, target / work[q]));
@@ -409,10 +531,29 @@ std::vector<GemmJob> gemm_jobs(const std::vector<GemmTask>& t, std::vector<GemmG
 GemmPlan* gemm_plan_upload(const std::vector<GemmTask>& t, std::vector<GemmGroup>& g, Stream s, int sums) {
   GemmPlan* p = new GemmPlan;
   p->ntasks = (int64_t)t.size();
+  // per group: columns in all, rows per lane; a table of at most kGemmFewSlices one-row slices
+  // per SM does not fill the GPU
+  std::vector<int64_t> ks(g.size(), 0);
+  std::vector<int> rpl(g.size(), 1);
+  int64_t slices = 0;
+  for (size_t q = 0; q < g.size(); ++q) {
+    GemmGroup& G = g[q];
+    if (G.m <= 0 || G.n <= 0) continue;
+    bool strided = false;
+    for (int k = G.task_begin; k < G.task_end; ++k) {
+      ks[q] += t[k].A ? t[k].k : 1;
+      strided = strided || (t[k].A && t[k].transB);
+    }
+    if (ks[q] == 0) continue;
+    G.rpl = rpl[q] = rows_per_lane(G.m, G.n, strided);
+    slices += ((int64_t)G.m * G.n + 31) / 32;
+  }
+  p->few = slices <= 152 * kGemmFewSlices;
+  const std::vector<int> one(p->few ? g.size() : 0, 1);  // the streamed kernel's rows per lane
   try {
     for (int kind = 0; kind < 2; ++kind) {
       if (!(sums & (kind == 0 ? GEMM_ORDERED : GEMM_SHARED))) continue;
-      const std::vector<GemmJob> jobs = gemm_jobs(t, g, kind == 0);  // also sets the groups' rpl
+      const std::vector<GemmJob> jobs = gemm_jobs(g, ks, kind == 0 && p->few ? one : rpl, kind == 0);
       if (jobs.size() > (size_t)std::numeric_limits<int>::max() - kGemmWarps)
         throw std::runtime_error("block-product table exceeds 2^31 jobs");
       p->njobs[kind] = (int)jobs.size();
@@ -440,9 +581,22 @@ template <bool kRemap>
 void gemm_launch(const GemmPlan* p, const Remap& rm, int sums, Stream s) {
   const int kind = sums == GEMM_ORDERED ? 0 : 1;
   if (!p || p->njobs[kind] == 0) return;
-  const int n = p->njobs[kind], grid = (n + kGemmWarps - 1) / kGemmWarps;
-  if (kind == 0) k_grouped_gemm<kRemap, true><<<grid, kGemmWarps * 32, 0, S(s)>>>(p->tasks, p->groups, p->jobs[0], n, rm);
-  else k_grouped_gemm<kRemap, false><<<grid, kGemmWarps * 32, 0, S(s)>>>(p->tasks, p->groups, p->jobs[1], n, rm);
+  const int n = p->njobs[kind];
+  // few ordered jobs: fewer warps per CTA, so that they spread over all SMs
+  const int w = kind == 1 || n > 152 * 4 ? kGemmWarps : n > 152 * 2 ? 4 : n > 152 ? 2 : 1;
+  auto run = [&](auto* f, size_t smem) {
+    f<<<(n + w - 1) / w, w * 32, smem, S(s)>>>(p->tasks, p->groups, p->jobs[kind], n, rm);
+  };
+  constexpr size_t direct = sizeof(double) * 128 * kGemmWarps, rings = sizeof(GemmWarpBuf) * kGemmWarps;
+  if (kind == 1) {
+    run(k_grouped_gemm<kRemap, false, false>, direct);
+  } else if (!p->few) {
+    run(k_grouped_gemm<kRemap, true, false>, direct);
+  } else {
+    auto* f = k_grouped_gemm<kRemap, true, true>;
+    ck(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)rings), "gemm smem");
+    run(f, rings / kGemmWarps * w);
+  }
   ++g_launches;
   ck(cudaGetLastError(), "grouped_gemm launch");
 }
