@@ -56,7 +56,9 @@ struct GemmPlan;  // device copy of a task/group table
 // rounding difference about a hundredfold per iteration until it converges).  GEMM_SHARED:
 // long task lists are shared by several warps, whose partial sums are added in a fixed order
 // (shorter chains, other rounding).  A plan carries a job table for each kind it is run with.
-enum { GEMM_ORDERED = 1, GEMM_SHARED = 2 };
+// GEMM_OVERWRITE (upload only): C_g = the sum instead of C_g += the sum (groups without
+// tasks are left as they are).
+enum { GEMM_ORDERED = 1, GEMM_SHARED = 2, GEMM_OVERWRITE = 4 };
 GemmPlan* gemm_plan_upload(const std::vector<GemmTask>& t, std::vector<GemmGroup>& g, Stream s,
                            int sums = GEMM_ORDERED);
 void gemm_plan_run(const GemmPlan* p, Stream s, int sums = GEMM_ORDERED);
@@ -125,9 +127,14 @@ void vec_combine(const double* V, int64_t ldv, int m, const double* c, double be
 void vec_axpby(double a, const double* x, double b, double* y, int64_t n, Stream s);
 // scale y by 1/sqrt(*nrm2_dev)
 void vec_normalize(double* y, const double* nrm2_dev, int64_t n, Stream s);
-// t = r / (theta - diag), |denominator| floored
-void vec_precondition(const double* r, const double* diag, const double* theta_dev, double* t,
-                      int64_t n, Stream s);
+// Ritz vector x = sum_j c_j V_j, residual r = sum_j c_j AV_j - theta x and preconditioned
+// residual t = r / (theta - d), |denominator| floored (c, theta on the device)
+void vec_ritz(const double* V, const double* AV, int64_t ldv, int m, const double* c, const double* theta, const double* d,
+              double* x, double* r, double* t, int64_t n, Stream s);
+// t -= sum_j c_j V_j
+void vec_project_out(const double* V, int64_t ldv, int m, const double* c, double* t, int64_t n, Stream s);
+// a = b = t / sqrt(*nrm2_dev)
+void vec_normalize2(const double* t, const double* nrm2_dev, double* a, double* b, int64_t n, Stream s);
 // ---- grouped Davidson (all instances of a batch, one launch per operation) ----
 // Workspace of one instance: subspace V and H V (n x (mmax + 1) each, column j at
 // V + j n), the Rayleigh matrix G and its eigenvectors C (mmax x mmax), Ritz values th,

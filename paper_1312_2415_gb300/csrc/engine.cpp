@@ -673,7 +673,6 @@ void Engine::update_left_from(int i, std::vector<CombOp>& comb) {
   upd_hint_out_ = out2.size();
   double* Z = (double*)dev_alloc(sizeof(double) * std::max<int64_t>(zsize, 1), stream_);
   for (size_t z = 0; z < g1.size(); ++z) g1[z].C = Z + zs[z].off;
-  dev_zero(Z, sizeof(double) * std::max<int64_t>(zsize, 1), stream_);
   std::vector<GemmGroup> g2;
   {
     std::vector<int64_t> zoff(zs.size());
@@ -687,7 +686,7 @@ void Engine::update_left_from(int i, std::vector<CombOp>& comb) {
                       g.push_back({E.data + ob.off, ob.cols, ob.rows, ob.cols, b0, b1, 0});
                     }, t2, g2);
   }
-  GemmPlan* p1 = gemm_plan_upload(t1, g1, stream_);
+  GemmPlan* p1 = gemm_plan_upload(t1, g1, stream_, GEMM_ORDERED | GEMM_OVERWRITE);
   GemmPlan* p2 = gemm_plan_upload(t2, g2, stream_);
   gemm_plan_run(p1, stream_);
   gemm_plan_run(p2, stream_);
@@ -758,7 +757,6 @@ void Engine::update_right_from(int j, std::vector<CombOp>& comb) {
   upd_hint_out_ = out2.size();
   double* Z = (double*)dev_alloc(sizeof(double) * std::max<int64_t>(zsize, 1), stream_);
   for (size_t z = 0; z < g1.size(); ++z) g1[z].C = Z + zs[z].off;
-  dev_zero(Z, sizeof(double) * std::max<int64_t>(zsize, 1), stream_);
   std::vector<GemmGroup> g2;
   {
     std::vector<int64_t> zoff(zs.size());
@@ -772,7 +770,7 @@ void Engine::update_right_from(int j, std::vector<CombOp>& comb) {
                       g.push_back({E.data + ob.off, ob.cols, ob.rows, ob.cols, b0, b1, 0});
                     }, t2, g2);
   }
-  GemmPlan* p1 = gemm_plan_upload(t1, g1, stream_);
+  GemmPlan* p1 = gemm_plan_upload(t1, g1, stream_, GEMM_ORDERED | GEMM_OVERWRITE);
   GemmPlan* p2 = gemm_plan_upload(t2, g2, stream_);
   gemm_plan_run(p1, stream_);
   gemm_plan_run(p2, stream_);
@@ -1243,7 +1241,7 @@ Engine::MatvecPlan* Engine::plan_matvec(int i, bool rdm) {
   P->tall_off = std::move(tall_off);
   P->tall_rows = std::move(tall_rows);
   P->sec_dim = br.dim;
-  P->p1 = gemm_plan_upload(t1, g1, stream_, rdm ? GEMM_SHARED : GEMM_ORDERED | GEMM_SHARED);
+  P->p1 = gemm_plan_upload(t1, g1, stream_, (rdm ? GEMM_SHARED : GEMM_ORDERED | GEMM_SHARED) | GEMM_OVERWRITE);
   P->pc = comb_plan_upload(cs, cd, stream_);
   if (!rdm) {
     P->p2 = gemm_plan_upload(t2, g2, stream_, GEMM_ORDERED | GEMM_SHARED);
@@ -1565,7 +1563,6 @@ void Engine::run_matvec(MatvecPlan* p, const double* x, double* y, bool tc, int 
     return;
   }
   if (x != p->xin) dev_d2d(p->xin, x, sizeof(double) * p->n, stream_);
-  if (p->zsize) dev_zero(p->Z, sizeof(double) * p->zsize, stream_);
   dev_zero(p->yout, sizeof(double) * std::max<int64_t>(p->n, 1), stream_);
   flush_events();
   if (!ev_[0]) for (auto& e : ev_) e = event_create();
@@ -1679,7 +1676,7 @@ void Engine::build_rq(MatvecPlan* P) {
     }
   }
   try {
-    P->rq1 = gemm_plan_upload(t1, g1, stream_, GEMM_SHARED);
+    P->rq1 = gemm_plan_upload(t1, g1, stream_, GEMM_SHARED | GEMM_OVERWRITE);
     P->rqc = comb_plan_upload(cs, cd, stream_);
     P->rq2 = gemm_plan_upload(t2, g2, stream_, GEMM_SHARED);
   } catch (...) {
@@ -1698,7 +1695,6 @@ void Engine::build_rq(MatvecPlan* P) {
 // stream, with the excited-state projectors added as in a matvec
 void Engine::run_rq(MatvecPlan* P) {
   build_rq(P);
-  if (P->zsize) dev_zero(P->Z, sizeof(double) * P->zsize, stream_);
   dev_zero(P->yout, sizeof(double) * std::max<int64_t>(P->n, 1), stream_);
   flush_events();
   if (!ev_[0]) for (auto& e : ev_) e = event_create();
@@ -1921,16 +1917,13 @@ double Engine::davidson_core(MatvecPlan* P, double* x, double tol, int maxit, bo
   int m = 1;
   for (; it < maxit; ++it) {
     small_eig(G, mmax, m, std::min(m, nkeep), th, C, stream_);
-    // u = V c0 -> x ; r = AV c0 - theta u
-    vec_combine(V, n, m, C, 0.0, x, n, stream_);
-    vec_combine(AV, n, m, C, 0.0, r, n, stream_);
-    dev_d2h(hs, th, sizeof(double), stream_);
-    dev_sync(stream_);
-    theta = hs[0];
-    vec_axpby(-theta, x, 1.0, r, n, stream_);
+    // Ritz vector, residual, its preconditioned form (used if the iteration goes on)
+    vec_ritz(V, AV, n, m, C, th, P->diag, x, r, t, n, stream_);
     vec_multidot(r, n, 1, r, n, dots, sc, stream_);
+    dev_d2h(hs, th, sizeof(double), stream_);
     dev_d2h(hs + 1, dots, sizeof(double), stream_);
     dev_sync(stream_);
+    theta = hs[0];
     st_.davidson_iters += 1;
     const double rn = std::sqrt(std::max(hs[1], 0.0));
     if (rn <= tol) { conv = true; break; }
@@ -1945,12 +1938,10 @@ double Engine::davidson_core(MatvecPlan* P, double* x, double tol, int maxit, bo
       if (k > 8 && rn <= 1e-4 * std::fabs(theta) && rn > 0.8 * rhist[k - 9]) break;
     }
     if (it + 1 >= maxit) break;  // no use expanding the subspace on the last iteration
-    vec_precondition(r, P->diag, th, t, n, stream_);
     for (int pass = 0; pass < 2; ++pass) {
       // t -= V (V^T t)
       vec_multidot(V, n, m, t, n, dots, sc, stream_);
-      vec_combine(V, n, m, dots, 0.0, tmp, n, stream_);
-      vec_axpby(-1.0, tmp, 1.0, t, n, stream_);
+      vec_project_out(V, n, m, dots, t, n, stream_);
     }
     vec_multidot(t, n, 1, t, n, dots, sc, stream_);
     dev_d2h(hs + 2, dots, sizeof(double), stream_);
@@ -1960,15 +1951,13 @@ double Engine::davidson_core(MatvecPlan* P, double* x, double tol, int maxit, bo
       dev_d2d(t, r, sizeof(double) * n, stream_);
       for (int pass = 0; pass < 2; ++pass) {
         vec_multidot(V, n, m, t, n, dots, sc, stream_);
-        vec_combine(V, n, m, dots, 0.0, tmp, n, stream_);
-        vec_axpby(-1.0, tmp, 1.0, t, n, stream_);
+        vec_project_out(V, n, m, dots, t, n, stream_);
       }
       vec_multidot(t, n, 1, t, n, dots, sc, stream_);
       dev_d2h(hs + 2, dots, sizeof(double), stream_);
       dev_sync(stream_);
       if (!(hs[2] > 1e-30)) { conv = true; break; }
     }
-    vec_normalize(t, dots, n, stream_);
     if (m == mmax) {
       // restart on the nkeep lowest Ritz vectors
       for (int v = 0; v < nkeep; ++v) {
@@ -1987,8 +1976,9 @@ double Engine::davidson_core(MatvecPlan* P, double* x, double tol, int maxit, bo
       dev_h2d(G, Gh.data(), sizeof(double) * Gh.size(), stream_);
       m = nkeep;
     }
-    dev_d2d(V + (size_t)m * n, t, sizeof(double) * n, stream_);
-    run_matvec(P, V + (size_t)m * n, AV + (size_t)m * n, tc, GEMM_ORDERED);
+    // the new basis vector, also as the matvec's input
+    vec_normalize2(t, dots, V + (size_t)m * n, P->xin, n, stream_);
+    run_matvec(P, P->xin, AV + (size_t)m * n, tc, GEMM_ORDERED);
     // row m of the Rayleigh matrix (lower triangle is what small_eig reads)
     vec_multidot(V, n, m + 1, AV + (size_t)m * n, n, G + (size_t)m * mmax, sc, stream_);
     ++m;
@@ -2568,7 +2558,6 @@ void Engine::rdm(double* gamma, double* Gamma) {
 void Engine::rdm_site(MatvecPlan* P, int i, double* dg, bool last) {
   const double n2 = 1.0;
   // W = sum coef Z (phases 1 and the combine of the FP64 matvec)
-  if (P->zsize) dev_zero(P->Z, sizeof(double) * P->zsize, stream_);
   gemm_plan_run(P->p1, stream_, GEMM_SHARED);
   comb_plan_run(P->pc, stream_);
   const size_t nw = P->witems.size();

@@ -406,7 +406,7 @@ __device__ __forceinline__ void gemm_stream(const GemmTask* __restrict__ tasks, 
 // or the warps' rings
 template <int R, bool kRemap, bool kOrdered, bool kStream>
 __device__ __forceinline__ void gemm_job(const GemmTask* __restrict__ tasks, const GemmGroup& g, const GemmJob& J,
-                                         const Remap& rm, void* buf, bool lead_only) {
+                                         const Remap& rm, void* buf, bool lead_only, bool over) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int slots = ((g.m + R - 1) / R) * g.n;
   const int nt = g.task_end - g.task_begin;
@@ -438,7 +438,10 @@ __device__ __forceinline__ void gemm_job(const GemmTask* __restrict__ tasks, con
     }
 #pragma unroll
     for (int r = 0; r < R; ++r)
-      if (valid && i0 + r < g.m) C[(size_t)(i0 + r) * g.ldc + j] += acc[r];
+      if (valid && i0 + r < g.m) {
+        double* c = C + (size_t)(i0 + r) * g.ldc + j;
+        *c = over ? acc[r] : *c + acc[r];
+      }
   }
 }
 
@@ -447,7 +450,7 @@ __device__ __forceinline__ void gemm_job(const GemmTask* __restrict__ tasks, con
 template <bool kRemap, bool kOrdered, bool kStream>
 __global__ void __launch_bounds__(kGemmWarps * 32, kGemmMinCtas)
     k_grouped_gemm(const GemmTask* __restrict__ tasks, const GemmGroup* __restrict__ groups,
-                   const GemmJob* __restrict__ jobs, int njobs, Remap rm) {
+                   const GemmJob* __restrict__ jobs, int njobs, bool over, Remap rm) {
   extern __shared__ __align__(16) unsigned char gemm_smem[];
   const int id = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   GemmJob J{-1, 0, 0, 0, 0};
@@ -460,11 +463,11 @@ __global__ void __launch_bounds__(kGemmWarps * 32, kGemmMinCtas)
     if (pass == 1) __syncthreads();
     if (J.group >= 0 && (pass == 0 || (J.ns > 1 && J.sidx == 0))) {
       if constexpr (kStream) {
-        gemm_job<1, kRemap, kOrdered, true>(tasks, g, J, rm, gemm_smem, pass == 1);
+        gemm_job<1, kRemap, kOrdered, true>(tasks, g, J, rm, gemm_smem, pass == 1, over);
       } else {
-        if (g.rpl == 4) gemm_job<4, kRemap, kOrdered, false>(tasks, g, J, rm, gemm_smem, pass == 1);
-        else if (g.rpl == 2) gemm_job<2, kRemap, kOrdered, false>(tasks, g, J, rm, gemm_smem, pass == 1);
-        else gemm_job<1, kRemap, kOrdered, false>(tasks, g, J, rm, gemm_smem, pass == 1);
+        if (g.rpl == 4) gemm_job<4, kRemap, kOrdered, false>(tasks, g, J, rm, gemm_smem, pass == 1, over);
+        else if (g.rpl == 2) gemm_job<2, kRemap, kOrdered, false>(tasks, g, J, rm, gemm_smem, pass == 1, over);
+        else gemm_job<1, kRemap, kOrdered, false>(tasks, g, J, rm, gemm_smem, pass == 1, over);
       }
     }
   }
@@ -531,6 +534,7 @@ std::vector<GemmJob> gemm_jobs(const std::vector<GemmGroup>& g, const std::vecto
 GemmPlan* gemm_plan_upload(const std::vector<GemmTask>& t, std::vector<GemmGroup>& g, Stream s, int sums) {
   GemmPlan* p = new GemmPlan;
   p->ntasks = (int64_t)t.size();
+  p->overwrite = (sums & GEMM_OVERWRITE) != 0;
   // per group: columns in all, rows per lane; a table of at most kGemmFewSlices one-row slices
   // per SM does not fill the GPU
   std::vector<int64_t> ks(g.size(), 0);
@@ -585,7 +589,7 @@ void gemm_launch(const GemmPlan* p, const Remap& rm, int sums, Stream s) {
   // few ordered jobs: fewer warps per CTA, so that they spread over all SMs
   const int w = kind == 1 || n > 152 * 4 ? kGemmWarps : n > 152 * 2 ? 4 : n > 152 ? 2 : 1;
   auto run = [&](auto* f, size_t smem) {
-    f<<<(n + w - 1) / w, w * 32, smem, S(s)>>>(p->tasks, p->groups, p->jobs[kind], n, rm);
+    f<<<(n + w - 1) / w, w * 32, smem, S(s)>>>(p->tasks, p->groups, p->jobs[kind], n, p->overwrite, rm);
   };
   constexpr size_t direct = sizeof(double) * 128 * kGemmWarps, rings = sizeof(GemmWarpBuf) * kGemmWarps;
   if (kind == 1) {
@@ -803,7 +807,7 @@ __global__ void k_multidot_partial(const double* __restrict__ V, int64_t ldv,
     if (threadIdx.x < o) sh[threadIdx.x] += sh[threadIdx.x + o];
     __syncthreads();
   }
-  if (threadIdx.x == 0) part[(size_t)j * nch + c] = sh[0];
+  if (threadIdx.x == 0) part[(size_t)j * nch + c] = sh[0];  // the result itself when nch == 1
 }
 
 __global__ void k_multidot_final(const double* __restrict__ part, int nch, int m, double* out) {
@@ -848,15 +852,57 @@ __global__ void k_normalize(double* __restrict__ y, const double* __restrict__ n
     y[i] *= s;
 }
 
-__global__ void k_precondition(const double* __restrict__ r, const double* __restrict__ d,
-                               const double* __restrict__ theta, double* __restrict__ t,
-                               int64_t n) {
+// One Davidson iteration's elementwise work, fused (each was three to five launches of 2 to 3
+// us over vectors that fit in L2; the same operations per element in the same order).
+// x = sum_j c_j V_j, r = sum_j c_j AV_j - theta x, t = r / (theta - d), the denominator floored
+__global__ void k_ritz(const double* __restrict__ V, const double* __restrict__ AV, int64_t ldv, int m,
+                       const double* __restrict__ c, const double* __restrict__ theta, const double* __restrict__ d,
+                       double* __restrict__ x, double* __restrict__ r, double* __restrict__ t, int64_t n) {
+  __shared__ double cs[128];
+  for (int j = threadIdx.x; j < m; j += blockDim.x) cs[j] = c[j];
+  __syncthreads();
   const double th = *theta;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
        i += (int64_t)gridDim.x * blockDim.x) {
+    double xs = 0.0, rs = 0.0;
+#pragma unroll 4
+    for (int j = 0; j < m; ++j) {
+      xs += cs[j] * V[(size_t)j * ldv + i];
+      rs += cs[j] * AV[(size_t)j * ldv + i];
+    }
+    x[i] = xs;
+    rs = fma(-th, xs, rs);
+    r[i] = rs;
     double den = th - d[i];
     if (fabs(den) < 1e-12) den = den < 0 ? -1e-12 : 1e-12;
-    t[i] = r[i] / den;
+    t[i] = rs / den;
+  }
+}
+
+// t -= sum_j c_j V_j
+__global__ void k_project_out(const double* __restrict__ V, int64_t ldv, int m, const double* __restrict__ c,
+                              double* __restrict__ t, int64_t n) {
+  __shared__ double cs[128];
+  for (int j = threadIdx.x; j < m; j += blockDim.x) cs[j] = c[j];
+  __syncthreads();
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
+       i += (int64_t)gridDim.x * blockDim.x) {
+    double s = 0.0;
+#pragma unroll 4
+    for (int j = 0; j < m; ++j) s += cs[j] * V[(size_t)j * ldv + i];
+    t[i] = t[i] - s;
+  }
+}
+
+// a = b = t / sqrt(*nrm2)
+__global__ void k_normalize2(const double* __restrict__ t, const double* __restrict__ nrm2, double* __restrict__ a,
+                             double* __restrict__ b, int64_t n) {
+  const double s = *nrm2 > 0.0 ? 1.0 / sqrt(*nrm2) : 0.0;
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
+       i += (int64_t)gridDim.x * blockDim.x) {
+    const double v = t[i] * s;
+    a[i] = v;
+    b[i] = v;
   }
 }
 
@@ -1227,10 +1273,12 @@ void vec_multidot(const double* V, int64_t ldv, int m, const double* w, int64_t 
   if (m <= 0) return;
   int nch = (int)std::min<int64_t>(kMaxChunks, std::max<int64_t>(1, (n + kDotChunk - 1) / kDotChunk));
   dim3 grid(nch, m);
-  k_multidot_partial<<<grid, 256, 0, S(s)>>>(V, ldv, w, n, nch, scratch);
+  k_multidot_partial<<<grid, 256, 0, S(s)>>>(V, ldv, w, n, nch, nch == 1 ? out : scratch);
   ++g_launches;
-  k_multidot_final<<<m, 256, 0, S(s)>>>(scratch, nch, m, out);
-  ++g_launches;
+  if (nch > 1) {
+    k_multidot_final<<<m, 256, 0, S(s)>>>(scratch, nch, m, out);
+    ++g_launches;
+  }
   ck(cudaGetLastError(), "multidot");
 }
 
@@ -1253,11 +1301,23 @@ void vec_normalize(double* y, const double* nrm2, int64_t n, Stream s) {
   ck(cudaGetLastError(), "normalize");
 }
 
-void vec_precondition(const double* r, const double* d, const double* th, double* t, int64_t n,
-                      Stream s) {
-  k_precondition<<<nblk(n, 256), 256, 0, S(s)>>>(r, d, th, t, n);
+void vec_ritz(const double* V, const double* AV, int64_t ldv, int m, const double* c, const double* theta, const double* d,
+              double* x, double* r, double* t, int64_t n, Stream s) {
+  k_ritz<<<nblk(n, 128), 128, 0, S(s)>>>(V, AV, ldv, m, c, theta, d, x, r, t, n);
   ++g_launches;
-  ck(cudaGetLastError(), "precondition");
+  ck(cudaGetLastError(), "ritz");
+}
+
+void vec_project_out(const double* V, int64_t ldv, int m, const double* c, double* t, int64_t n, Stream s) {
+  k_project_out<<<nblk(n, 128), 128, 0, S(s)>>>(V, ldv, m, c, t, n);
+  ++g_launches;
+  ck(cudaGetLastError(), "project out");
+}
+
+void vec_normalize2(const double* t, const double* nrm2, double* a, double* b, int64_t n, Stream s) {
+  k_normalize2<<<nblk(n, 256), 256, 0, S(s)>>>(t, nrm2, a, b, n);
+  ++g_launches;
+  ck(cudaGetLastError(), "normalize2");
 }
 
 namespace {
@@ -2456,8 +2516,7 @@ void noalloc_matvec_run(const GemmPlan* p1, const CombPlan* pc, const GemmPlan* 
   rm.lo[1] = (const char*)yout; rm.hi[1] = (const char*)(yout + n);    rm.to[1] = (char*)y;
   rm.lo[2] = (const char*)Z;    rm.hi[2] = (const char*)(Z + zsize);   rm.to[2] = (char*)scratch;
   rm.lo[3] = (const char*)Wb;   rm.hi[3] = (const char*)(Wb + wsize);  rm.to[3] = (char*)(scratch + zsize);
-  // phase 1 accumulates into Z and phase 2 into y: both start at zero; W is overwritten
-  if (zsize) ck(cudaMemsetAsync(scratch, 0, sizeof(double) * zsize, S(s)), "memset scratch");
+  // phase 2 accumulates into y, which starts at zero; Z and W are overwritten
   if (n) ck(cudaMemsetAsync(y, 0, sizeof(double) * n, S(s)), "memset y");
   gemm_launch<true>(p1, rm, GEMM_SHARED, s);
   if (pc && pc->ndst) {

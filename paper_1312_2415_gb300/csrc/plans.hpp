@@ -19,6 +19,7 @@ struct GemmPlan {
   GemmGroup* groups = nullptr;
   GemmJob* jobs[2] = {nullptr, nullptr};  // ordered sums, shared sums
   int njobs[2] = {0, 0};
+  bool overwrite = false;  // C = sum instead of C += sum
   bool few = false;  // too small to fill the GPU: the streamed kernel
   int64_t ntasks = 0;
 };
