@@ -619,6 +619,22 @@ void Engine::group_right(int j, std::vector<CombOp>& out, double** scratch, int6
   *scratch = materialise(out, E, stream_, scratch_n);
 }
 
+// The patterns' allowed site transitions (patterns are only ever added).
+const std::vector<Engine::SiteOk>& Engine::site_ok() {
+  static const int ls_of[4] = {0, 1, 1, 2};
+  for (size_t k = site_ok_.size(); k < pt_.pats.size(); ++k) {
+    const Pattern& P = pt_.pats[k];
+    SiteOk ok{};
+    const int nq = (P.tka + 1) * (P.tkb + 1);
+    for (int q = 0; q < nq; ++q)
+      for (int br = 0; br < 4; ++br)
+        for (int kt = 0; kt < 4; ++kt)
+          if (P.w[(size_t)q * 16 + br * 4 + kt] != 0.0) ok[ls_of[kt]][ls_of[br]] = true;
+    site_ok_.push_back(ok);
+  }
+  return site_ok_;
+}
+
 // L_b(bond i+1)[jM' <- jM] = sum coef T[i]^T C_{b,P}[jL' <- jL] T[i], T[i] left-normalised.
 void Engine::update_left_from(int i, std::vector<CombOp>& comb) {
   Timer tm;
@@ -642,8 +658,12 @@ void Engine::update_left_from(int i, std::vector<CombOp>& comb) {
   g1.reserve(upd_hint_z_ + upd_hint_z_ / 4);
   zs.reserve(upd_hint_z_ + upd_hint_z_ / 4);
   out2.reserve(upd_hint_out_ + upd_hint_out_ / 4);
+  // the pattern's forbidden site transitions (most of the nine) are skipped before their
+  // zero coefficient is looked up
+  const auto& okp = site_ok();
   for (auto& c : comb) {
     if (c.target == id_op) continue;
+    const SiteOk& ok = okp[c.pattern];
     for (const BlockRef& cb : *c.blocks) {
       for (int t : by_l[cb.c]) {
         const SiteBlock& tb = T.blocks[t];
@@ -651,6 +671,7 @@ void Engine::update_left_from(int i, std::vector<CombOp>& comb) {
         int zid = -1;
         for (int tp : by_l[cb.r]) {
           const SiteBlock& tpb = T.blocks[tp];
+          if (!ok[tb.ls][tpb.ls]) continue;
           double coef = c.scalar * cp_->left(c.pattern, bl.sec[tb.l].tj, tb.ls, bm.sec[tb.r].tj,
                                               bl.sec[tpb.l].tj, tpb.ls, bm.sec[tpb.r].tj);
           if (coef == 0.0) continue;
@@ -725,14 +746,17 @@ void Engine::update_right_from(int j, std::vector<CombOp>& comb) {
   g1.reserve(upd_hint_z_ + upd_hint_z_ / 4);
   zs.reserve(upd_hint_z_ + upd_hint_z_ / 4);
   out2.reserve(upd_hint_out_ + upd_hint_out_ / 4);
+  const auto& okp = site_ok();
   for (auto& c : comb) {
     if (c.target == h_op) continue;
+    const SiteOk& ok = okp[c.pattern];
     for (const BlockRef& db : *c.blocks) {
       for (int t : by_r[db.c]) {
         const SiteBlock& tb = T.blocks[t];
         int zid = -1;
         for (int tp : by_r[db.r]) {
           const SiteBlock& tpb = T.blocks[tp];
+          if (!ok[tb.ls][tpb.ls]) continue;
           double coef = c.scalar * f(tb) * f(tpb) *
                         cp_->right(c.pattern, tb.ls, br.sec[tb.r].tj, bm.sec[tb.l].tj, tpb.ls,
                                    br.sec[tpb.r].tj, bm.sec[tpb.l].tj);
@@ -865,20 +889,6 @@ struct Engine::MatvecPlan {
   double* lowc = nullptr;
 };
 
-namespace {
-// site transitions allowed by a pattern: ok[ket ls][bra ls]
-void allowed(const Pattern& P, bool ok[3][3]) {
-  static const int ls_of[4] = {0, 1, 1, 2};
-  for (int a = 0; a < 3; ++a)
-    for (int b = 0; b < 3; ++b) ok[a][b] = false;
-  const int nq = (P.tka + 1) * (P.tkb + 1);
-  for (int q = 0; q < nq; ++q)
-    for (int br = 0; br < 4; ++br)
-      for (int kt = 0; kt < 4; ++kt)
-        if (P.w[(size_t)q * 16 + br * 4 + kt] != 0.0) ok[ls_of[kt]][ls_of[br]] = true;
-}
-}  // namespace
-
 Engine::MatvecPlan* Engine::plan_matvec(int i, bool rdm) {
   Timer tm;
   ensure_left(i);
@@ -954,13 +964,7 @@ Engine::MatvecPlan* Engine::plan_matvec(int i, bool rdm) {
   };
   // site transitions allowed by each pattern, and the recoupled coefficient of a
   // (left pattern, right pattern, block labels) combination, memoised
-  std::vector<std::array<std::array<bool, 3>, 3>> okp(pt_.pats.size());
-  for (size_t q = 0; q < pt_.pats.size(); ++q) {
-    bool ok[3][3];
-    allowed(pt_.pats[q], ok);
-    for (int a = 0; a < 3; ++a)
-      for (int c = 0; c < 3; ++c) okp[q][a][c] = ok[a][c];
-  }
+  const auto& okp = site_ok();
   using K2 = CoefKey;
   // W(gl, C block, X') = sum coef * Z rows of X ; phase 2: y_X' += C_blk W
   struct WItem { int gl, cbi, xp; int64_t off; int rows, cols; int src_begin, src_end; };
@@ -997,7 +1001,7 @@ Engine::MatvecPlan* Engine::plan_matvec(int i, bool rdm) {
   std::mutex worker_mu;
   std::exception_ptr worker_err;
   auto worker_body = [&]() {
-    Coupling cp = *cp_;  // private memo tables
+    std::unique_ptr<Coupling> cpw;  // private memo tables, copied at the first coefficient not seen before
     auto& coef_cache = new_coefs[next_worker.fetch_add(1)];
     coef_cache.reserve(1 << 12);
     std::vector<int> slot(P->X.size(), -1), touched;
@@ -1043,6 +1047,8 @@ Engine::MatvecPlan* Engine::plan_matvec(int i, bool rdm) {
                   } else if (mi != master.end()) {
                     coef = mi->second;
                   } else {
+                    if (!cpw) cpw.reset(new Coupling(*cp_));
+                    Coupling& cp = *cpw;
                     for (int tjM = std::abs(tjL - t1s); tjM <= tjL + t1s; tjM += 2) {
                       if (!triangle(t2s, tjR, tjM)) continue;
                       double ov = cp.overlap(tjL, X.ls1, X.ls2, X.tj, tjR, tjM);
@@ -1089,8 +1095,10 @@ Engine::MatvecPlan* Engine::plan_matvec(int i, bool rdm) {
     }
   };
   {
-    const unsigned hc = std::thread::hardware_concurrency();
-    const int nth = (int)std::max(1u, std::min(16u, hc ? hc : 1u));
+    // a thread for every kItemsPerThread items (a small pair's tables take less time than
+    // starting 15 threads)
+    constexpr size_t kItemsPerThread = 96;
+    const int nth = (int)std::min<size_t>(nthw, items.size() / kItemsPerThread + 1);
     std::vector<std::thread> th;
     auto worker = [&]() {
       try {
@@ -1101,7 +1109,7 @@ Engine::MatvecPlan* Engine::plan_matvec(int i, bool rdm) {
         next_item.store(items.size());
       }
     };
-    for (int t = 1; t < nth && (size_t)t < items.size(); ++t) th.emplace_back(worker);
+    for (int t = 1; t < nth; ++t) th.emplace_back(worker);
     worker();
     for (auto& t : th) t.join();
     if (worker_err) std::rethrow_exception(worker_err);

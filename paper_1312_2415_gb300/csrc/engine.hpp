@@ -1,5 +1,6 @@
 // Host orchestration of the two-site spin-adapted DMRG on one GPU.
 #pragma once
+#include <array>
 #include <cstdint>
 #include <map>
 #include <memory>
@@ -243,6 +244,10 @@ class Engine {
   bool have_integrals_ = false, have_mps_ = false;
   std::vector<OpSet> opsets_;
   PatternTable pt_;
+  // site transitions a pattern allows: ok[ket local state][bra local state]
+  using SiteOk = std::array<std::array<bool, 3>, 3>;
+  const std::vector<SiteOk>& site_ok();
+  std::vector<SiteOk> site_ok_;
   std::unique_ptr<Coupling> cp_;
   std::vector<std::vector<WEntry>> W_;
   std::vector<std::vector<WEntry>> Wg_;  // W_ with the terms of every allowed integral
