@@ -113,13 +113,7 @@ void wait_user(uintptr_t stream) {
   }
 }
 
-dmrg::Stream dev_stream(dmrg_ctx* c);
-int64_t xsize(dmrg_ctx* c, int site) {
-  std::vector<int64_t> t;
-  int64_t n = 0;
-  c->eng->layout(site, t, n);
-  return n;
-}
+int64_t xsize(dmrg_ctx* c, int site) { return c->eng->x_size(site); }
 
 }  // namespace
 

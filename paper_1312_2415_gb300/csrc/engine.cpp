@@ -23,8 +23,6 @@ namespace dmrg {
 
 namespace {
 
-inline int64_t bkey(int r, int c) { return ((int64_t)r << 32) | (uint32_t)c; }
-
 // Tasks tagged with an output index, grouped per output in increasing index order
 // (stable: a group's tasks keep their order); zs[id] gives the Z offset of a task whose
 // B holds a Z id.
@@ -394,20 +392,22 @@ void Engine::alloc_env(OpStore& e, int bond, const OpSet& ops) {
   const Bond& B = bonds_[bond];
   e.bond = bond;
   e.blocks.resize(ops.ops.size());
-  e.at.resize(ops.ops.size());
+  e.col.resize(ops.ops.size());
   int64_t off = 0;
   for (size_t o = 0; o < ops.ops.size(); ++o) {
     const OpInfo& op = ops.ops[o];
+    e.col[o].reserve(B.sec.size() + 1);
     for (int c = 0; c < (int)B.sec.size(); ++c) {
+      e.col[o].push_back((int)e.blocks[o].size());
       const Sector& sc = B.sec[c];
       for (int tj = std::abs(sc.tj - op.tk); tj <= sc.tj + op.tk; tj += 2) {
         int r = B.find({tj, sc.n + op.dn, sc.ir ^ op.ir});
         if (r < 0) continue;
-        e.at[o][bkey(r, c)] = (int)e.blocks[o].size();
         e.blocks[o].push_back({r, c, off, B.dim[r], B.dim[c]});
         off += (int64_t)B.dim[r] * B.dim[c];
       }
     }
+    e.col[o].push_back((int)e.blocks[o].size());
   }
   e.size = off;
   e.data = (double*)dev_alloc(sizeof(double) * std::max<int64_t>(off, 1), stream_);
@@ -523,18 +523,16 @@ double* materialise(std::vector<CombOp>& comb, const OpStore& src, Stream st, in
     if (c.sources.size() <= 1) continue;
     const auto& proto = src.blocks[c.sources[0].first];
     c.own_blocks.clear();
-    c.own_at.clear();
     for (size_t bi = 0; bi < proto.size(); ++bi) {
       const BlockRef& pb = proto[bi];
       BlockRef nb = pb;
       nb.off = off;
-      c.own_at[bkey(pb.r, pb.c)] = (int)c.own_blocks.size();
       c.own_blocks.push_back(nb);
       CombDst d{buf + off, pb.cols, pb.rows, pb.cols, (int)cs.size(), 0, 0};
       for (auto& s : c.sources) {
-        auto it = src.at[s.first].find(bkey(pb.r, pb.c));
-        if (it == src.at[s.first].end()) throw std::logic_error("combined sources differ in blocks");
-        const BlockRef& sb = src.blocks[s.first][it->second];
+        const int at = src.find(s.first, pb.r, pb.c);
+        if (at < 0) throw std::logic_error("combined sources differ in blocks");
+        const BlockRef& sb = src.blocks[s.first][at];
         cs.push_back({src.data + sb.off, sb.cols, s.second});
       }
       d.src_end = (int)cs.size();
@@ -542,7 +540,6 @@ double* materialise(std::vector<CombOp>& comb, const OpStore& src, Stream st, in
       off += (int64_t)pb.rows * pb.cols;
     }
     c.blocks = &c.own_blocks;
-    c.at = &c.own_at;
     c.data = buf;
     c.scalar = 1.0;
   }
@@ -578,7 +575,6 @@ void Engine::group_left(int i, std::vector<CombOp>& out, double** scratch, int64
   for (auto& c : out)
     if (c.sources.size() == 1) {
       c.blocks = &E.blocks[c.sources[0].first];
-      c.at = &E.at[c.sources[0].first];
       c.data = E.data;
       c.scalar = c.sources[0].second;
       c.identity = c.sources[0].first == id_op;
@@ -611,7 +607,6 @@ void Engine::group_right(int j, std::vector<CombOp>& out, double** scratch, int6
   for (auto& c : out)
     if (c.sources.size() == 1) {
       c.blocks = &E.blocks[c.sources[0].first];
-      c.at = &E.at[c.sources[0].first];
       c.data = E.data;
       c.scalar = c.sources[0].second;
       c.identity = c.sources[0].first == h_op;  // partner of H is the identity
@@ -675,8 +670,8 @@ void Engine::update_left_from(int i, std::vector<CombOp>& comb) {
           double coef = c.scalar * cp_->left(c.pattern, bl.sec[tb.l].tj, tb.ls, bm.sec[tb.r].tj,
                                               bl.sec[tpb.l].tj, tpb.ls, bm.sec[tpb.r].tj);
           if (coef == 0.0) continue;
-          auto it = E.at[c.target].find(bkey(tpb.r, tb.r));
-          if (it == E.at[c.target].end()) continue;
+          const int at = E.find(c.target, tpb.r, tb.r);
+          if (at < 0) continue;
           if (zid < 0) {
             zid = (int)zs.size();
             zs.push_back({zsize, cb.rows, tb.cols});
@@ -684,7 +679,7 @@ void Engine::update_left_from(int i, std::vector<CombOp>& comb) {
             t1.push_back({c.data + cb.off, T.data + tb.off, cb.cols, tb.cols, cb.cols, 0, 0, 1.0});
             g1.push_back({nullptr, tb.cols, cb.rows, tb.cols, (int)t1.size() - 1, (int)t1.size(), 0});
           }
-          out2.push_back({bbase[c.target] + it->second,
+          out2.push_back({bbase[c.target] + at,
                           {T.data + tpb.off, (const double*)(intptr_t)zid, tpb.cols, tb.cols, tpb.rows, 1, 0, coef}});
         }
       }
@@ -761,8 +756,8 @@ void Engine::update_right_from(int j, std::vector<CombOp>& comb) {
                         cp_->right(c.pattern, tb.ls, br.sec[tb.r].tj, bm.sec[tb.l].tj, tpb.ls,
                                    br.sec[tpb.r].tj, bm.sec[tpb.l].tj);
           if (coef == 0.0) continue;
-          auto it = E.at[c.target].find(bkey(tpb.l, tb.l));
-          if (it == E.at[c.target].end()) continue;
+          const int at = E.find(c.target, tpb.l, tb.l);
+          if (at < 0) continue;
           if (zid < 0) {
             // Z1 = D_blk (dR' x dR) . T_t^T (dR x dM)
             zid = (int)zs.size();
@@ -771,7 +766,7 @@ void Engine::update_right_from(int j, std::vector<CombOp>& comb) {
             t1.push_back({c.data + db.off, T.data + tb.off, db.cols, tb.cols, db.cols, 0, 1, 1.0});
             g1.push_back({nullptr, tb.rows, db.rows, tb.rows, (int)t1.size() - 1, (int)t1.size(), 0});
           }
-          out2.push_back({bbase[c.target] + it->second,
+          out2.push_back({bbase[c.target] + at,
                           {T.data + tpb.off, (const double*)(intptr_t)zid, tpb.cols, tb.rows, tpb.cols, 0, 0, coef}});
         }
       }
@@ -1512,6 +1507,15 @@ Engine::TcView Engine::prepare_tc(int i, TcTune tune) {
     throw;
   }
   return {&p->tch, p->serial, p->xin, p->yout, p->n, p->flops, p->diag};
+}
+
+int64_t Engine::x_size(int i) const {
+  check_ready();
+  if (i < 0 || i > L_ - 2) throw std::out_of_range("site out of range");
+  if (cached_ && cached_site_ == i) return cached_->n;  // a plan lives only as long as its bonds
+  int64_t n = 0;
+  x_layout(i, &n);
+  return n;
 }
 
 double Engine::rayleigh_fp64(int i, const double* x) {
@@ -2641,9 +2645,9 @@ void Engine::rdm_site(MatvecPlan* P, int i, double* dg, bool last) {
         const int64_t gi = C.grad[s].first;
         if (gi < 0) continue;
         const int a = C.sources[s].first;
-        auto it = E.at[a].find(bkey(cb.r, cb.c));
-        if (it == E.at[a].end()) continue;
-        const BlockRef& lb = E.blocks[a][it->second];
+        const int at = E.find(a, cb.r, cb.c);
+        if (at < 0) continue;
+        const BlockRef& lb = E.blocks[a][at];
         dots[gi].push_back({E.data + lb.off, gb, lb.cols, cb.cols, cb.rows, cb.cols, C.grad[s].second});
       }
     }

@@ -28,7 +28,13 @@ struct OpStore {
   int bond = -1;
   uint64_t serial = 0;  // distinct for every allocation (overlaps record the one they match)
   std::vector<std::vector<BlockRef>> blocks;         // per operator
-  std::vector<std::unordered_map<int64_t, int>> at;  // (r << 32 | c) -> block index
+  std::vector<std::vector<int>> col;  // per operator: its first block of every column sector (at most three each)
+  // block of operator op from column sector c to row sector r, -1: none
+  int find(int op, int r, int c) const {
+    for (int b = col[op][c]; b < col[op][c + 1]; ++b)
+      if (blocks[op][b].r == r) return b;
+    return -1;
+  }
   double* data = nullptr;
   int64_t size = 0;
 };
@@ -58,11 +64,9 @@ struct CombOp {
   double scalar = 1.0;           // multiplies the blocks (alias) or 1 (materialised)
   bool identity = false;         // the operator is the identity (scaled by scalar)
   const std::vector<BlockRef>* blocks = nullptr;
-  const std::unordered_map<int64_t, int>* at = nullptr;
   const double* data = nullptr;  // base of the blocks
   // materialised storage
   std::vector<BlockRef> own_blocks;
-  std::unordered_map<int64_t, int> own_at;
   std::vector<std::pair<int, double>> sources;  // (operator index, scalar)
   std::vector<std::pair<int64_t, double>> grad;  // (gi, gc) of each source's recursion term
 };
@@ -134,6 +138,7 @@ class Engine {
   // two-site probes (site i means orbitals i, i+1); the MPS must be in mixed canonical
   // form around i (left-normalised left of i, right-normalised right of i+1)
   void layout(int i, std::vector<int64_t>& table, int64_t& n);
+  int64_t x_size(int i) const;  // elements of the two-site vector
   void tt_to_x(int i, double* x_dev);
   void matvec(int i, const double* x_dev, double* y_dev);
   void diag(int i, double* d_dev);
