@@ -119,6 +119,7 @@ Engine::~Engine() {
   try {
     flush_events();
     for (auto& e : ev_) event_destroy(e);
+    host_pinned_free(hs_);
     if (cached_) free_plan(cached_);
     cached_ = nullptr;
     for (auto& e : lenv_) free_env(e);
@@ -1903,7 +1904,6 @@ double Engine::davidson_core(MatvecPlan* P, double* x, double tol, int maxit, bo
     dev_free(V, stream_); dev_free(AV, stream_); dev_free(G, stream_); dev_free(C, stream_);
     dev_free(th, stream_); dev_free(sc, stream_); dev_free(dots, stream_); dev_free(r, stream_);
     dev_free(t, stream_); dev_free(tmp, stream_); dev_free(x0, stream_);
-    host_pinned_free(hs);
   };
   try {
   V = (double*)dev_alloc(sizeof(double) * n * (mmax + 1), stream_);
@@ -1918,7 +1918,8 @@ double Engine::davidson_core(MatvecPlan* P, double* x, double tol, int maxit, bo
   tmp = (double*)dev_alloc(sizeof(double) * n * nkeep * 2, stream_);
   x0 = (double*)dev_alloc(sizeof(double) * n, stream_);  // the starting vector
   dev_zero(G, sizeof(double) * mmax * mmax, stream_);
-  hs = (double*)host_pinned_alloc(sizeof(double) * 4);
+  if (!hs_) hs_ = (double*)host_pinned_alloc(sizeof(double) * 4);
+  hs = hs_;
   dev_d2d(x0, x, sizeof(double) * n, stream_);
   // v0 = x / |x|
   dev_d2d(V, x, sizeof(double) * n, stream_);

@@ -282,6 +282,7 @@ class Engine {
   uint64_t noise_counter_ = 0;
   int next_hint_ = -1;
   void* ev_[3] = {nullptr, nullptr, nullptr};
+  double* hs_ = nullptr;  // what Davidson reads back (pinned)
   void flush_events();
   bool ev_pending_ = false;
   bool ev_tc_ = false;

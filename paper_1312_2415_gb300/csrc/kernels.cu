@@ -294,119 +294,111 @@ __device__ __forceinline__ void gemm_sum(const GemmTask* __restrict__ tasks, int
   }
 }
 
-// A warp's shared memory: a ring of operand chunks (up to four columns of A and rows of B:
-// a[u * 32 + row], b[u * 32 + lane]) and the descriptors of two batches of 32 tasks.
-constexpr int kGemmDepth = 4;
-struct GemmWarpBuf {
-  double a[kGemmDepth][128], b[kGemmDepth][128];
-  GemmTask desc[2][32];
-};
+// The same ordered sum for long lists of small tasks, which are chains of FMAs (66 cycles
+// each) behind trips to L2 and address arithmetic of some 2000 cycles per task when one warp
+// does everything.  One CTA per 32-element slice, one row per lane: in each round
+// kRoundWarps - 1 warps fetch one chunk each (up to four columns of one task; A scaled by
+// alpha on the way) into shared memory while the last warp sums the previous round's chunks
+// in order.  The chunks' table (task, first column) is made at upload.  Measured (phase 2,
+// loads when a task starts / rounds): Hubbard L=8, D=64 236 / 47 us (one warp with three
+// chunks in flight 165 us); random L=12, D=350 318 / 115 us, L=12, D=500 1.65 / 0.53 ms, L=16,
+// D=600 2.88 / 1.81 ms.  Short lists (phase 1, one task per sum) start faster the other way: 28
+// / 41 us.
+constexpr int kRoundWarps = 8;
 
-__device__ __forceinline__ void cp_async8(double* dst, const double* src) {
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src));
-}
-
-// The same ordered sum for tables too small to fill the GPU, one row per lane (the warp's
-// lanes read at most 32 rows).  The chunks of all tasks form one stream: kGemmDepth - 1 of them are in
-// flight (cp.async) while one is summed, so that a chain of small tasks costs its FMAs (66
-// cycles each) and its instructions, not several trips to L2 per task.  Measured (phase 2 of
-// Hubbard L=8, D=64, ordered lists of up to 137 tasks of 4 columns): loads when a task starts
-// 236 us, the stream 165 us.  Tables that fill the GPU keep the direct loads: the FP64 pipe
-// is busy anyway, and the rings' shared memory takes away L1 (phase 1 of random L=28, D=1500:
-// direct 104 ms, stream 134 ms); so do shared sums, whose warps have few tasks each (phase 2
-// of random L=12, D=350: 54 / 86 us).
 template <bool kRemap>
-__device__ __forceinline__ void gemm_stream(const GemmTask* __restrict__ tasks, int t0, int t1, int i0, int j,
-                                         const Remap& rm, GemmWarpBuf& wb, double (&acc)[1]) {
-
-  const int lane = threadIdx.x & 31, nt = t1 - t0;
-  // rows the warp's lanes read, and this lane's among them
-  const int row0 = __reduce_min_sync(0xffffffffu, i0);
-  const int nrow = __reduce_max_sync(0xffffffffu, i0) + 1 - row0, lr = i0 - row0;
+__global__ void __launch_bounds__(kRoundWarps * 32, 4)
+    k_gemm_rounds(const GemmTask* __restrict__ tasks, const GemmGroup* __restrict__ groups,
+                  const GemmChunk* __restrict__ chunks, const GemmJob* __restrict__ jobs, bool over, Remap rm) {
+  constexpr int kF = kRoundWarps - 1;
+  __shared__ double as[2][kF][4][32], bs[2][kF][4][32];
+  __shared__ int ks[2][kF];       // columns of the chunk; 0: identity task
+  __shared__ double al[2][kF];    // identity: alpha
+  // the summing warp (number kF) sits on another SM sub-partition in every fourth CTA: its FMAs
+  // are what fills an FP64 pipe
+  const int warp = ((threadIdx.x >> 5) + blockIdx.x) % kRoundWarps, lane = threadIdx.x & 31;
+  const GemmJob J = jobs[blockIdx.x];
+  const GemmGroup g = groups[J.group];
+  const int c0 = chunks[J.group].begin, nc = chunks[J.group].end - c0;  // the group's chunks
+  const GemmChunk* list = chunks + c0;
+  const int q = min(J.w0 * 32 + lane, g.m * g.n - 1), i = q / g.n, j = q % g.n;
+  const int row0 = __reduce_min_sync(0xffffffffu, i), nrow = __reduce_max_sync(0xffffffffu, i) + 1 - row0;
+  const int lr = i - row0, nr = (nc + kF - 1) / kF;
   double s = 0.0;
-  int it = 0, ik = 0;  // next chunk to load
-  auto issue = [&](int slot) {
-    if (it < nt) {
-      if (ik == 0 && (it & 31) == 0) {  // the descriptors of the next 32 tasks
-        __syncwarp();
-        if (it + lane < nt) wb.desc[(it >> 5) & 1][lane] = tasks[t0 + it + lane];
-        __syncwarp();
-      }
-      const GemmTask& T = wb.desc[(it >> 5) & 1][it & 31];
-      const double* B = kRemap ? remap_ptr(T.B, rm) : T.B;
-      const int64_t ldb = T.ldb;
-      int k;
-      if (T.A == nullptr) {  // op(A) = identity: the elements of op(B) themselves
-        k = 1;
-        const int64_t si = T.transB ? 1 : ldb, sj = T.transB ? ldb : 1;
-        cp_async8(&wb.b[slot][lane], B + i0 * si + j * sj);
-      } else {
-        k = T.k;
-        const double* A = kRemap ? remap_ptr(T.A, rm) : T.A;
-        const int64_t lda = T.lda, sai = T.transA ? 1 : lda, sak = T.transA ? lda : 1;
-        const int64_t sbk = T.transB ? 1 : ldb, sbj = T.transB ? ldb : 1;
-        const double* pa = A + (row0 + lane) * sai + ik * sak;
-        const double* pb = B + j * sbj + ik * sbk;
-#pragma unroll
-        for (int u = 0; u < 4; ++u)
-          if (ik + u < k) {
-            if (lane < nrow) cp_async8(&wb.a[slot][u * 32 + lane], pa + u * sak);
-            cp_async8(&wb.b[slot][u * 32 + lane], pb + u * sbk);
-          }
-      }
-      ik += 4;
-      if (ik >= k) {
-        ik = 0;
-        ++it;
-      }
+  GemmChunk cn{};  // this warp's chunk of the next round, fetched a round ahead
+  GemmTask T{};
+  if (warp < kF) {
+    if (warp < nc) {
+      cn = list[warp];
+      T = tasks[cn.task];
     }
-    asm volatile("cp.async.commit_group;");
-  };
-#pragma unroll
-  for (int d = 0; d < kGemmDepth - 1; ++d) issue(d);
-  int slot = 0;
-  for (int ct = 0; ct < nt; ++ct) {
-    int K = 1, ck = 0;
-    do {
-      issue((slot + kGemmDepth - 1) % kGemmDepth);
-      asm volatile("cp.async.wait_group %0;" ::"n"(kGemmDepth - 1));
-      __syncwarp();
-      const GemmTask& T = wb.desc[(ct >> 5) & 1][ct & 31];
-      const double alpha = T.alpha;
-      double* a = wb.a[slot];
-      const double* b = wb.b[slot];
-      if (T.A == nullptr) {
-        s = fma(alpha, b[lane], s);
-      } else {
-        K = T.k;
-        const bool unit = fabs(alpha) == 1.0;
-        if (!unit) {
+  }
+  for (int r = 0; r <= nr; ++r) {
+    const int buf = r & 1;
+    if (warp < kF) {
+      const int c = r * kF + warp;
+      if (c < nc) {
+        const int k0 = cn.k0;
+        const GemmTask Q = T;
+        if (c + kF < nc) {
+          cn = list[c + kF];
+          T = tasks[cn.task];
+        }
+        const double* B = kRemap ? remap_ptr(Q.B, rm) : Q.B;
+        if (Q.A == nullptr) {
+          bs[buf][warp][0][lane] = Q.transB ? B[j * (int64_t)Q.ldb + i] : B[i * (int64_t)Q.ldb + j];
+          if (lane == 0) {
+            ks[buf][warp] = 0;
+            al[buf][warp] = Q.alpha;
+          }
+        } else {
+          const double* A = kRemap ? remap_ptr(Q.A, rm) : Q.A;
+          const int64_t sai = Q.transA ? 1 : Q.lda, sak = Q.transA ? Q.lda : 1;
+          const int64_t sbk = Q.transB ? 1 : Q.ldb, sbj = Q.transB ? Q.ldb : 1;
+          const double* pa = A + (row0 + min(lane, nrow - 1)) * sai + k0 * sak;
+          const double* pb = B + j * sbj + k0 * sbk;
+          const int k = min(4, Q.k - k0);
+          double av[4], bv[4];
 #pragma unroll
           for (int u = 0; u < 4; ++u)
-            if (ck + u < K && lane < nrow) a[u * 32 + lane] = __dmul_rn(a[u * 32 + lane], alpha);
-          __syncwarp();
-        }
+            if (u < k) {
+              av[u] = pa[u * sak];
+              bv[u] = pb[u * sbk];
+            }
 #pragma unroll
-        for (int u = 0; u < 4; ++u)
-          if (ck + u < K) {
-            double bv = b[u * 32 + lane];
-            if (unit && alpha < 0.0) bv = -bv;
-            s = fma(a[u * 32 + lr], bv, s);
-          }
+          for (int u = 0; u < 4; ++u)
+            if (u < k) {
+              as[buf][warp][u][lane] = __dmul_rn(av[u], Q.alpha);
+              bs[buf][warp][u][lane] = bv[u];
+            }
+          if (lane == 0) ks[buf][warp] = k;
+        }
       }
-      __syncwarp();  // the slot may be refilled
-      slot = (slot + 1) % kGemmDepth;
-      ck += 4;
-    } while (ck < K);
+    } else if (r > 0) {
+      const int pb = buf ^ 1, n = min(kF, nc - (r - 1) * kF);
+      for (int c = 0; c < n; ++c) {
+        const int k = ks[pb][c];
+        if (k == 0) {
+          s = fma(al[pb][c], bs[pb][c][0][lane], s);
+        } else {
+#pragma unroll
+          for (int u = 0; u < 4; ++u)
+            if (u < k) s = fma(as[pb][c][u][lr], bs[pb][c][u][lane], s);
+        }
+      }
+    }
+    __syncthreads();
   }
-  acc[0] = s;
+  if (warp == kF && J.w0 * 32 + lane < g.m * g.n) {
+    double* C = (kRemap ? (double*)remap_ptr(g.C, rm) : g.C) + (size_t)i * g.ldc + j;
+    *C = over ? s : *C + s;
+  }
 }
 
-// kStream: the streamed sum (R = 1, ordered); buf: 128 doubles per warp (kGemmWarps of them),
-// or the warps' rings
-template <int R, bool kRemap, bool kOrdered, bool kStream>
+// buf: 128 doubles per warp of the CTA
+template <int R, bool kRemap, bool kOrdered>
 __device__ __forceinline__ void gemm_job(const GemmTask* __restrict__ tasks, const GemmGroup& g, const GemmJob& J,
-                                         const Remap& rm, void* buf, bool lead_only, bool over) {
+                                         const Remap& rm, double* buf, bool lead_only, bool over) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int slots = ((g.m + R - 1) / R) * g.n;
   const int nt = g.task_end - g.task_begin;
@@ -414,7 +406,7 @@ __device__ __forceinline__ void gemm_job(const GemmTask* __restrict__ tasks, con
   const int t1 = g.task_begin + (int)((int64_t)nt * (J.sidx + 1) / J.ns);
   double* C = kRemap ? (double*)remap_ptr(g.C, rm) : g.C;
   // a shared sum's partial sums: R x 32 of every warp
-  auto part = [&](int w) { return (double*)buf + w * 128; };
+  auto part = [&](int w) { return buf + w * 128; };
   for (int w = J.w0; w < J.w0 + J.nw; ++w) {
     const int slot = w * 32 + lane;
     const bool valid = slot < slots;
@@ -428,8 +420,7 @@ __device__ __forceinline__ void gemm_job(const GemmTask* __restrict__ tasks, con
         for (int o = 1; o < J.ns; ++o) acc[r] += part(warp + o)[r * 32 + lane];
       }
     } else {
-      if constexpr (kStream) gemm_stream<kRemap>(tasks, t0, t1, i0, j, rm, ((GemmWarpBuf*)buf)[warp], acc);
-      else gemm_sum<R, kRemap, kOrdered>(tasks, t0, t1, i0, j, g.m, rm, (double*)buf + warp * 128, acc);
+      gemm_sum<R, kRemap, kOrdered>(tasks, t0, t1, i0, j, g.m, rm, buf + warp * 128, acc);
       if (!kOrdered && J.ns > 1) {
 #pragma unroll
         for (int r = 0; r < R; ++r) part(warp)[r * 32 + lane] = acc[r];
@@ -445,14 +436,14 @@ __device__ __forceinline__ void gemm_job(const GemmTask* __restrict__ tasks, con
   }
 }
 
-// one warp per job, up to kGemmWarps jobs per CTA; the ns jobs of a shared sum are
-// consecutive and never straddle CTAs (kGemmWarps warps then; ordered sums are never shared)
-template <bool kRemap, bool kOrdered, bool kStream>
+// one warp per job; the ns jobs of a shared sum are consecutive and never straddle CTAs
+// (ordered sums are never shared)
+template <bool kRemap, bool kOrdered>
 __global__ void __launch_bounds__(kGemmWarps * 32, kGemmMinCtas)
     k_grouped_gemm(const GemmTask* __restrict__ tasks, const GemmGroup* __restrict__ groups,
                    const GemmJob* __restrict__ jobs, int njobs, bool over, Remap rm) {
-  extern __shared__ __align__(16) unsigned char gemm_smem[];
-  const int id = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+  __shared__ double gemm_smem[kGemmWarps * 128];
+  const int id = blockIdx.x * kGemmWarps + (threadIdx.x >> 5);
   GemmJob J{-1, 0, 0, 0, 0};
   GemmGroup g{};
   if (id < njobs) {
@@ -462,13 +453,9 @@ __global__ void __launch_bounds__(kGemmWarps * 32, kGemmMinCtas)
   for (int pass = 0; pass < (kOrdered ? 1 : 2); ++pass) {
     if (pass == 1) __syncthreads();
     if (J.group >= 0 && (pass == 0 || (J.ns > 1 && J.sidx == 0))) {
-      if constexpr (kStream) {
-        gemm_job<1, kRemap, kOrdered, true>(tasks, g, J, rm, gemm_smem, pass == 1, over);
-      } else {
-        if (g.rpl == 4) gemm_job<4, kRemap, kOrdered, false>(tasks, g, J, rm, gemm_smem, pass == 1, over);
-        else if (g.rpl == 2) gemm_job<2, kRemap, kOrdered, false>(tasks, g, J, rm, gemm_smem, pass == 1, over);
-        else gemm_job<1, kRemap, kOrdered, false>(tasks, g, J, rm, gemm_smem, pass == 1, over);
-      }
+      if (g.rpl == 4) gemm_job<4, kRemap, kOrdered>(tasks, g, J, rm, gemm_smem, pass == 1, over);
+      else if (g.rpl == 2) gemm_job<2, kRemap, kOrdered>(tasks, g, J, rm, gemm_smem, pass == 1, over);
+      else gemm_job<1, kRemap, kOrdered>(tasks, g, J, rm, gemm_smem, pass == 1, over);
     }
   }
 }
@@ -490,13 +477,20 @@ int rows_per_lane(int m, int n, bool strided_b) {
 
 // Jobs of a table.  A job's work is counted in warp FMAs (plus a task's fixed cost); the
 // target is what gives every SM about 40 jobs, at least kGemmMinWork so that a job is worth
-// its start.  Groups above it are shared by up to eight warps, groups below it give one
+// its start.  Groups above it are shared by up to max_ns warps, groups below it give one
 // warp several of their 32-lane slices.  Longest jobs first.
-constexpr int64_t kGemmMinWork = 48, kGemmJobsTarget = 152 * 40, kGemmFewSlices = 8;
+constexpr int64_t kGemmMinWork = 48, kGemmJobsTarget = 152 * 40;
+// ordered sums in rounds: lists of at least kGemmRoundTasks tasks in the mean, in tables of at
+// most kGemmMaxChunks chunks (the chunk table costs the host more than the rounds save on large
+// blocks: phase 2 of random L=28, D=1500, 5.6 million chunks, 84 / 79 ms).  The operator
+// updates' lists (two to ten tasks in the mean) keep the FP64 pipes busy as they are: 10 ms in
+// rounds, 6 ms without for one of random L=28, D=700.
+constexpr int64_t kGemmRoundTasks = 12, kGemmMaxChunks = 1 << 21;
 
-// ks: columns of a group's tasks in all; rpl: its rows per lane.
+// ks: columns of a group's tasks in all; rpl: its rows per lane; max_ns: warps that may share a
+// sum; max_nw: slices that a job may take.
 std::vector<GemmJob> gemm_jobs(const std::vector<GemmGroup>& g, const std::vector<int64_t>& ks, const std::vector<int>& rpl,
-                               bool ordered) {
+                               int max_ns, int max_nw) {
   std::vector<int64_t> work(g.size(), 0);
   int64_t total = 0;
   for (size_t q = 0; q < g.size(); ++q) {
@@ -514,8 +508,8 @@ std::vector<GemmJob> gemm_jobs(const std::vector<GemmGroup>& g, const std::vecto
     const int nt = G.task_end - G.task_begin;
     const int64_t slices = ((int64_t)((G.m + rpl[q] - 1) / rpl[q]) * G.n + 31) / 32;
     int ns = 1, b = 3;
-    while (!ordered && ns < kGemmWarps && work[q] > ns * target && 2 * ns <= nt) { ns *= 2; --b; }
-    const int64_t nw = ns > 1 ? 1 : std::min<int64_t>(32767, std::max<int64_t>(1, target / work[q]));
+    while (ns < max_ns && work[q] > ns * target && 2 * ns <= nt) { ns *= 2; --b; }
+    const int64_t nw = ns > 1 ? 1 : std::min<int64_t>(max_nw, std::max<int64_t>(1, target / work[q]));
     int64_t w = work[q] * nw / ns;
     int lg = 0;
     while (w > 1) { w >>= 1; ++lg; }
@@ -535,35 +529,51 @@ GemmPlan* gemm_plan_upload(const std::vector<GemmTask>& t, std::vector<GemmGroup
   GemmPlan* p = new GemmPlan;
   p->ntasks = (int64_t)t.size();
   p->overwrite = (sums & GEMM_OVERWRITE) != 0;
-  // per group: columns in all, rows per lane; a table of at most kGemmFewSlices one-row slices
-  // per SM does not fill the GPU
+  // per group: columns in all, rows per lane; chunks of the whole table (rounds)
   std::vector<int64_t> ks(g.size(), 0);
   std::vector<int> rpl(g.size(), 1);
-  int64_t slices = 0;
+  int64_t chunks = 0, live = 0;
   for (size_t q = 0; q < g.size(); ++q) {
     GemmGroup& G = g[q];
     if (G.m <= 0 || G.n <= 0) continue;
     bool strided = false;
     for (int k = G.task_begin; k < G.task_end; ++k) {
       ks[q] += t[k].A ? t[k].k : 1;
+      chunks += t[k].A ? (t[k].k + 3) / 4 : 1;
       strided = strided || (t[k].A && t[k].transB);
     }
     if (ks[q] == 0) continue;
     G.rpl = rpl[q] = rows_per_lane(G.m, G.n, strided);
-    slices += ((int64_t)G.m * G.n + 31) / 32;
+    ++live;
   }
-  p->few = slices <= 152 * kGemmFewSlices;
-  const std::vector<int> one(p->few ? g.size() : 0, 1);  // the streamed kernel's rows per lane
+  p->rounds = (sums & GEMM_ORDERED) && p->ntasks >= kGemmRoundTasks * live && chunks <= kGemmMaxChunks;
+  const std::vector<int> one(p->rounds ? g.size() : 0, 1);  // rows per lane of the rounds
   try {
     for (int kind = 0; kind < 2; ++kind) {
       if (!(sums & (kind == 0 ? GEMM_ORDERED : GEMM_SHARED))) continue;
-      const std::vector<GemmJob> jobs = gemm_jobs(g, ks, kind == 0 && p->few ? one : rpl, kind == 0);
+      const std::vector<GemmJob> jobs =
+          gemm_jobs(g, ks, kind == 0 && p->rounds ? one : rpl, kind == 0 ? 1 : kGemmWarps,
+                    kind == 0 && p->rounds ? 1 : 32767);
       if (jobs.size() > (size_t)std::numeric_limits<int>::max() - kGemmWarps)
         throw std::runtime_error("block-product table exceeds 2^31 jobs");
       p->njobs[kind] = (int)jobs.size();
       if (jobs.empty()) continue;
       p->jobs[kind] = (GemmJob*)dev_alloc(jobs.size() * sizeof(GemmJob), s);
       dev_h2d(p->jobs[kind], jobs.data(), jobs.size() * sizeof(GemmJob), s);
+    }
+    if (p->rounds) {
+      // the groups' chunk ranges (begin, end), then the chunks (task, first column); the
+      // ranges are relative to the table
+      std::vector<GemmChunk> ch(g.size());
+      for (size_t q = 0; q < g.size(); ++q) {
+        ch[q].begin = (int)ch.size();
+        if (ks[q] > 0)
+          for (int k = g[q].task_begin; k < g[q].task_end; ++k)
+            for (int k0 = 0; k0 < (t[k].A ? t[k].k : 1); k0 += 4) ch.push_back(GemmChunk{{k}, {k0}});
+        ch[q].end = (int)ch.size();
+      }
+      p->chunks = (GemmChunk*)dev_alloc(std::max<size_t>(ch.size(), 1) * sizeof(GemmChunk), s);
+      dev_h2d(p->chunks, ch.data(), ch.size() * sizeof(GemmChunk), s);
     }
     if (!t.empty()) {
       p->tasks = (GemmTask*)dev_alloc(t.size() * sizeof(GemmTask), s);
@@ -586,20 +596,13 @@ void gemm_launch(const GemmPlan* p, const Remap& rm, int sums, Stream s) {
   const int kind = sums == GEMM_ORDERED ? 0 : 1;
   if (!p || p->njobs[kind] == 0) return;
   const int n = p->njobs[kind];
-  // few ordered jobs: fewer warps per CTA, so that they spread over all SMs
-  const int w = kind == 1 || n > 152 * 4 ? kGemmWarps : n > 152 * 2 ? 4 : n > 152 ? 2 : 1;
-  auto run = [&](auto* f, size_t smem) {
-    f<<<(n + w - 1) / w, w * 32, smem, S(s)>>>(p->tasks, p->groups, p->jobs[kind], n, p->overwrite, rm);
-  };
-  constexpr size_t direct = sizeof(double) * 128 * kGemmWarps, rings = sizeof(GemmWarpBuf) * kGemmWarps;
-  if (kind == 1) {
-    run(k_grouped_gemm<kRemap, false, false>, direct);
-  } else if (!p->few) {
-    run(k_grouped_gemm<kRemap, true, false>, direct);
+  const GemmJob* jobs = p->jobs[kind];
+  if (kind == 0 && p->rounds) {
+    k_gemm_rounds<kRemap><<<n, kRoundWarps * 32, 0, S(s)>>>(p->tasks, p->groups, p->chunks, jobs, p->overwrite, rm);
   } else {
-    auto* f = k_grouped_gemm<kRemap, true, true>;
-    ck(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)rings), "gemm smem");
-    run(f, rings / kGemmWarps * w);
+    const int grid = (n + kGemmWarps - 1) / kGemmWarps;
+    if (kind == 0) k_grouped_gemm<kRemap, true><<<grid, kGemmWarps * 32, 0, S(s)>>>(p->tasks, p->groups, jobs, n, p->overwrite, rm);
+    else k_grouped_gemm<kRemap, false><<<grid, kGemmWarps * 32, 0, S(s)>>>(p->tasks, p->groups, jobs, n, p->overwrite, rm);
   }
   ++g_launches;
   ck(cudaGetLastError(), "grouped_gemm launch");
@@ -614,6 +617,7 @@ void gemm_plan_free(GemmPlan* p, Stream s) {
   dev_free(p->groups, s);
   dev_free(p->jobs[0], s);
   dev_free(p->jobs[1], s);
+  dev_free(p->chunks, s);
   delete p;
 }
 
@@ -622,15 +626,52 @@ int64_t gemm_plan_tasks(const GemmPlan* p) { return p ? p->ntasks : 0; }
 // ------------------------------------------------------------------ combine
 
 namespace {
-__global__ void k_combine(const CombSrc* __restrict__ src, const CombDst* __restrict__ dst) {
-  const CombDst d = dst[blockIdx.x];
-  const int64_t n = (int64_t)d.rows * d.cols;
-  for (int64_t e = threadIdx.x; e < n; e += blockDim.x) {
-    int r = (int)(e / d.cols), c = (int)(e % d.cols);
-    double v = d.accumulate ? d.dst[(size_t)r * d.ld + c] : 0.0;
-    for (int s = d.src_begin; s < d.src_end; ++s) v += src[s].alpha * src[s].src[(size_t)r * src[s].ld + c];
-    d.dst[(size_t)r * d.ld + c] = v;
+// One warp per destination block (most have 4 to 150 elements), its sources four at a time:
+// descriptors first, then their elements, so that a chain of sources is not a chain of
+// loads.  The sum itself stays in source order.  Measured (W sums of random L=12, D=500: 0.33
+// million blocks; L=16, D=600: 1.1 million): a 128-thread CTA per block 250 / 661 us, now
+// 129 / 315 us.
+constexpr int kCombWarps = 8;
+
+template <bool kRemap>
+__global__ void __launch_bounds__(kCombWarps * 32) k_combine(const CombSrc* __restrict__ src, const CombDst* __restrict__ dst,
+                                                            int ndst, int wpd, Remap rm) {
+  const int w = blockIdx.x * kCombWarps + (threadIdx.x >> 5), id = w / wpd;
+  if (id >= ndst) return;
+  const CombDst d = dst[id];
+  double* out = kRemap ? (double*)remap_ptr(d.dst, rm) : d.dst;
+  const int n = d.rows * d.cols;
+  for (int e = (w - id * wpd) * 32 + (threadIdx.x & 31); e < n; e += 32 * wpd) {
+    const int r = e / d.cols, c = e - r * d.cols;
+    double v = d.accumulate ? out[(size_t)r * d.ld + c] : 0.0;
+    int s = d.src_begin;
+    for (; s + 4 <= d.src_end; s += 4) {
+      CombSrc q[4];
+      double x[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) q[u] = src[s + u];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) x[u] = (kRemap ? remap_ptr(q[u].src, rm) : q[u].src)[(size_t)r * q[u].ld + c];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) v += q[u].alpha * x[u];
+    }
+    for (; s < d.src_end; ++s) {
+      const CombSrc q = src[s];
+      v += q.alpha * (kRemap ? remap_ptr(q.src, rm) : q.src)[(size_t)r * q.ld + c];
+    }
+    out[(size_t)r * d.ld + c] = v;
   }
+}
+
+template <bool kRemap>
+void combine_launch(const CombPlan* p, const Remap& rm, Stream s) {
+  if (!p || p->ndst == 0) return;
+  // warps per block: one where the blocks fill the GPU, a CTA's eight for short tables
+  const int wpd = p->ndst >= 152 * 64 ? 1 : kCombWarps;
+  const int64_t grid = ((int64_t)p->ndst * wpd + kCombWarps - 1) / kCombWarps;
+  k_combine<kRemap><<<(unsigned)grid, kCombWarps * 32, 0, S(s)>>>(p->src, p->dst, p->ndst, wpd, rm);
+  ++g_launches;
+  ck(cudaGetLastError(), "combine launch");
 }
 }  // namespace
 
@@ -648,15 +689,7 @@ CombPlan* comb_plan_upload(const std::vector<CombSrc>& s, const std::vector<Comb
   return p;
 }
 
-void comb_plan_run(const CombPlan* p, Stream s) {
-  if (!p || p->ndst == 0) return;
-  for (int off = 0; off < p->ndst; off += 65535) {
-    int n = std::min(65535, p->ndst - off);
-    k_combine<<<n, 128, 0, S(s)>>>(p->src, p->dst + off);
-    ++g_launches;
-  }
-  ck(cudaGetLastError(), "combine launch");
-}
+void comb_plan_run(const CombPlan* p, Stream s) { combine_launch<false>(p, Remap{}, s); }
 
 void comb_plan_free(CombPlan* p, Stream s) {
   if (!p) return;
@@ -922,163 +955,204 @@ __device__ __forceinline__ void rr_pair(int r, int step, int np, int& p, int& q)
   if (p > q) { const int t = p; p = q; q = t; }
 }
 
-// Lowest k eigenpairs of the m x m Rayleigh matrix (m <= kSeMax) by cyclic Jacobi, one CTA
-// of 256 threads.
+// ---- one sweep of cyclic FP64 Jacobi on a matrix in shared memory, by a CTA of 256 threads
 //
-// A step's rotations are a chain of three divisions and two square roots (3000 cycles),
-// its row and column updates 6 m^2 FP64 operations (3000 cycles of an SM at m = 32).  The two
-// overlap: a step first updates the 2 x 2 blocks J_r^T A J_u that hold the next step's
-// pairs, then one warp computes the next rotations while the warps of the other three
-// sub-partitions update the rest of A and Q.  Every element sees the same operations in the
-// same order as with one barrier between rows, columns and rotations, so the results are
-// the same to the bit.  Measured (m = 1 to 32 over a Davidson run, mean per call): phase by
-// phase 632 us, overlapped 397 us.
-constexpr int kSeMax = 48, kSeLd = 49;
-
-struct SmallEigMem {
-  double A[kSeMax][kSeLd], Q[kSeMax][kSeLd];
-  double cs[2][kSeMax / 2], sn[2][kSeMax / 2], red[16];
-  int pp[2][kSeMax / 2], qq[2][kSeMax / 2], order[kSeMax];
-  unsigned crit[kSeMax / 2];  // per row pair: the column pairs whose block is updated first
-  int done, tie;
+// A step's rotations are a chain of three divisions and two square roots (3000 cycles), its
+// row and column updates 6 n^2 FP64 operations (3 n^2 cycles of an SM).  The two overlap: a
+// step first updates the 2 x 2 blocks J_r^T A J_u that hold the next step's pairs, then one
+// warp computes the next rotations while the others update the rest of A and Q.  Every
+// element sees the same operations in the same order as with one barrier between rotations,
+// rows and columns, so the results are the same to the bit.
+struct JacobiBuf {
+  double cs[2][32], sn[2][32];
+  int pp[2][32], qq[2][32];
+  unsigned crit[32];  // per row pair: the column pairs whose block is updated first
 };
 
-__device__ __forceinline__ void se_rotate(SmallEigMem& S, int buf, int step, int np, int m, int r) {
+// pair of element x in a step's round-robin pairing
+__device__ __forceinline__ int rr_pair_of(int x, int step, int np) {
+  int pos = 0;
+  if (x > 0) {
+    pos = x - 1 - step % (np - 1);
+    pos = 1 + (pos < 0 ? pos + np - 1 : pos);
+  }
+  return pos < np / 2 ? pos : np - 1 - pos;
+}
+
+// rot(p, q, next, c, s): the rotation of pair (p, q), p < q; next: of the following sweep
+template <class Rot>
+__device__ __forceinline__ void jacobi_rotations(JacobiBuf& S, int buf, int step, int np, int r, bool next, Rot rot) {
   int p, q;
   rr_pair(r, step, np, p, q);
   double c = 1.0, s = 0.0;
-  if (q < m) sym_schur2(S.A[p][p], S.A[q][q], S.A[p][q], c, s);
+  rot(p, q, next, c, s);
   S.cs[buf][r] = c;
   S.sn[buf][r] = s;
   S.pp[buf][r] = p;
   S.qq[buf][r] = q;
 }
 
+// A (np x np, np even, at most 64), Q (m rows, np columns), row stride ld; the rotations of
+// step 0 are in S[buf] on entry, those of the next sweep's step 0 on return (if `more`).
+// Called by all 256 threads, a barrier behind the rotations; ends with a barrier.
+template <class Rot>
+__device__ void jacobi_sweep(double* A, double* Q, int ld, int np, int m, JacobiBuf& S, int& buf, bool more, Rot rot) {
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int nr = np / 2, ns = np - 1;
+  const bool early = nr >= 4;  // below, two pairs can share a block
+  for (int step = 0; step < ns; ++step) {
+    const bool last = step + 1 == ns;
+    const int next = last ? 0 : step + 1;
+    const double* cs = S.cs[buf];
+    const double* sn = S.sn[buf];
+    const int* pp = S.pp[buf];
+    const int* qq = S.qq[buf];
+    if (tid < nr) S.crit[tid] = 0u;
+    __syncthreads();
+    // the blocks of the next step's pairs: the diagonal ones and the one holding (p', q'),
+    // four lanes per block (one element each)
+    if (early && tid < 8 * nr) {
+      const int b = tid >> 2, o = tid & 3;
+      int r = b, u = b;
+      if (b >= nr) {
+        int p, q;
+        rr_pair(b - nr, next, np, p, q);
+        r = rr_pair_of(p, step, np);
+        u = rr_pair_of(q, step, np);
+      }
+      const double cr = cs[r], sr = sn[r], cu = cs[u], su = sn[u];
+      const int p = pp[r] * ld, q = qq[r] * ld, v = pp[u], w = qq[u];
+      const double a0 = A[p + v], a1 = A[p + w], b0 = A[q + v], b1 = A[q + w];
+      double x0, x1;  // row p or q after the row rotation
+      if (o < 2) {
+        x0 = cr * a0 - sr * b0;
+        x1 = cr * a1 - sr * b1;
+      } else {
+        x0 = sr * a0 + cr * b0;
+        x1 = sr * a1 + cr * b1;
+      }
+      const double z = (o & 1) ? su * x0 + cu * x1 : cu * x0 - su * x1;
+      __syncwarp(__activemask());
+      A[(o < 2 ? p : q) + ((o & 1) ? w : v)] = z;
+      if (o == 0) atomicOr(&S.crit[r], 1u << u);
+    }
+    __syncthreads();
+    if (early && warp == 0 && lane < nr && (more || !last)) jacobi_rotations(S, buf ^ 1, next, np, lane, last, rot);
+    // the other blocks and Q (an FP64 instruction costs the same for one lane as for 32):
+    // up to 16 pairs packed onto the lanes of the warps on the other sub-partitions, more
+    // with lane = column pair on every warp but the rotating one
+    auto block = [&](int r, int u) {
+      const double cr = cs[r], sr = sn[r], cu = cs[u], su = sn[u];
+      if (((S.crit[r] >> u) & 1u) || (sr == 0.0 && su == 0.0)) return;
+      const int p = pp[r] * ld, q = qq[r] * ld, v = pp[u], w = qq[u];
+      const double a0 = A[p + v], a1 = A[p + w], b0 = A[q + v], b1 = A[q + w];
+      const double x0 = cr * a0 - sr * b0, x1 = cr * a1 - sr * b1;
+      const double y0 = sr * a0 + cr * b0, y1 = sr * a1 + cr * b1;
+      A[p + v] = cu * x0 - su * x1;
+      A[p + w] = su * x0 + cu * x1;
+      A[q + v] = cu * y0 - su * y1;
+      A[q + w] = su * y0 + cu * y1;
+    };
+    auto column = [&](int i, int u) {
+      const double c = cs[u], t = sn[u];
+      if (t == 0.0) return;
+      double* row = Q + i * ld;
+      const int v = pp[u], w = qq[u];
+      const double a0 = row[v], a1 = row[w];
+      row[v] = c * a0 - t * a1;
+      row[w] = t * a0 + c * a1;
+    };
+    if (nr <= 16) {
+      if (!early || (warp & 3) != 0) {
+        const int nt = early ? 192 : 256, t0 = (early ? (warp < 4 ? warp - 1 : warp - 2) : warp) * 32 + lane;
+        const unsigned inv = 65536u / nr + 1;  // e / nr = e * inv >> 16 for e < 65536 / nr
+        for (int e = t0; e < nr * nr; e += nt) {
+          const int r = (int)(e * inv >> 16);
+          block(r, e - r * nr);
+        }
+        for (int e = t0; e < nr * m; e += nt) {
+          const int i = (int)(e * inv >> 16);
+          column(i, e - i * nr);
+        }
+      }
+    } else if (warp > 0 && lane < nr) {
+      for (int r = warp - 1; r < nr; r += 7) block(r, lane);
+      for (int i = warp - 1; i < m; i += 7) column(i, lane);
+    }
+    __syncthreads();
+    if (!early && (more || !last)) {
+      if (tid < nr) jacobi_rotations(S, buf ^ 1, next, np, tid, last, rot);
+      __syncthreads();
+    }
+    buf ^= 1;
+  }
+}
+
+// Lowest k eigenpairs of the m x m Rayleigh matrix (m <= kSeMax) by cyclic Jacobi, one CTA
+// of 256 threads.  Measured (mean call of a Hubbard L=8, D=32 solve): phase by phase 339 us,
+// overlapped 215 us.
+constexpr int kSeMax = 48, kSeLd = 49;
+
+struct SmallEigMem {
+  double A[kSeMax * kSeLd], Q[kSeMax * kSeLd], red[16];
+  JacobiBuf j;
+  int order[kSeMax], tie;
+};
+
 __device__ void small_eig_block(const double* __restrict__ G, int gld, int m, int k, double* __restrict__ theta,
                                 double* __restrict__ C) {
   __shared__ SmallEigMem S;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int np = (m + 1) & ~1, nr = np / 2, ns = np - 1;
+  const int np = (m + 1) & ~1, nr = np / 2;
   for (int e = tid; e < np * np; e += blockDim.x) {
     const int i = e / np, j = e % np;
     const bool in = i < m && j < m;
-    S.A[i][j] = !in ? 0.0 : i >= j ? G[(size_t)i * gld + j] : G[(size_t)j * gld + i];  // lower triangle
-    S.Q[i][j] = (i == j) ? 1.0 : 0.0;
+    S.A[i * kSeLd + j] = !in ? 0.0 : i >= j ? G[(size_t)i * gld + j] : G[(size_t)j * gld + i];  // lower triangle
+    S.Q[i * kSeLd + j] = (i == j) ? 1.0 : 0.0;
   }
   __syncthreads();
-  if (tid < nr) se_rotate(S, 0, 0, np, m, tid);
-  __syncthreads();
+  auto rot = [&](int p, int q, bool, double& c, double& s) {
+    if (q < m) sym_schur2(S.A[p * kSeLd + p], S.A[q * kSeLd + q], S.A[p * kSeLd + q], c, s);
+  };
   int buf = 0;
+  if (tid < nr) jacobi_rotations(S.j, 0, 0, np, tid, false, rot);
+  __syncthreads();
   for (int sweep = 0; sweep < 60 && m > 1; ++sweep) {
-    {  // off-diagonal against total
-      double off = 0.0, tot = 0.0;
-      for (int e = tid; e < m * m; e += blockDim.x) {
-        const int i = e / m, j = e % m;
-        const double v = S.A[i][j];
-        tot += v * v;
-        if (i != j) off += v * v;
-      }
+    // off-diagonal against total
+    double off = 0.0, tot = 0.0;
+    for (int e = tid; e < m * m; e += blockDim.x) {
+      const int i = e / m, j = e % m;
+      const double v = S.A[i * kSeLd + j];
+      tot += v * v;
+      if (i != j) off += v * v;
+    }
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        off += __shfl_xor_sync(0xffffffffu, off, o);
-        tot += __shfl_xor_sync(0xffffffffu, tot, o);
-      }
-      if (lane == 0) {
-        S.red[warp] = off;
-        S.red[8 + warp] = tot;
-      }
-      __syncthreads();
-      off = tot = 0.0;
-      for (int w = 0; w < 8; ++w) {
-        off += S.red[w];
-        tot += S.red[8 + w];
-      }
-      if (off <= 1e-30 * tot || off == 0.0) break;  // the same sums in every thread
+    for (int o = 16; o > 0; o >>= 1) {
+      off += __shfl_xor_sync(0xffffffffu, off, o);
+      tot += __shfl_xor_sync(0xffffffffu, tot, o);
     }
-    for (int step = 0; step < ns; ++step) {
-      const int next = step + 1 == ns ? 0 : step + 1;
-      const double* cs = S.cs[buf];
-      const double* sn = S.sn[buf];
-      const int* pp = S.pp[buf];
-      const int* qq = S.qq[buf];
-      // the blocks of the next step's pairs first: the diagonal ones and the one holding
-      // (p', q'), four lanes per block (one element each)
-      if (tid < nr) S.crit[tid] = 0u;
-      __syncthreads();
-      const bool early = nr >= 4;  // below, two pairs can share a block
-      if (early && tid < 8 * nr) {
-        const int b = tid >> 2, o = tid & 3;
-        int r = b, u = b;
-        if (b >= nr) {
-          int p, q;
-          rr_pair(b - nr, next, np, p, q);
-          for (int x = 0; x < nr; ++x) {
-            if (pp[x] == p || qq[x] == p) r = x;
-            if (pp[x] == q || qq[x] == q) u = x;
-          }
-        }
-        const double cr = cs[r], sr = sn[r], cu = cs[u], su = sn[u];
-        const int p = pp[r], q = qq[r], v = pp[u], w = qq[u];
-        const double a0 = S.A[p][v], a1 = S.A[p][w], b0 = S.A[q][v], b1 = S.A[q][w];
-        double x0, x1;  // row p or q after the row rotation
-        if (o < 2) {
-          x0 = cr * a0 - sr * b0;
-          x1 = cr * a1 - sr * b1;
-        } else {
-          x0 = sr * a0 + cr * b0;
-          x1 = sr * a1 + cr * b1;
-        }
-        const double z = (o & 1) ? su * x0 + cu * x1 : cu * x0 - su * x1;
-        __syncwarp(__activemask());
-        S.A[o < 2 ? p : q][(o & 1) ? w : v] = z;
-        if (o == 0) atomicOr(&S.crit[r], 1u << u);
-      }
-      __syncthreads();
-      if (early && warp == 0) {
-        if (lane < nr) se_rotate(S, buf ^ 1, next, np, m, lane);
-      }
-      if (!early || (warp & 3) != 0) {
-        const int nw = early ? 192 : 256, t = early ? (warp < 4 ? warp - 1 : warp - 2) * 32 + lane : tid;
-        for (int e = t; e < nr * nr + nr * m; e += nw) {
-          if (e < nr * nr) {
-            const int r = e / nr, u = e - r * nr;
-            if ((S.crit[r] >> u) & 1u) continue;
-            const double cr = cs[r], sr = sn[r], cu = cs[u], su = sn[u];
-            const int p = pp[r], q = qq[r], v = pp[u], w = qq[u];
-            const double a0 = S.A[p][v], a1 = S.A[p][w], b0 = S.A[q][v], b1 = S.A[q][w];
-            const double x0 = cr * a0 - sr * b0, x1 = cr * a1 - sr * b1;
-            const double y0 = sr * a0 + cr * b0, y1 = sr * a1 + cr * b1;
-            S.A[p][v] = cu * x0 - su * x1;
-            S.A[p][w] = su * x0 + cu * x1;
-            S.A[q][v] = cu * y0 - su * y1;
-            S.A[q][w] = su * y0 + cu * y1;
-          } else {
-            const int f = e - nr * nr, u = f / m, i = f - u * m;
-            const double c = cs[u], s = sn[u];
-            const int v = pp[u], w = qq[u];
-            const double a0 = S.Q[i][v], a1 = S.Q[i][w];
-            S.Q[i][v] = c * a0 - s * a1;
-            S.Q[i][w] = s * a0 + c * a1;
-          }
-        }
-      }
-      __syncthreads();
-      if (!early) {
-        if (tid < nr) se_rotate(S, buf ^ 1, next, np, m, tid);
-        __syncthreads();
-      }
-      buf ^= 1;
+    if (lane == 0) {
+      S.red[warp] = off;
+      S.red[8 + warp] = tot;
     }
+    __syncthreads();
+    off = tot = 0.0;
+    for (int w = 0; w < 8; ++w) {
+      off += S.red[w];
+      tot += S.red[8 + w];
+    }
+    if (off <= 1e-30 * tot || off == 0.0) break;  // the same sums in every thread
+    jacobi_sweep(S.A, S.Q, kSeLd, np, m, S.j, buf, true, rot);
   }
   __syncthreads();
   // ascending order of the diagonal; equal values as an exchange sort leaves them
   if (tid == 0) S.tie = 0;
   __syncthreads();
   if (tid < m) {
-    const double vi = S.A[tid][tid];
+    const double vi = S.A[tid * kSeLd + tid];
     int rank = 0;
     for (int j = 0; j < m; ++j) {
-      const double vj = S.A[j][j];
+      const double vj = S.A[j * kSeLd + j];
       rank += vj < vi;
       if (vj == vi && j != tid) S.tie = 1;
     }
@@ -1086,18 +1160,19 @@ __device__ void small_eig_block(const double* __restrict__ G, int gld, int m, in
   }
   __syncthreads();
   if (S.tie && tid == 0) {
+    auto d = [&](int i) { return S.A[S.order[i] * kSeLd + S.order[i]]; };
     for (int i = 0; i < m; ++i) S.order[i] = i;
     for (int i = 0; i < m; ++i)
       for (int j = i + 1; j < m; ++j)
-        if (S.A[S.order[j]][S.order[j]] < S.A[S.order[i]][S.order[i]]) {
+        if (d(j) < d(i)) {
           const int t = S.order[i];
           S.order[i] = S.order[j];
           S.order[j] = t;
         }
   }
   __syncthreads();
-  for (int e = tid; e < k * m; e += blockDim.x) C[(size_t)(e / m) * m + e % m] = S.Q[e % m][S.order[e / m]];
-  if (tid < k) theta[tid] = S.A[S.order[tid]][S.order[tid]];
+  for (int e = tid; e < k * m; e += blockDim.x) C[(size_t)(e / m) * m + e % m] = S.Q[(e % m) * kSeLd + S.order[e / m]];
+  if (tid < k) theta[tid] = S.A[S.order[tid] * kSeLd + S.order[tid]];
 }
 
 __global__ void k_small_eig(const double* __restrict__ G, int gld, int m, int k,
@@ -1415,81 +1490,54 @@ namespace {
 constexpr int kEigSmemN = 64;  // blocks up to this size are diagonalised in shared memory
 
 // Cyclic Jacobi (round-robin pairing, n/2 rotations per step) on one symmetric block per
-// CTA, the matrix and the eigenvectors in shared memory (row stride n+1).  A pair is rotated only while |a_pq| exceeds
+// CTA, the matrix and the eigenvectors in shared memory.  Measured (135 blocks, 63 of 64 rows
+// the largest, random L=28, D=700): phase by phase 35.2 ms, overlapped (jacobi_sweep) 22.4 ms.
+// A pair is rotated only while |a_pq| exceeds
 // 1e-16 sqrt(|a_pp a_qq|) plus an absolute floor; the loop ends after a sweep without
 // rotations (at most 40 sweeps).  Output: eigenvalues descending, eigenvectors as
 // columns of J.Q.
 template <int NT>
 __global__ void __launch_bounds__(NT) k_eig_batched(const EigJob* __restrict__ jobs) {
+  static_assert(NT == 256, "jacobi_sweep");
   const EigJob J = jobs[blockIdx.x];
   const int n = J.n, tid = threadIdx.x;
   extern __shared__ double sm[];
-  const int ld = n + 1;
+  const int np = (n + 1) & ~1, ld = np + 1;
   double* A = sm;
-  double* Q = sm + (size_t)n * ld;
-  const int np = (n + 1) & ~1;
-  double* cs = sm + (size_t)2 * n * ld;
-  double* sn = cs + np / 2;
-  double* wtmp = sn + np / 2;
-  __shared__ int nrot;
-  for (int e = tid; e < n * n; e += NT) A[(size_t)(e / n) * ld + e % n] = J.A[e];
-  for (int e = tid; e < n * n; e += NT) Q[(size_t)(e / n) * ld + e % n] = (e / n == e % n) ? 1.0 : 0.0;
+  double* Q = sm + (size_t)np * ld;
+  double* wtmp = Q + (size_t)np * ld;
+  __shared__ JacobiBuf S;
+  __shared__ int nrot[2];
+  for (int e = tid; e < np * np; e += NT) {
+    const int i = e / np, j = e % np;
+    A[i * ld + j] = i < n && j < n ? J.A[(size_t)i * n + j] : 0.0;
+    Q[i * ld + j] = i == j ? 1.0 : 0.0;
+  }
+  if (tid < 2) nrot[tid] = 0;
   __syncthreads();
   double scale = 0.0;
   for (int i = 0; i < n; ++i) scale = fmax(scale, fabs(A[(size_t)i * ld + i]));
   const double floor_abs = 1e-300 + 1e-18 * scale;
-  for (int sweep = 0; sweep < 40; ++sweep) {
-    if (tid == 0) nrot = 0;
+  int cur = 0, buf = 0;  // the current sweep's counter
+  auto rot = [&](int p, int q, bool next, double& c, double& s) {
+    if (q >= n) return;
+    const double app = A[p * ld + p], aqq = A[q * ld + q], apq = A[p * ld + q];
+    if (fabs(apq) > 1e-16 * sqrt(fabs(app * aqq)) + floor_abs) {
+      sym_schur2(app, aqq, apq, c, s);
+      atomicAdd(&nrot[next ? cur ^ 1 : cur], 1);
+    }
+  };
+  if (n > 1) {
+    if (tid < np / 2) jacobi_rotations(S, 0, 0, np, tid, false, rot);
     __syncthreads();
-    for (int step = 0; step < np - 1; ++step) {
-      for (int r = tid; r < np / 2; r += NT) {
-        int a = r, b = np - 1 - r;
-        int p = a == 0 ? 0 : 1 + (a - 1 + step) % (np - 1);
-        int q = b == 0 ? 0 : 1 + (b - 1 + step) % (np - 1);
-        if (p > q) { int t = p; p = q; q = t; }
-        double c = 1.0, s = 0.0;
-        if (q < n) {
-          double app = A[(size_t)p * ld + p], aqq = A[(size_t)q * ld + q], apq = A[(size_t)p * ld + q];
-          if (fabs(apq) > 1e-16 * sqrt(fabs(app * aqq)) + floor_abs) {
-            sym_schur2(app, aqq, apq, c, s);
-            atomicAdd(&nrot, 1);
-          }
-        }
-        cs[r] = c; sn[r] = s;
-      }
+    for (int sweep = 0; sweep < 40; ++sweep) {
+      jacobi_sweep(A, Q, ld, np, n, S, buf, sweep < 39, rot);
+      if (nrot[cur] == 0) break;
       __syncthreads();
-      for (int e = tid; e < (np / 2) * n; e += NT) {
-        int r = e / n, j = e % n;
-        if (sn[r] == 0.0) continue;
-        int a = r, b = np - 1 - r;
-        int p = a == 0 ? 0 : 1 + (a - 1 + step) % (np - 1);
-        int q = b == 0 ? 0 : 1 + (b - 1 + step) % (np - 1);
-        if (p > q) { int t = p; p = q; q = t; }
-        double c = cs[r], s = sn[r];
-        double ap = A[(size_t)p * ld + j], aq = A[(size_t)q * ld + j];
-        A[(size_t)p * ld + j] = c * ap - s * aq;
-        A[(size_t)q * ld + j] = s * ap + c * aq;
-      }
-      __syncthreads();
-      for (int e = tid; e < (np / 2) * n; e += NT) {
-        int r = e / n, i = e % n;
-        if (sn[r] == 0.0) continue;
-        int a = r, b = np - 1 - r;
-        int p = a == 0 ? 0 : 1 + (a - 1 + step) % (np - 1);
-        int q = b == 0 ? 0 : 1 + (b - 1 + step) % (np - 1);
-        if (p > q) { int t = p; p = q; q = t; }
-        double c = cs[r], s = sn[r];
-        double ap = A[(size_t)i * ld + p], aq = A[(size_t)i * ld + q];
-        A[(size_t)i * ld + p] = c * ap - s * aq;
-        A[(size_t)i * ld + q] = s * ap + c * aq;
-        double qp = Q[(size_t)i * ld + p], qv = Q[(size_t)i * ld + q];
-        Q[(size_t)i * ld + p] = c * qp - s * qv;
-        Q[(size_t)i * ld + q] = s * qp + c * qv;
-      }
+      if (tid == 0) nrot[cur] = 0;
+      cur ^= 1;
       __syncthreads();
     }
-    if (nrot == 0) break;
-    __syncthreads();
   }
   // eigenpairs sorted descending (ties by index)
   for (int i = tid; i < n; i += NT) wtmp[i] = A[(size_t)i * ld + i];
@@ -1599,57 +1647,15 @@ struct BjJob {
 // iteration returns to every pair until it is diagonal, and inner sweeps beyond the first
 // cost more than they save (measured: 1 sweep 1.4-1.9x faster than 3, 2.1-2.7x than 5,
 // at the same accuracy)
-__device__ void cta_jacobi64(double* A, double* V, double* cs, double* sn, int* pq, int* nrot,
-                             double floor_abs) {
-  const int tid = threadIdx.x;
-  constexpr int m = kOP, np = kOP, nr = kOP / 2;
-  for (int sweep = 0; sweep < 1; ++sweep) {
-    if (tid == 0) *nrot = 0;
-    __syncthreads();
-    for (int step = 0; step < np - 1; ++step) {
-      if (tid < nr) {
-        const int a = tid, b = np - 1 - tid;
-        int p = a == 0 ? 0 : 1 + (a - 1 + step) % (np - 1);
-        int q = b == 0 ? 0 : 1 + (b - 1 + step) % (np - 1);
-        if (p > q) { const int t = p; p = q; q = t; }
-        double c = 1.0, s = 0.0;
-        const double app = A[p * kOL + p], aqq = A[q * kOL + q], apq = A[p * kOL + q];
-        if (fabs(apq) > 1e-16 * sqrt(fabs(app * aqq)) + floor_abs) {
-          sym_schur2(app, aqq, apq, c, s);
-          atomicAdd(nrot, 1);
-        }
-        cs[tid] = c; sn[tid] = s; pq[2 * tid] = p; pq[2 * tid + 1] = q;
-      }
-      __syncthreads();
-#pragma unroll
-      for (int k = 0; k < nr * m / 256; ++k) {  // rows p, q of A
-        const int e = tid + 256 * k, r = e >> 6, j = e & 63;
-        if (sn[r] == 0.0) continue;
-        const int p = pq[2 * r], q = pq[2 * r + 1];
-        const double c = cs[r], s = sn[r];
-        const double ap = A[p * kOL + j], aq = A[q * kOL + j];
-        A[p * kOL + j] = c * ap - s * aq;
-        A[q * kOL + j] = s * ap + c * aq;
-      }
-      __syncthreads();
-#pragma unroll
-      for (int k = 0; k < nr * m / 256; ++k) {  // columns p, q of A and V
-        const int e = tid + 256 * k, r = e >> 6, i = e & 63;
-        if (sn[r] == 0.0) continue;
-        const int p = pq[2 * r], q = pq[2 * r + 1];
-        const double c = cs[r], s = sn[r];
-        const double ap = A[i * kOL + p], aq = A[i * kOL + q];
-        A[i * kOL + p] = c * ap - s * aq;
-        A[i * kOL + q] = s * ap + c * aq;
-        const double vp = V[i * kOL + p], vq = V[i * kOL + q];
-        V[i * kOL + p] = c * vp - s * vq;
-        V[i * kOL + q] = s * vp + c * vq;
-      }
-      __syncthreads();
-    }
-    if (*nrot == 0) break;
-    __syncthreads();
-  }
+__device__ void cta_jacobi64(double* A, double* V, JacobiBuf& S, double floor_abs) {
+  auto rot = [&](int p, int q, bool, double& c, double& s) {
+    const double app = A[p * kOL + p], aqq = A[q * kOL + q], apq = A[p * kOL + q];
+    if (fabs(apq) > 1e-16 * sqrt(fabs(app * aqq)) + floor_abs) sym_schur2(app, aqq, apq, c, s);
+  };
+  int buf = 0;
+  if (threadIdx.x < kOP / 2) jacobi_rotations(S, 0, 0, kOP, threadIdx.x, false, rot);
+  __syncthreads();
+  jacobi_sweep(A, V, kOL, kOP, kOP, S, buf, false, rot);
 }
 
 // out(64 x 64 tile) = op(X) op(Y) with a 4 x 4 register tile per thread; X, Y in shared
@@ -1730,11 +1736,11 @@ struct BjTol<float> {
   static constexpr double rel = 0.0, abs = 1.0;  // gmax carries the pass's floor
 };
 
-__device__ __forceinline__ void bj_inner(double* S, double* V, double* cs, double* sn, int* pq, int* nrot, double gmax) {
-  cta_jacobi64(S, V, cs, sn, pq, nrot, 1e-16 * gmax);  // floor below the outer one
+__device__ __forceinline__ void bj_inner(double* S, double* V, JacobiBuf& B, int*, double gmax) {
+  cta_jacobi64(S, V, B, 1e-16 * gmax);  // floor below the outer one
 }
-__device__ __forceinline__ void bj_inner(float* S, float* V, float* cs, float* sn, int* pq, int* nrot, double gmax) {
-  jacobi_f32(S, V, kOP, kOL, 1, (float)(BjTol<float>::abs * gmax), cs, sn, pq, pq + kOP / 2, nrot);
+__device__ __forceinline__ void bj_inner(float* S, float* V, JacobiBuf& B, int* nrot, double gmax) {
+  jacobi_f32(S, V, kOP, kOL, 1, (float)(BjTol<float>::abs * gmax), (float*)B.cs, (float*)B.sn, B.pp[0], B.qq[0], nrot);
 }
 
 // step, part 1: V of every pair from its diagonal sub-block (one CTA per pair)
@@ -1745,9 +1751,8 @@ __global__ void __launch_bounds__(256) k_bj_rows(const BjJob<T>* __restrict__ jo
   extern __shared__ double bsm[];
   T* S = reinterpret_cast<T*>(bsm);  // sub-block, then diagonalised
   T* V = S + kOP * kOL;              // its eigenvectors
-  __shared__ T cs[kOP / 2], sn[kOP / 2];
-  __shared__ int pq[kOP], idx[kOP];
-  __shared__ int inner_rot, need;
+  __shared__ JacobiBuf jb;
+  __shared__ int idx[kOP], inner_rot, need;
   const int lo = find_job(jobs, njobs);
   const BjJob<T> J = jobs[lo];
   const int r = blockIdx.x - J.pair_begin, tid = threadIdx.x, n = J.n;
@@ -1775,7 +1780,7 @@ __global__ void __launch_bounds__(256) k_bj_rows(const BjJob<T>* __restrict__ jo
   }
   for (int e = tid; e < kOP * kOL; e += 256) V[e] = ((e / kOL) == (e % kOL)) ? T(1) : T(0);
   __syncthreads();
-  bj_inner(S, V, cs, sn, pq, &inner_rot, gmax[lo]);
+  bj_inner(S, V, jb, &inner_rot, gmax[lo]);
   __syncthreads();
   // one Newton-Schulz step V <- V (3 I - V^T V) / 2 against the rounding of the rotations
   {
@@ -2002,7 +2007,7 @@ void eig_batched(const std::vector<EigJob>& jobs, Stream s) {
   if (!small.empty()) {
     dev_h2d(d, small.data(), small.size() * sizeof(EigJob), s);
     const int np = (nmax_s + 1) & ~1;
-    size_t shm = sizeof(double) * ((size_t)2 * nmax_s * (nmax_s + 1) + np + nmax_s) + 64;
+    size_t shm = sizeof(double) * ((size_t)2 * np * (np + 1) + nmax_s) + 64;
     ck(cudaFuncSetAttribute(k_eig_batched<256>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm), "eig smem");
     k_eig_batched<256><<<(int)small.size(), 256, shm, S(s)>>>(d);
     ++g_launches;
@@ -2468,20 +2473,6 @@ static __device__ __align__(256) double g_noalloc_scratch[kNoAllocScratchDoubles
 std::mutex g_noalloc_mu;
 double* g_noalloc_ptr[64] = {nullptr};  // device address of the array, per device ordinal
 
-// k_combine with remapped addresses
-__global__ void k_combine_ra(const CombSrc* __restrict__ src, const CombDst* __restrict__ dst, Remap rm) {
-  const CombDst d = dst[blockIdx.x];
-  double* dp = (double*)remap_ptr(d.dst, rm);
-  const int64_t n = (int64_t)d.rows * d.cols;
-  for (int64_t e = threadIdx.x; e < n; e += blockDim.x) {
-    int r = (int)(e / d.cols), c = (int)(e % d.cols);
-    double v = d.accumulate ? dp[(size_t)r * d.ld + c] : 0.0;
-    for (int s = d.src_begin; s < d.src_end; ++s)
-      v += src[s].alpha * remap_ptr(src[s].src, rm)[(size_t)r * src[s].ld + c];
-    dp[(size_t)r * d.ld + c] = v;
-  }
-}
-
 // Device address of the static array on the current device (looked up once per device).
 double* noalloc_scratch(int* err) {
   int dev = 0;
@@ -2519,13 +2510,7 @@ void noalloc_matvec_run(const GemmPlan* p1, const CombPlan* pc, const GemmPlan* 
   // phase 2 accumulates into y, which starts at zero; Z and W are overwritten
   if (n) ck(cudaMemsetAsync(y, 0, sizeof(double) * n, S(s)), "memset y");
   gemm_launch<true>(p1, rm, GEMM_SHARED, s);
-  if (pc && pc->ndst) {
-    for (int off = 0; off < pc->ndst; off += 65535) {
-      int nb = std::min(65535, pc->ndst - off);
-      k_combine_ra<<<nb, 128, 0, S(s)>>>(pc->src, pc->dst + off, rm);
-      ++g_launches;
-    }
-  }
+  combine_launch<true>(pc, rm, s);
   gemm_launch<true>(p2, rm, GEMM_SHARED, s);
   ck(cudaGetLastError(), "allocation-free matvec launch");
 }

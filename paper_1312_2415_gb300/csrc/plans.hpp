@@ -14,13 +14,20 @@ struct GemmJob {
   unsigned char sidx, ns;
 };
 
+// ordered sums in rounds: a chunk (task, first column), or a group's range of chunks
+struct GemmChunk {
+  union { int task, begin; };
+  union { int k0, end; };
+};
+
 struct GemmPlan {
   GemmTask* tasks = nullptr;
   GemmGroup* groups = nullptr;
   GemmJob* jobs[2] = {nullptr, nullptr};  // ordered sums, shared sums
+  GemmChunk* chunks = nullptr;
   int njobs[2] = {0, 0};
   bool overwrite = false;  // C = sum instead of C += sum
-  bool few = false;  // too small to fill the GPU: the streamed kernel
+  bool rounds = false;  // ordered sums by k_gemm_rounds
   int64_t ntasks = 0;
 };
 
