@@ -324,19 +324,16 @@ def matvec_kernel_rates(delta):
     return out
 
 
-# DRAM bytes per launch (dram__bytes_read.sum + dram__bytes_write.sum) of the mixed
-# matvec's main kernel from one ncu capture (a smaller case scaled to a full launch by the
-# units processed, as the profile summary states), keyed by the workload and the SHA-256
-# prefix of the kernel source it was taken with: a changed kernel reports traffic null.
-# DRAM bytes per launch of k_tc_matvec (dram__bytes_read.sum + dram__bytes_write.sum, one
-# ncu pass, every launch of the timed steps of the default run), keyed by workload and
-# the kernel source it was measured on (a changed kernel reports null):
+# DRAM bytes per matvec of k_tc_matvec (dram__bytes_read.sum + dram__bytes_write.sum, one
+# ncu pass, every launch of the timed steps of the default run, the launches of a matvec's
+# tile classes added up), keyed by workload and the kernel source it was measured on (a
+# changed kernel reports null):
 #   ncu --metrics dram__bytes_read.sum,dram__bytes_write.sum --clock-control none --nvtx
-#       --nvtx-include "steps/" -k regex:k_tc_matvec -c 48 --csv
+#       --nvtx-include "steps/" -k regex:k_tc_matvec -c 150 --csv
 #       python bench.py --no-fp64 --no-e2e --no-cpu-baseline --no-batch
 NCU_TRAFFIC = {
-    (("random28", 2500), "f73a6011045fa39d"): {
-        "bytes": 4.06e10, "how": "mean over the 48 launches of the timed steps (3.39e10 .. 4.55e10), ncu one pass"},
+    (("random28", 2500), "02bac149931afcda"): {
+        "bytes": 3.35e10, "how": "mean over the 48 matvecs of the timed steps (120 launches), ncu one pass"},
 }
 
 

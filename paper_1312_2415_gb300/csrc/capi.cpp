@@ -661,15 +661,15 @@ int dmrg_batch_run(dmrg_batch* b, const double* const* x, double* const* y, uint
       if (b->ctx[i]->eng->tc_serial(b->site[i]) != b->serial[i])
         throw std::invalid_argument("a context of the batch changed its tables since the batch was made");
     cudaStream_t s = stream ? (cudaStream_t)stream : cudaStreamLegacy;
-    for (size_t i = 0; x && i < b->ctx.size(); ++i)
-      if (x[i] && x[i] != b->x[i])
-        if (cudaMemcpyAsync(b->x[i], x[i], sizeof(double) * b->n[i], cudaMemcpyDeviceToDevice, s) != cudaSuccess)
-          throw std::runtime_error("cuda batch input copy");
+    // one launch per 64 instances each way, not one copy call per instance
+    std::vector<dmrg::CopyJob> in, out;
+    for (size_t i = 0; i < b->ctx.size(); ++i) {
+      if (x && x[i] && x[i] != b->x[i]) in.push_back({b->x[i], x[i], b->n[i]});
+      if (y && y[i] && y[i] != b->y[i]) out.push_back({y[i], b->y[i], b->n[i]});
+    }
+    dmrg::copy_batched(in, (dmrg::Stream)s);
     dmrg::tc_graph_launch(b->graph, (dmrg::Stream)s);
-    for (size_t i = 0; y && i < b->ctx.size(); ++i)
-      if (y[i] && y[i] != b->y[i])
-        if (cudaMemcpyAsync(y[i], b->y[i], sizeof(double) * b->n[i], cudaMemcpyDeviceToDevice, s) != cudaSuccess)
-          throw std::runtime_error("cuda batch output copy");
+    dmrg::copy_batched(out, (dmrg::Stream)s);
     return DMRG_OK;
   });
 }

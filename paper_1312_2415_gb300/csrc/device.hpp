@@ -34,6 +34,14 @@ void stream_destroy(Stream s);
 void stream_wait(Stream s, void* ev);  // work queued on s after this waits for ev
 void event_sync(void* ev);
 
+// ---- copies of doubles within the device, their table passed with the launch ----
+struct CopyJob {
+  double* dst;
+  const double* src;
+  int64_t n;
+};
+void copy_batched(const std::vector<CopyJob>& jobs, Stream s);
+
 // ---- grouped GEMM: C_g = C_g + sum_t alpha_t op(A_t) op(B_t), row-major blocks;
 // A == nullptr means op(A) = identity (C_g += alpha op(B)) ----
 struct GemmTask {
