@@ -2092,11 +2092,26 @@ double Engine::truncate(int i, int dir, int D, const double* x, bool refined) {
     g.woff = wsz; wsz += g.n;
     g.aoff = asz; asz += (int64_t)g.R * g.C;  // room for U (R x r) or V (r x C)
   }
-  double* M = (double*)dev_alloc(sizeof(double) * std::max<int64_t>(msz, 1), stream_);
-  double* Gm = (double*)dev_alloc(sizeof(double) * std::max<int64_t>(gsz, 1), stream_);
-  double* Q = (double*)dev_alloc(sizeof(double) * std::max<int64_t>(gsz, 1), stream_);
-  double* W = (double*)dev_alloc(sizeof(double) * std::max<int64_t>(wsz, 1), stream_);
-  double* Aux = (double*)dev_alloc(sizeof(double) * std::max<int64_t>(asz, 1), stream_);
+  // released on every way out, a failed allocation's too
+  struct Scratch {
+    Stream s;
+    std::vector<double*> p;
+    double* get(int64_t n) {
+      p.push_back(nullptr);
+      p.back() = (double*)dev_alloc(sizeof(double) * std::max<int64_t>(n, 1), s);
+      return p.back();
+    }
+    ~Scratch() {
+      for (double* q : p) {
+        try { dev_free(q, s); } catch (...) {}
+      }
+    }
+  } scratch{stream_, {}};
+  double* M = scratch.get(msz);
+  double* Gm = scratch.get(gsz);
+  double* Q = scratch.get(gsz);
+  double* W = scratch.get(wsz);
+  double* Aux = scratch.get(asz);
   dev_zero(M, sizeof(double) * std::max<int64_t>(msz, 1), stream_);
   dev_zero(Gm, sizeof(double) * std::max<int64_t>(gsz, 1), stream_);
   dev_zero(Aux, sizeof(double) * std::max<int64_t>(asz, 1), stream_);
@@ -2237,11 +2252,6 @@ double Engine::truncate(int i, int dir, int D, const double* x, bool refined) {
     }
   }
   scatter_batched(sj, stream_);
-  dev_free(M, stream_);
-  dev_free(Gm, stream_);
-  dev_free(Q, stream_);
-  dev_free(W, stream_);
-  dev_free(Aux, stream_);
   st_.last_w_disc = w_disc;
   st_.max_w_disc = std::max(st_.max_w_disc, w_disc);
   st_.t_trunc_ms += tm.ms();

@@ -2206,12 +2206,22 @@ void eig_refined(const std::vector<EigJob>& jobs, const std::vector<EigSource>& 
     toff.push_back(toff.back() + (int64_t)src[k].inner * jobs[k].n);
     nmax = std::max(nmax, jobs[k].n);
   }
-  if (sizeof(double) * 2 * (size_t)nmax > 200 * 1024) return eig_batched(jobs, s);
+  // Small blocks: the passes' launches and tables cost some 0.7 ms whatever the sizes.  Whole
+  // call, Hubbard chains, Jacobi / refined: largest block 11 rows 0.59 / 0.84 ms, 20 rows 0.89 /
+  // 1.02, 26 rows 1.37 / 1.16, 49 rows 4.5 / 2.1.
+  constexpr int kRefineRows = 23;
+  if (nmax < kRefineRows || sizeof(double) * 2 * (size_t)nmax > 200 * 1024) return eig_batched(jobs, s);
   const int64_t tot = off.back();
   const int nj = (int)jobs.size();
   // X, X2, S, R, T (FP64), A32, Q32 (FP32)
   const int64_t ttot = toff.back();
-  double* buf = (double*)dev_alloc(sizeof(double) * (size_t)(tot * 5 + ttot), s);
+  double* buf = nullptr;
+  try {
+    buf = (double*)dev_alloc(sizeof(double) * (size_t)(tot * 5 + ttot), s);
+  } catch (const std::exception&) {  // no room (the cap, or the device): the solver in place
+    cudaGetLastError();
+    return eig_batched(jobs, s);
+  }
   double *X = buf, *X2 = X + tot, *Sm = X2 + tot, *R = Sm + tot, *T = R + tot;
   float *A32 = (float*)(T + ttot), *Q32 = A32 + tot;
   ReJob* d = nullptr;

@@ -66,3 +66,34 @@ def test_truncation_by_refined_eigenvectors(Context, L, D0, kind, direction):  #
     if 0 <= nxt <= L - 2:
         v = ctx.tt_to_x(nxt)
         assert abs(ctx.energy(nxt, v) - e) <= 1e-10 * max(1.0, abs(e))
+
+
+def test_truncation_without_room_for_the_refined_solver(Context):  # noqa: F811
+    """Under a device-memory cap that leaves room for the decomposition's own matrices only,
+    the eigenproblems are solved in place and the result is the same state (1e-10)."""
+    from paper_1312_2415_gb300 import binding
+    L, D = 12, 400
+    site = L // 2 - 1
+    ctx = Context(L, [0] * L, L, 0, 0)
+    ctx.set_integrals(*hubbard_chain(L, 1.0, 4.0))
+    ctx.set_schedule([D], [1e-8], [1], [0.0])
+    ctx.init_mps(3)
+    ctx.canonicalize(site)
+    x = vector(ctx, site, "falling", 5)
+    w = ctx.truncate(site, 1, D // 2, x)
+    y = ctx.tt_to_x(site)
+    used = binding.device_memory_in_use()
+    n = ctx.layout(site)[0]
+    try:
+        for room in (1, 2, 3, 4, 6, 8, 12, 16, 24, 32, 64):  # multiples of the vector's bytes
+            binding.set_device_memory_cap(used + room * 8 * n)
+            try:
+                w2 = ctx.truncate(site, 1, D // 2, x)
+            except binding.DMRGError as e:
+                assert e.code == binding.ENOMEM
+                continue
+            assert abs(w2 - w) <= 1e-12
+            binding.set_device_memory_cap(0)
+            assert np.abs(ctx.tt_to_x(site) - y).max() <= 1e-10
+    finally:
+        binding.set_device_memory_cap(0)
