@@ -1066,7 +1066,7 @@ __device__ void jacobi_sweep(double* A, double* Q, int ld, int np, int m, Jacobi
         x1 = sr * a1 + cr * b1;
       }
       const double z = (o & 1) ? su * x0 + cu * x1 : cu * x0 - su * x1;
-      __syncwarp(__activemask());
+      __syncwarp(0xfu << (lane & ~3));  // the block's four lanes have all read before one writes
       A[(o < 2 ? p : q) + ((o & 1) ? w : v)] = z;
       if (o == 0) atomicOr(&S.crit[r], 1u << u);
     }
