@@ -317,6 +317,13 @@ int dmrg_set_device_memory_cap(size_t bytes);
  * cleared when it is read, and with the hook off the next call computes normally.  No
  * fault, trap or endless wait is involved.  Library-wide. */
 int dmrg_test_tc_timeout(int on);
+
+/* Test hook: the Rayleigh-Ritz eigensolver of Davidson on its own.  The k lowest eigenpairs
+ * of the symmetric m x m matrix G (row-major, the lower triangle is read; m <= 48): theta
+ * (k, ascending) and C (k x m, one eigenvector per row).  Host pointers.  A NaN in
+ * the matrix gives NaN, and no error. */
+int dmrg_test_small_eig(const double* G, int m, int k, double* theta, double* C);
+
 int dmrg_device_memory_in_use(size_t* bytes);
 
 int dmrg_stats(dmrg_ctx* ctx, dmrg_stats_t* out);

@@ -89,6 +89,7 @@ _SIGS = {
     "dmrg_batch_last_error": (ctypes.c_char_p, [_P]),
     "dmrg_batch_destroy": (None, [_P]),
     "dmrg_test_tc_timeout": (ctypes.c_int, [ctypes.c_int]),
+    "dmrg_test_small_eig": (ctypes.c_int, [_D, ctypes.c_int, ctypes.c_int, _D, _D]),
     "dmrg_set_device_memory_cap": (ctypes.c_int, [ctypes.c_size_t]),
     "dmrg_device_memory_in_use": (ctypes.c_int, [ctypes.POINTER(ctypes.c_size_t)]),
     "dmrg_stats": (ctypes.c_int, [_P, ctypes.POINTER(Stats)]),
@@ -330,6 +331,17 @@ def test_tc_timeout(on, path=None):
     rc = load(path).dmrg_test_tc_timeout(int(on))
     if rc != OK:
         raise DMRGError(rc, "dmrg_test_tc_timeout")
+
+
+def test_small_eig(G, k, path=None):
+    """Test hook: the k lowest eigenpairs of G by Davidson's Rayleigh-Ritz solver."""
+    G = np.ascontiguousarray(G, dtype=np.float64)
+    m = len(G)
+    theta, C = np.zeros(k), np.zeros((k, m))
+    rc = load(path).dmrg_test_small_eig(_dptr(G), m, int(k), _dptr(theta), _dptr(C))
+    if rc != OK:
+        raise DMRGError(rc, "dmrg_test_small_eig")
+    return theta, C
 
 
 def device_memory_in_use(path=None):

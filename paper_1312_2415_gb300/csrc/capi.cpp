@@ -494,6 +494,22 @@ int dmrg_stats(dmrg_ctx* c, dmrg_stats_t* out) {
   });
 }
 
+int dmrg_test_small_eig(const double* G, int m, int k, double* theta, double* C) {
+  if (!G || !theta || !C || m < 1 || m > 48 || k < 1 || k > m) return DMRG_EINVAL;
+  std::string err;
+  return guard_err(err, [&] {
+    dmrg::Stream s = (dmrg::Stream)cudaStreamLegacy;
+    DevBuf b((int64_t)m * m + m + (int64_t)k * m, s);
+    double *dg = b.p, *dt = dg + m * m, *dc = dt + m;
+    dmrg::dev_h2d(dg, G, sizeof(double) * m * m, s);
+    dmrg::small_eig(dg, m, m, k, dt, dc, s);
+    dmrg::dev_d2h(theta, dt, sizeof(double) * k, s);
+    dmrg::dev_d2h(C, dc, sizeof(double) * k * m, s);
+    dmrg::dev_sync(s);
+    return DMRG_OK;
+  });
+}
+
 int dmrg_test_tc_timeout(int on) {
   try {
     dmrg::tc_inject_timeout(on);

@@ -1179,7 +1179,8 @@ __device__ void small_eig_block(const double* __restrict__ G, int gld, int m, in
     jacobi_sweep(S.A, S.Q, kSeLd, np, m, S.j, buf, true, rot);
   }
   __syncthreads();
-  // ascending order of the diagonal; equal values as an exchange sort leaves them
+  // ascending order of the diagonal; equal and unordered values (NaN) as an exchange sort
+  // leaves them, so that `order` is a permutation whatever the matrix holds
   if (tid == 0) S.tie = 0;
   __syncthreads();
   if (tid < m) {
@@ -1188,7 +1189,7 @@ __device__ void small_eig_block(const double* __restrict__ G, int gld, int m, in
     for (int j = 0; j < m; ++j) {
       const double vj = S.A[j * kSeLd + j];
       rank += vj < vi;
-      if (vj == vi && j != tid) S.tie = 1;
+      if (!(vj < vi) && !(vj > vi) && j != tid) S.tie = 1;
     }
     S.order[rank] = tid;
   }
