@@ -680,8 +680,8 @@ int dmrg_batch_run(dmrg_batch* b, const double* const* x, double* const* y, uint
     // one launch per 64 instances each way, not one copy call per instance
     std::vector<dmrg::CopyJob> in, out;
     for (size_t i = 0; i < b->ctx.size(); ++i) {
-      if (x && x[i] && x[i] != b->x[i]) in.push_back({b->x[i], x[i], b->n[i]});
-      if (y && y[i] && y[i] != b->y[i]) out.push_back({y[i], b->y[i], b->n[i]});
+      if (x && x[i] && x[i] != b->x[i]) in.push_back({b->x[i], x[i], b->n[i], x[i]});
+      if (y && y[i] && y[i] != b->y[i]) out.push_back({y[i], b->y[i], b->n[i], y[i]});
     }
     dmrg::copy_batched(in, (dmrg::Stream)s);
     dmrg::tc_graph_launch(b->graph, (dmrg::Stream)s);

@@ -39,7 +39,9 @@ struct CopyJob {
   double* dst;
   const double* src;
   int64_t n;
+  const void* user;  // which of the two is the caller's
 };
+// As one copy call per job, in order, whatever the jobs are
 void copy_batched(const std::vector<CopyJob>& jobs, Stream s);
 
 // ---- grouped GEMM: C_g = C_g + sum_t alpha_t op(A_t) op(B_t), row-major blocks;

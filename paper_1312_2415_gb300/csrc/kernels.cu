@@ -154,9 +154,44 @@ __global__ void __launch_bounds__(256) k_copy_batched(const __grid_constant__ Co
   const CopyJob J = t.job[blockIdx.y];
   for (int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x; i < J.n; i += (int64_t)gridDim.x * 256) J.dst[i] = J.src[i];
 }
+
+// One launch may do the jobs if the caller's pointers are aligned device memory and no job
+// writes what another one reads or writes (an instance given twice, buffers of the batch
+// passed as vectors): the launch has no order between jobs.
+bool one_launch(const std::vector<CopyJob>& jobs) {
+  struct Range {
+    uintptr_t lo, hi;
+    bool write;
+  };
+  std::vector<Range> r;
+  for (const CopyJob& j : jobs) {
+    if (((uintptr_t)j.dst | (uintptr_t)j.src) % sizeof(double)) return false;
+    cudaPointerAttributes a;
+    if (cudaPointerGetAttributes(&a, j.user) != cudaSuccess) {
+      cudaGetLastError();
+      return false;
+    }
+    if (a.type != cudaMemoryTypeDevice) return false;
+    const uintptr_t d = (uintptr_t)j.dst, q = (uintptr_t)j.src, b = sizeof(double) * (size_t)j.n;
+    r.push_back({d, d + b, true});
+    r.push_back({q, q + b, false});
+  }
+  std::sort(r.begin(), r.end(), [](const Range& x, const Range& y) { return x.lo < y.lo; });
+  uintptr_t read = 0, written = 0;  // ends of the ranges so far
+  for (const Range& x : r) {
+    if (x.lo < written || (x.write && x.lo < read)) return false;
+    uintptr_t& end = x.write ? written : read;
+    end = std::max(end, x.hi);
+  }
+  return true;
+}
 }  // namespace
 
 void copy_batched(const std::vector<CopyJob>& jobs, Stream s) {
+  if (!one_launch(jobs)) {
+    for (const CopyJob& j : jobs) dev_d2d(j.dst, j.src, sizeof(double) * (size_t)j.n, s);
+    return;
+  }
   for (size_t b = 0; b < jobs.size(); b += 64) {
     CopyTable t{};
     const size_t n = std::min<size_t>(64, jobs.size() - b);
