@@ -318,6 +318,11 @@ int dmrg_set_device_memory_cap(size_t bytes);
  * fault, trap or endless wait is involved.  Library-wide. */
 int dmrg_test_tc_timeout(int on);
 
+/* Test hook: 1 if the refined eigensolver of dmrg_truncate corrects a pair of eigenvectors
+ * with off-diagonal g and eigenvalues gap apart (the largest is gm) in its one step, 0 if
+ * such a pair sends the block to the FP64 solver (unless g is rounding itself).  Host only. */
+int dmrg_test_refine_accepts(double g, double gap, double gm);
+
 /* Test hook: the Rayleigh-Ritz eigensolver of Davidson on its own.  The k lowest eigenpairs
  * of the symmetric m x m matrix G (row-major, the lower triangle is read; m <= 48): theta
  * (k, ascending) and C (k x m, one eigenvector per row).  Host pointers.  A NaN in

@@ -89,6 +89,7 @@ _SIGS = {
     "dmrg_batch_last_error": (ctypes.c_char_p, [_P]),
     "dmrg_batch_destroy": (None, [_P]),
     "dmrg_test_tc_timeout": (ctypes.c_int, [ctypes.c_int]),
+    "dmrg_test_refine_accepts": (ctypes.c_int, [ctypes.c_double] * 3),
     "dmrg_test_small_eig": (ctypes.c_int, [_D, ctypes.c_int, ctypes.c_int, _D, _D]),
     "dmrg_set_device_memory_cap": (ctypes.c_int, [ctypes.c_size_t]),
     "dmrg_device_memory_in_use": (ctypes.c_int, [ctypes.POINTER(ctypes.c_size_t)]),

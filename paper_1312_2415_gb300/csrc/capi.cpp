@@ -510,6 +510,8 @@ int dmrg_test_small_eig(const double* G, int m, int k, double* theta, double* C)
   });
 }
 
+int dmrg_test_refine_accepts(double g, double gap, double gm) { return dmrg::eig_refine_accepts(g, gap, gm) ? 1 : 0; }
+
 int dmrg_test_tc_timeout(int on) {
   try {
     dmrg::tc_inject_timeout(on);

@@ -205,6 +205,8 @@ struct EigSource {
   int ld, inner, trans;
 };
 void eig_refined(const std::vector<EigJob>& jobs, const std::vector<EigSource>& src, Stream s);
+// its rule for a pair of eigenvectors: off-diagonal g, eigenvalues gap apart, the largest one gm
+bool eig_refine_accepts(double g, double gap, double gm);
 
 // ---- global selection of the D largest values (ties: earlier group, lower index) ----
 // vals: concatenated eigenvalues (lambda^2) of groups with offsets goff (size G+1);

@@ -2180,6 +2180,15 @@ __global__ void k_re_half(const ReJob* __restrict__ jobs) {  // R <- R / 2 (Newt
     J.R[e] *= 0.5;
 }
 
+// May the refinement step take E = g / gap for a pair (gm: the largest eigenvalue)?  The step
+// is of first order: it leaves an off-diagonal of about g E, and an error of E^2 in the
+// eigenvectors.  So E is small and g E below the rounding of the Gram route (which has errors
+// of eps gm / gap in such a pair's vectors too); a pass that stopped at its sweep limit with
+// more than that left goes to the FP64 solver.
+__host__ __device__ inline bool refine_accepts(double g, double gap, double gm) {
+  return fabs(g) < 1e-5 * fabs(gap) && fabs(g) * fabs(g) <= 1e-16 * gm * fabs(gap);
+}
+
 // R <- E; bad[job] = 1 where the refinement cannot be trusted
 __global__ void __launch_bounds__(256) k_re_correct(const ReJob* __restrict__ jobs, int* __restrict__ bad) {
   const ReJob J = jobs[blockIdx.x];
@@ -2204,7 +2213,7 @@ __global__ void __launch_bounds__(256) k_re_correct(const ReJob* __restrict__ jo
     if (!(fabs(r) <= 1e-9)) fail = 1;  // also not finite
     if (i != j) {
       const double g = J.S[e] + lam[j] * r, gap = lam[j] - lam[i];
-      if (fabs(g) < 1e-5 * fabs(gap)) v = g / gap;
+      if (refine_accepts(g, gap, gm)) v = g / gap;
       else if (!(fabs(g) <= 1e-14 * gm)) fail = 1;
     }
     J.R[e] = v;
@@ -2232,6 +2241,8 @@ __global__ void __launch_bounds__(256) k_re_finish(const ReJob* __restrict__ job
   for (int64_t e = tid; e < (int64_t)n * n; e += 256) J.Q[(e / n) * n + rank[e % n]] = J.X[e];
 }
 }  // namespace
+
+bool eig_refine_accepts(double g, double gap, double gm) { return refine_accepts(g, gap, gm); }
 
 void eig_refined(const std::vector<EigJob>& jobs, const std::vector<EigSource>& src, Stream s) {
   if (jobs.empty()) return;
