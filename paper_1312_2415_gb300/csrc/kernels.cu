@@ -7,6 +7,7 @@
 #include <cstdio>
 #include <limits>
 #include <mutex>
+#include <new>
 #include <stdexcept>
 #include <string>
 #include <unordered_map>
@@ -1557,6 +1558,33 @@ void vec_add_noise(double* x, int64_t n, double amp, uint64_t seed, Stream s) {
 // ------------------------------------------------------------------ batched Jacobi
 
 namespace {
+// device arrays of one call, released on every way out of it
+struct DevScratch {
+  Stream s;
+  std::vector<void*> p;
+  explicit DevScratch(Stream st) : s(st) {}
+  DevScratch(const DevScratch&) = delete;
+  template <class T>
+  T* get(size_t n) {
+    p.push_back(nullptr);
+    p.back() = dev_alloc(sizeof(T) * n, s);
+    return (T*)p.back();
+  }
+  ~DevScratch() {
+    for (void* q : p) {
+      try {
+        dev_free(q, s);
+      } catch (...) {
+      }
+    }
+  }
+};
+
+// an allocation that failed (the cap, the device or the host), not another error
+bool no_room(const std::exception& e) {
+  return dynamic_cast<const std::bad_alloc*>(&e) || std::string(e.what()).find("out of memory") != std::string::npos;
+}
+
 constexpr int kEigSmemN = 64;  // blocks up to this size are diagonalised in shared memory
 
 // Cyclic Jacobi (round-robin pairing, n/2 rotations per step) on one symmetric block per
@@ -2002,11 +2030,12 @@ void bj_sweeps(std::vector<BjJob<T>>& bj, const double* gmax, int sweeps, Stream
   }
   const int nj = (int)bj.size();
   const int nch = (nmax + kOP - 1) / kOP;  // 64-wide chunks of the largest matrix
-  BjJob<T>* d = (BjJob<T>*)dev_alloc(sizeof(BjJob<T>) * nj, s);
+  DevScratch mem(s);
+  BjJob<T>* d = mem.get<BjJob<T>>(nj);
   dev_h2d(d, bj.data(), sizeof(BjJob<T>) * nj, s);
-  T* vbuf = (T*)dev_alloc(sizeof(T) * (size_t)pairs * kOP * kOP, s);
-  int* flag = (int*)dev_alloc(sizeof(int) * pairs, s);
-  int* nrot = (int*)dev_alloc(sizeof(int) * nj, s);
+  T* vbuf = mem.get<T>((size_t)pairs * kOP * kOP);
+  int* flag = mem.get<int>(pairs);
+  int* nrot = mem.get<int>(nj);
   std::vector<int> hrot(nj);
   const size_t sh = sizeof(T) * 2 * kOP * kOL;
   static bool attr = false;  // per element type
@@ -2031,10 +2060,6 @@ void bj_sweeps(std::vector<BjJob<T>>& bj, const double* gmax, int sweeps, Stream
     for (int v : hrot) any = any || v > 0;
     if (!any) break;
   }
-  dev_free(nrot, s);
-  dev_free(flag, s);
-  dev_free(vbuf, s);
-  dev_free(d, s);
 }
 
 }  // namespace
@@ -2050,9 +2075,10 @@ static void eig_block_jacobi(const std::vector<EigJob>& jobs, Stream s) {
   const int nj = (int)bj.size();
   const size_t shf = sizeof(double) * 2 * nmax;
   if (shf > 220 * 1024) throw std::runtime_error("eig_batched: block too large");
-  BjJob<double>* d = (BjJob<double>*)dev_alloc(sizeof(BjJob<double>) * nj, s);
+  DevScratch mem(s);
+  BjJob<double>* d = mem.get<BjJob<double>>(nj);
   dev_h2d(d, bj.data(), sizeof(BjJob<double>) * nj, s);
-  double* gmax = (double*)dev_alloc(sizeof(double) * nj, s);
+  double* gmax = mem.get<double>(nj);
   k_bj_prep<<<nj, 256, 0, S(s)>>>(d, gmax);
   ++g_launches;
   bj_sweeps(bj, gmax, 40, s);
@@ -2061,8 +2087,6 @@ static void eig_block_jacobi(const std::vector<EigJob>& jobs, Stream s) {
   k_bj_finish<<<nj, 256, shf, S(s)>>>(d);
   ++g_launches;
   ck(cudaGetLastError(), "bj finish");
-  dev_free(gmax, s);
-  dev_free(d, s);
 }
 
 void eig_batched(const std::vector<EigJob>& jobs, Stream s) {
@@ -2073,7 +2097,8 @@ void eig_batched(const std::vector<EigJob>& jobs, Stream s) {
     if (j.n <= kEigSmemN) { small.push_back(j); nmax_s = std::max(nmax_s, j.n); }
     else { large.push_back(j); nmax_l = std::max(nmax_l, j.n); }
   }
-  EigJob* d = (EigJob*)dev_alloc(jobs.size() * sizeof(EigJob), s);
+  DevScratch mem(s);
+  EigJob* d = mem.get<EigJob>(jobs.size());
   if (!small.empty()) {
     dev_h2d(d, small.data(), small.size() * sizeof(EigJob), s);
     const int np = (nmax_s + 1) & ~1;
@@ -2084,7 +2109,6 @@ void eig_batched(const std::vector<EigJob>& jobs, Stream s) {
     ck(cudaGetLastError(), "eig_batched (shared)");
   }
   if (!large.empty()) eig_block_jacobi(large, s);
-  dev_free(d, s);
 }
 
 // ------------------------------------------------------------------ refined eigensolver
@@ -2244,175 +2268,180 @@ __global__ void __launch_bounds__(256) k_re_finish(const ReJob* __restrict__ job
 
 bool eig_refine_accepts(double g, double gap, double gm) { return refine_accepts(g, gap, gm); }
 
-void eig_refined(const std::vector<EigJob>& jobs, const std::vector<EigSource>& src, Stream s) {
-  if (jobs.empty()) return;
+namespace {
+// the jobs that have to go to eig_batched (their Gram matrices are as they were)
+std::vector<EigJob> refined_passes(const std::vector<EigJob>& jobs, const std::vector<EigSource>& src, int nmax, Stream s) {
   std::vector<int64_t> off(1, 0), toff(1, 0);
-  int nmax = 1;
   for (size_t k = 0; k < jobs.size(); ++k) {
     off.push_back(off.back() + (int64_t)jobs[k].n * jobs[k].n);
     toff.push_back(toff.back() + (int64_t)src[k].inner * jobs[k].n);
-    nmax = std::max(nmax, jobs[k].n);
   }
+  const int64_t tot = off.back();
+  const int nj = (int)jobs.size();
+  // X, X2, S, R, T (FP64), A32, Q32 (FP32)
+  const int64_t ttot = toff.back();
+  DevScratch mem(s);
+  double* buf = mem.get<double>((size_t)(tot * 5 + ttot));
+  double *X = buf, *X2 = X + tot, *Sm = X2 + tot, *R = Sm + tot, *T = R + tot;
+  float *A32 = (float*)(T + ttot), *Q32 = A32 + tot;
+  std::vector<int> hbad(nj, 0);
+  struct Plans {
+    Stream s;
+    GemmPlan *pq = nullptr, *pr = nullptr, *pn = nullptr, *pt = nullptr, *ps = nullptr;
+    ~Plans() {
+      for (GemmPlan* p : {pq, pr, pn, pt, ps}) {
+        try {
+          gemm_plan_free(p, s);
+        } catch (...) {
+        }
+      }
+    }
+  } g{s};
+  GemmPlan *&pq = g.pq, *&pr = g.pr, *&pn = g.pn, *&pt = g.pt, *&ps = g.ps;
+  std::vector<ReJob> re;
+  std::vector<int> small;
+  std::vector<BjJob<float>> big;
+  int nsm = 1;
+  for (int k = 0; k < nj; ++k) {
+    const EigJob& j = jobs[k];
+    const int64_t o = off[k];
+    re.push_back({j.A, X + o, Sm + o, R + o, j.w, j.Q, A32 + o, Q32 + o, j.n, 0});
+    if (j.n <= kEigSmemN) {
+      small.push_back(k);
+      nsm = std::max(nsm, j.n);
+    } else {
+      big.push_back({A32 + o, Q32 + o, nullptr, j.n, 0, 0, 0});
+    }
+  }
+  ReJob* d = mem.get<ReJob>(nj);
+  dev_h2d(d, re.data(), sizeof(ReJob) * nj, s);
+  int* dsmall = mem.get<int>(small.size() + 1);
+  dev_h2d(dsmall, small.data(), sizeof(int) * small.size(), s);
+  int* dbad = mem.get<int>(nj);
+  // the three passes: floor (of the largest diagonal entry, scaled to 1: a little above
+  // what FP32 rounding leaves of the part that the pass resolves), sweeps at most, and
+  // Newton-Schulz steps (FP32 rotations leave Q orthonormal to 1e-5 where they are large)
+  constexpr double kFloor[3] = {1e-6, 5e-13, 5e-16};
+  constexpr int kSweeps[3] = {10, 8, 4}, kSchulz[3] = {2, 2, 1};
+  const size_t nb = big.size();
+  double* gbig = mem.get<double>(std::max<size_t>(3 * nb, 1));
+  std::vector<double> fl;
+  for (double f : kFloor) fl.insert(fl.end(), nb, f);
+  dev_h2d(gbig, fl.data(), sizeof(double) * fl.size(), s);
+  // one n-column product per job: C (m x n) += alpha op(A) B
+  auto plan = [&](auto task) {
+    std::vector<GemmTask> t;
+    std::vector<GemmGroup> g;
+    for (int k = 0; k < nj; ++k) {
+      double* c = nullptr;
+      int m = jobs[k].n;
+      t.push_back(task(k, c, m));
+      g.push_back({c, jobs[k].n, m, jobs[k].n, k, k + 1, 0});
+    }
+    return gemm_plan_upload(t, g, s, GEMM_SHARED);
+  };
+  pq = plan([&](int k, double*& c, int&) {  // X2 = X Q (Q widened into S)
+    const int n = jobs[k].n;
+    c = X2 + off[k];
+    return GemmTask{X + off[k], Sm + off[k], n, n, n, 0, 0, 1.0};
+  });
+  pr = plan([&](int k, double*& c, int&) {  // R -= X^T X
+    const int n = jobs[k].n;
+    c = R + off[k];
+    return GemmTask{X + off[k], X + off[k], n, n, n, 1, 0, -1.0};
+  });
+  pn = plan([&](int k, double*& c, int&) {  // X2 += X R
+    const int n = jobs[k].n;
+    c = X2 + off[k];
+    return GemmTask{X + off[k], R + off[k], n, n, n, 0, 0, 1.0};
+  });
+  pt = plan([&](int k, double*& c, int& m) {  // T = M^T X or M X
+    const int n = jobs[k].n;
+    c = T + toff[k];
+    m = src[k].inner;
+    return GemmTask{src[k].M, X + off[k], src[k].ld, n, n, src[k].trans, 0, 1.0};
+  });
+  ps = plan([&](int k, double*& c, int&) {  // S = T^T T
+    const int n = jobs[k].n;
+    c = Sm + off[k];
+    return GemmTask{T + toff[k], T + toff[k], n, n, src[k].inner, 1, 0, 1.0};
+  });
+  const size_t bytes = sizeof(double) * (size_t)tot;
+  const dim3 grid(nj, std::max(1, std::min(64, nmax * nmax / 4096)));
+  const int np = (nsm + 1) & ~1;
+  const size_t shs = sizeof(float) * 2 * (size_t)np * (np + 1), shc = sizeof(double) * 2 * (size_t)nmax;
+  if (shc > 48 * 1024) {
+    ck(cudaFuncSetAttribute(k_re_correct, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shc), "eig smem");
+    ck(cudaFuncSetAttribute(k_re_finish, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shc), "eig smem");
+  }
+  // X <- X2 + ... where X2 holds a copy of X, then X = X2
+  auto residual = [&]() {  // R = I - X^T X
+    k_re_identity<<<grid, 256, 0, S(s)>>>(d);
+    gemm_plan_run(pr, s, GEMM_SHARED);
+    ++g_launches;
+  };
+  auto add_correction = [&]() {  // X <- X + X R
+    dev_d2d(X2, X, bytes, s);
+    gemm_plan_run(pn, s, GEMM_SHARED);
+    dev_d2d(X, X2, bytes, s);
+  };
+  auto schulz = [&]() {  // X <- X (3 I - X^T X) / 2
+    residual();
+    k_re_half<<<grid, 256, 0, S(s)>>>(d);
+    ++g_launches;
+    add_correction();
+  };
+  for (int pass = 0; pass < 3; ++pass) {
+    k_re_start<<<nj, 256, 0, S(s)>>>(d, pass == 0);
+    if (!small.empty()) k_re_small<<<(int)small.size(), 256, shs, S(s)>>>(d, dsmall, kSweeps[pass], (float)kFloor[pass]);
+    bj_sweeps(big, gbig + pass * nb, kSweeps[pass], s);
+    k_re_widen<<<grid, 256, 0, S(s)>>>(d, pass == 0);
+    g_launches += 3;
+    if (pass > 0) {
+      dev_zero(X2, bytes, s);
+      gemm_plan_run(pq, s, GEMM_SHARED);
+      dev_d2d(X, X2, bytes, s);
+    }
+    for (int u = 0; u < kSchulz[pass]; ++u) schulz();
+    dev_zero(T, sizeof(double) * (size_t)ttot, s);
+    gemm_plan_run(pt, s, GEMM_SHARED);
+    dev_zero(Sm, bytes, s);
+    gemm_plan_run(ps, s, GEMM_SHARED);
+  }
+  residual();
+  k_re_correct<<<nj, 256, shc, S(s)>>>(d, dbad);
+  add_correction();
+  schulz();
+  ck(cudaGetLastError(), "refined eig");
+  dev_d2h(hbad.data(), dbad, sizeof(int) * nj, s);
+  k_re_finish<<<nj, 256, shc, S(s)>>>(d);
+  g_launches += 2;
+  ck(cudaGetLastError(), "refined eig");
+  dev_sync(s);
+  std::vector<EigJob> again;
+  for (int k = 0; k < nj; ++k)
+    if (hbad[k]) again.push_back(jobs[k]);
+  return again;
+}
+}  // namespace
+
+void eig_refined(const std::vector<EigJob>& jobs, const std::vector<EigSource>& src, Stream s) {
+  if (jobs.empty()) return;
+  int nmax = 1;
+  for (const EigJob& j : jobs) nmax = std::max(nmax, j.n);
   // Small blocks: the passes' launches and tables cost some 0.7 ms whatever the sizes.  Whole
   // call, Hubbard chains, Jacobi / refined: largest block 11 rows 0.59 / 0.84 ms, 20 rows 0.89 /
   // 1.02, 26 rows 1.37 / 1.16, 49 rows 4.5 / 2.1.
   constexpr int kRefineRows = 23;
   if (nmax < kRefineRows || sizeof(double) * 2 * (size_t)nmax > 200 * 1024) return eig_batched(jobs, s);
-  const int64_t tot = off.back();
-  const int nj = (int)jobs.size();
-  // X, X2, S, R, T (FP64), A32, Q32 (FP32)
-  const int64_t ttot = toff.back();
-  double* buf = nullptr;
-  try {
-    buf = (double*)dev_alloc(sizeof(double) * (size_t)(tot * 5 + ttot), s);
-  } catch (const std::exception&) {  // no room (the cap, or the device): the solver in place
-    cudaGetLastError();
-    return eig_batched(jobs, s);
-  }
-  double *X = buf, *X2 = X + tot, *Sm = X2 + tot, *R = Sm + tot, *T = R + tot;
-  float *A32 = (float*)(T + ttot), *Q32 = A32 + tot;
-  ReJob* d = nullptr;
-  int *dsmall = nullptr, *dbad = nullptr;
-  double* gbig = nullptr;
-  GemmPlan *pq = nullptr, *pr = nullptr, *pn = nullptr, *pt = nullptr, *ps = nullptr;
-  std::vector<int> hbad(nj, 0);
-  auto cleanup = [&]() {
-    for (GemmPlan* p : {pq, pr, pn, pt, ps}) gemm_plan_free(p, s);
-    dev_free(d, s);
-    dev_free(dsmall, s);
-    dev_free(dbad, s);
-    dev_free(gbig, s);
-    dev_free(buf, s);
-  };
-  try {
-    std::vector<ReJob> re;
-    std::vector<int> small;
-    std::vector<BjJob<float>> big;
-    int nsm = 1;
-    for (int k = 0; k < nj; ++k) {
-      const EigJob& j = jobs[k];
-      const int64_t o = off[k];
-      re.push_back({j.A, X + o, Sm + o, R + o, j.w, j.Q, A32 + o, Q32 + o, j.n, 0});
-      if (j.n <= kEigSmemN) {
-        small.push_back(k);
-        nsm = std::max(nsm, j.n);
-      } else {
-        big.push_back({A32 + o, Q32 + o, nullptr, j.n, 0, 0, 0});
-      }
-    }
-    d = (ReJob*)dev_alloc(sizeof(ReJob) * nj, s);
-    dev_h2d(d, re.data(), sizeof(ReJob) * nj, s);
-    dsmall = (int*)dev_alloc(sizeof(int) * (small.size() + 1), s);
-    dev_h2d(dsmall, small.data(), sizeof(int) * small.size(), s);
-    dbad = (int*)dev_alloc(sizeof(int) * nj, s);
-    // the three passes: floor (of the largest diagonal entry, scaled to 1: a little above
-    // what FP32 rounding leaves of the part that the pass resolves), sweeps at most, and
-    // Newton-Schulz steps (FP32 rotations leave Q orthonormal to 1e-5 where they are large)
-    constexpr double kFloor[3] = {1e-6, 5e-13, 5e-16};
-    constexpr int kSweeps[3] = {10, 8, 4}, kSchulz[3] = {2, 2, 1};
-    const size_t nb = big.size();
-    gbig = (double*)dev_alloc(sizeof(double) * std::max<size_t>(3 * nb, 1), s);
-    std::vector<double> fl;
-    for (double f : kFloor) fl.insert(fl.end(), nb, f);
-    dev_h2d(gbig, fl.data(), sizeof(double) * fl.size(), s);
-    // one n-column product per job: C (m x n) += alpha op(A) B
-    auto plan = [&](auto task) {
-      std::vector<GemmTask> t;
-      std::vector<GemmGroup> g;
-      for (int k = 0; k < nj; ++k) {
-        double* c = nullptr;
-        int m = jobs[k].n;
-        t.push_back(task(k, c, m));
-        g.push_back({c, jobs[k].n, m, jobs[k].n, k, k + 1, 0});
-      }
-      return gemm_plan_upload(t, g, s, GEMM_SHARED);
-    };
-    pq = plan([&](int k, double*& c, int&) {  // X2 = X Q (Q widened into S)
-      const int n = jobs[k].n;
-      c = X2 + off[k];
-      return GemmTask{X + off[k], Sm + off[k], n, n, n, 0, 0, 1.0};
-    });
-    pr = plan([&](int k, double*& c, int&) {  // R -= X^T X
-      const int n = jobs[k].n;
-      c = R + off[k];
-      return GemmTask{X + off[k], X + off[k], n, n, n, 1, 0, -1.0};
-    });
-    pn = plan([&](int k, double*& c, int&) {  // X2 += X R
-      const int n = jobs[k].n;
-      c = X2 + off[k];
-      return GemmTask{X + off[k], R + off[k], n, n, n, 0, 0, 1.0};
-    });
-    pt = plan([&](int k, double*& c, int& m) {  // T = M^T X or M X
-      const int n = jobs[k].n;
-      c = T + toff[k];
-      m = src[k].inner;
-      return GemmTask{src[k].M, X + off[k], src[k].ld, n, n, src[k].trans, 0, 1.0};
-    });
-    ps = plan([&](int k, double*& c, int&) {  // S = T^T T
-      const int n = jobs[k].n;
-      c = Sm + off[k];
-      return GemmTask{T + toff[k], T + toff[k], n, n, src[k].inner, 1, 0, 1.0};
-    });
-    const size_t bytes = sizeof(double) * (size_t)tot;
-    const dim3 grid(nj, std::max(1, std::min(64, nmax * nmax / 4096)));
-    const int np = (nsm + 1) & ~1;
-    const size_t shs = sizeof(float) * 2 * (size_t)np * (np + 1), shc = sizeof(double) * 2 * (size_t)nmax;
-    if (shc > 48 * 1024) {
-      ck(cudaFuncSetAttribute(k_re_correct, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shc), "eig smem");
-      ck(cudaFuncSetAttribute(k_re_finish, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shc), "eig smem");
-    }
-    // X <- X2 + ... where X2 holds a copy of X, then X = X2
-    auto residual = [&]() {  // R = I - X^T X
-      k_re_identity<<<grid, 256, 0, S(s)>>>(d);
-      gemm_plan_run(pr, s, GEMM_SHARED);
-      ++g_launches;
-    };
-    auto add_correction = [&]() {  // X <- X + X R
-      dev_d2d(X2, X, bytes, s);
-      gemm_plan_run(pn, s, GEMM_SHARED);
-      dev_d2d(X, X2, bytes, s);
-    };
-    auto schulz = [&]() {  // X <- X (3 I - X^T X) / 2
-      residual();
-      k_re_half<<<grid, 256, 0, S(s)>>>(d);
-      ++g_launches;
-      add_correction();
-    };
-    for (int pass = 0; pass < 3; ++pass) {
-      k_re_start<<<nj, 256, 0, S(s)>>>(d, pass == 0);
-      if (!small.empty()) k_re_small<<<(int)small.size(), 256, shs, S(s)>>>(d, dsmall, kSweeps[pass], (float)kFloor[pass]);
-      bj_sweeps(big, gbig + pass * nb, kSweeps[pass], s);
-      k_re_widen<<<grid, 256, 0, S(s)>>>(d, pass == 0);
-      g_launches += 3;
-      if (pass > 0) {
-        dev_zero(X2, bytes, s);
-        gemm_plan_run(pq, s, GEMM_SHARED);
-        dev_d2d(X, X2, bytes, s);
-      }
-      for (int u = 0; u < kSchulz[pass]; ++u) schulz();
-      dev_zero(T, sizeof(double) * (size_t)ttot, s);
-      gemm_plan_run(pt, s, GEMM_SHARED);
-      dev_zero(Sm, bytes, s);
-      gemm_plan_run(ps, s, GEMM_SHARED);
-    }
-    residual();
-    k_re_correct<<<nj, 256, shc, S(s)>>>(d, dbad);
-    add_correction();
-    schulz();
-    ck(cudaGetLastError(), "refined eig");
-    dev_d2h(hbad.data(), dbad, sizeof(int) * nj, s);
-    k_re_finish<<<nj, 256, shc, S(s)>>>(d);
-    g_launches += 2;
-    ck(cudaGetLastError(), "refined eig");
-    dev_sync(s);
-  } catch (...) {
-    cleanup();
-    throw;
-  }
-  cleanup();
   std::vector<EigJob> again;
-  for (int k = 0; k < nj; ++k)
-    if (hbad[k]) again.push_back(jobs[k]);
+  try {
+    again = refined_passes(jobs, src, nmax, s);
+  } catch (const std::exception& e) {
+    if (!no_room(e)) throw;
+    cudaGetLastError();
+    again = jobs;  // the workspace has been released: the solver in place
+  }
   eig_batched(again, s);
 }
 
