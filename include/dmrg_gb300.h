@@ -318,6 +318,16 @@ int dmrg_set_device_memory_cap(size_t bytes);
  * fault, trap or endless wait is involved.  Library-wide. */
 int dmrg_test_tc_timeout(int on);
 
+/* Test hook: the grouped block products on their own, on blocks inside data (n doubles, host
+ * pointers throughout; the groups' blocks may not overlap any other).  groups: ngroups x 6
+ * (C offset, ldc, rows, columns, first task, end task); tasks: ntasks x 7 (A offset or -1 for
+ * the identity, B offset, lda, ldb, inner size, transA, transB), alpha per task; C += sum of
+ * alpha op(A) op(B).  upload: a sum of 1 (ordered sums), 2 (shared sums), 4 (C = the sum),
+ * 8 (ordered: lane kernel), 16 (ordered: kernel in rounds); run: 1 or 2.  DMRG_EINVAL for
+ * blocks outside data, DMRG_EINTERNAL for a run of a kind not uploaded. */
+int dmrg_test_block_products(const int64_t* tasks, const double* alpha, int ntasks, const int64_t* groups, int ngroups,
+                             double* data, int64_t n, int upload, int run);
+
 /* Test hook: 1 if the refined eigensolver of dmrg_truncate corrects a pair of eigenvectors
  * with off-diagonal g and eigenvalues gap apart (the largest is gm) in its one step, 0 if
  * such a pair sends the block to the FP64 solver (unless g is rounding itself).  Host only. */

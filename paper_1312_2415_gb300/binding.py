@@ -89,6 +89,8 @@ _SIGS = {
     "dmrg_batch_last_error": (ctypes.c_char_p, [_P]),
     "dmrg_batch_destroy": (None, [_P]),
     "dmrg_test_tc_timeout": (ctypes.c_int, [ctypes.c_int]),
+    "dmrg_test_block_products": (ctypes.c_int, [_I64, _D, ctypes.c_int, _I64, ctypes.c_int, _D, ctypes.c_int64,
+                                                ctypes.c_int, ctypes.c_int]),
     "dmrg_test_refine_accepts": (ctypes.c_int, [ctypes.c_double] * 3),
     "dmrg_test_small_eig": (ctypes.c_int, [_D, ctypes.c_int, ctypes.c_int, _D, _D]),
     "dmrg_set_device_memory_cap": (ctypes.c_int, [ctypes.c_size_t]),
@@ -332,6 +334,19 @@ def test_tc_timeout(on, path=None):
     rc = load(path).dmrg_test_tc_timeout(int(on))
     if rc != OK:
         raise DMRGError(rc, "dmrg_test_tc_timeout")
+
+
+def test_block_products(tasks, alpha, groups, data, upload, run, path=None):
+    """Test hook: the grouped block products on host data (see the header); returns the data."""
+    t = np.ascontiguousarray(tasks, dtype=np.int64)
+    a = np.ascontiguousarray(alpha, dtype=np.float64)
+    g = np.ascontiguousarray(groups, dtype=np.int64)
+    d = np.array(data, dtype=np.float64)
+    rc = load(path).dmrg_test_block_products(t.ctypes.data_as(_I64), _dptr(a), len(a), g.ctypes.data_as(_I64), len(g),
+                                             _dptr(d), d.size, int(upload), int(run))
+    if rc != OK:
+        raise DMRGError(rc, "dmrg_test_block_products")
+    return d
 
 
 def test_small_eig(G, k, path=None):

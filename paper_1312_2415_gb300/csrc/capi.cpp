@@ -510,6 +510,53 @@ int dmrg_test_small_eig(const double* G, int m, int k, double* theta, double* C)
   });
 }
 
+int dmrg_test_block_products(const int64_t* tasks, const double* alpha, int ntasks, const int64_t* groups, int ngroups,
+                             double* data, int64_t n, int upload, int run) {
+  if (!tasks || !alpha || !groups || !data || ntasks < 0 || ngroups < 0 || n < 1) return DMRG_EINVAL;
+  std::string err;
+  return guard_err(err, [&] {
+    // every block inside data, the groups' blocks apart from all others' (the caller's part)
+    auto inside = [&](int64_t off, int64_t ld, int64_t rows, int64_t cols) {
+      return off >= 0 && rows >= 0 && cols >= 0 && rows <= n && ld >= cols && ld <= n &&
+             (rows == 0 || cols == 0 || off + (rows - 1) * ld + cols <= n);
+    };
+    for (int q = 0; q < ngroups; ++q) {
+      const int64_t* g = groups + 6 * q;  // C, ldc, m, n, first task, end
+      if (!inside(g[0], g[1], g[2], g[3]) || g[4] < 0 || g[4] > g[5] || g[5] > ntasks) return DMRG_EINVAL;
+      for (int64_t k = g[4]; k < g[5]; ++k) {
+        const int64_t* t = tasks + 7 * k;  // A (-1: identity), B, lda, ldb, k, transA, transB
+        const int64_t kk = t[0] < 0 ? g[2] : t[4];
+        if (t[0] >= 0 && (kk < 1 || !(t[5] ? inside(t[0], t[2], kk, g[2]) : inside(t[0], t[2], g[2], kk)))) return DMRG_EINVAL;
+        if (!(t[6] ? inside(t[1], t[3], g[3], kk) : inside(t[1], t[3], kk, g[3]))) return DMRG_EINVAL;
+      }
+    }
+    dmrg::Stream s = (dmrg::Stream)cudaStreamLegacy;
+    DevBuf b(n, s);
+    dmrg::dev_h2d(b.p, data, sizeof(double) * n, s);
+    std::vector<dmrg::GemmTask> t;
+    std::vector<dmrg::GemmGroup> g;
+    for (int k = 0; k < ntasks; ++k) {
+      const int64_t* q = tasks + 7 * k;
+      t.push_back({q[0] < 0 ? nullptr : b.p + q[0], b.p + q[1], (int)q[2], (int)q[3], (int)q[4], (int)q[5], (int)q[6], alpha[k]});
+    }
+    for (int k = 0; k < ngroups; ++k) {
+      const int64_t* q = groups + 6 * k;
+      g.push_back({b.p + q[0], (int)q[1], (int)q[2], (int)q[3], (int)q[4], (int)q[5], 0});
+    }
+    dmrg::GemmPlan* p = dmrg::gemm_plan_upload(t, g, s, upload);
+    try {
+      dmrg::gemm_plan_run(p, s, run);
+      dmrg::dev_d2h(data, b.p, sizeof(double) * n, s);
+      dmrg::dev_sync(s);
+    } catch (...) {
+      dmrg::gemm_plan_free(p, s);
+      throw;
+    }
+    dmrg::gemm_plan_free(p, s);
+    return DMRG_OK;
+  });
+}
+
 int dmrg_test_refine_accepts(double g, double gap, double gm) { return dmrg::eig_refine_accepts(g, gap, gm) ? 1 : 0; }
 
 int dmrg_test_tc_timeout(int on) {

@@ -598,6 +598,7 @@ std::vector<GemmJob> gemm_jobs(const std::vector<GemmGroup>& g, const std::vecto
 GemmPlan* gemm_plan_upload(const std::vector<GemmTask>& t, std::vector<GemmGroup>& g, Stream s, int sums) {
   GemmPlan* p = new GemmPlan;
   p->ntasks = (int64_t)t.size();
+  p->kinds = sums & (GEMM_ORDERED | GEMM_SHARED);
   p->overwrite = (sums & GEMM_OVERWRITE) != 0;
   // per group: columns in all, rows per lane; chunks of the whole table (rounds)
   std::vector<int64_t> ks(g.size(), 0);
@@ -617,6 +618,7 @@ GemmPlan* gemm_plan_upload(const std::vector<GemmTask>& t, std::vector<GemmGroup
     ++live;
   }
   p->rounds = (sums & GEMM_ORDERED) && p->ntasks >= kGemmRoundTasks * live && chunks <= kGemmMaxChunks;
+  if (sums & (GEMM_LANES | GEMM_ROUNDS)) p->rounds = (sums & GEMM_ROUNDS) != 0;
   const std::vector<int> one(p->rounds ? g.size() : 0, 1);  // rows per lane of the rounds
   try {
     for (int kind = 0; kind < 2; ++kind) {
@@ -664,6 +666,7 @@ namespace {
 template <bool kRemap>
 void gemm_launch(const GemmPlan* p, const Remap& rm, int sums, Stream s) {
   const int kind = sums == GEMM_ORDERED ? 0 : 1;
+  if (p && !(p->kinds & sums)) throw std::logic_error("block products run with sums they were not uploaded for");
   if (!p || p->njobs[kind] == 0) return;
   const int n = p->njobs[kind];
   const GemmJob* jobs = p->jobs[kind];

@@ -26,6 +26,7 @@ struct GemmPlan {
   GemmJob* jobs[2] = {nullptr, nullptr};  // ordered sums, shared sums
   GemmChunk* chunks = nullptr;
   int njobs[2] = {0, 0};
+  int kinds = 0;           // GEMM_ORDERED, GEMM_SHARED: the job tables it has
   bool overwrite = false;  // C = sum instead of C += sum
   bool rounds = false;  // ordered sums by k_gemm_rounds
   int64_t ntasks = 0;
