@@ -10,6 +10,7 @@
 #include <new>
 #include <stdexcept>
 #include <string>
+#include <type_traits>
 #include <unordered_map>
 
 #include "device.hpp"
@@ -313,52 +314,53 @@ __device__ __forceinline__ void gemm_sum(const GemmTask* __restrict__ tasks, int
       pa[r] = A + ro[r] * sai;
       s[r] = kOrdered ? acc[r] : 0.0;
     }
-    // what multiplies an element of A (ordered sums): alpha, or its sign moved to B
-    const double fa = kOrdered && !unit ? cur.alpha : 1.0;
-    const double fb = kOrdered && unit && cur.alpha < 0.0 ? -0.0 : 0.0;
-    auto flip = [&](double v) {
-      return __longlong_as_double(__double_as_longlong(v) ^ __double_as_longlong(fb));
-    };
-    int k = cur.k;
-    for (; k >= 4; k -= 4) {
-      double b[4], a[R][4];
+    // What multiplies an element of A (ordered sums): alpha, or its sign moved to B.  The two
+    // are separate loops: a multiplication behind a test inside the loop is issued whether it
+    // is wanted or not, and costs as much as the FMA.  Measured (one loop / two): tables of
+    // 16 to 150 rows with alpha = +-1 380..520 / 740..1210 GFLOP/s (shared sums the same);
+    // phase 1 of random L=28, D=2500, sites 13, 14 after a step 231 / 105 ms, phase 2 174 / 77
+    // ms (32 x 32 tiles staged in shared memory: 155 and 155 ms).
+    const long long fb = kOrdered && unit && cur.alpha < 0.0 ? (long long)(1ull << 63) : 0ll;
+    auto flip = [&](double v) { return __longlong_as_double(__double_as_longlong(v) ^ fb); };
+    auto sum = [&](auto scale) {
+      constexpr bool kScale = decltype(scale)::value;
+      int k = cur.k;
+      for (; k >= 4; k -= 4) {
+        double b[4], a[R][4];
 #pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        b[u] = kOrdered ? flip(pb[u * sbk]) : pb[u * sbk];
+        for (int u = 0; u < 4; ++u) {
+          b[u] = kOrdered && !kScale ? flip(pb[u * sbk]) : pb[u * sbk];
 #pragma unroll
-        for (int r = 0; r < R; ++r) a[r][u] = pa[r][u * sak];
-      }
-      if (kOrdered && fa != 1.0) {
+          for (int r = 0; r < R; ++r) a[r][u] = kScale ? pa[r][u * sak] * cur.alpha : pa[r][u * sak];
+        }
 #pragma unroll
         for (int u = 0; u < 4; ++u)
 #pragma unroll
-          for (int r = 0; r < R; ++r) a[r][u] *= fa;
+          for (int r = 0; r < R; ++r) s[r] = fma(a[r][u], b[u], s[r]);
+        pb += 4 * sbk;
+#pragma unroll
+        for (int r = 0; r < R; ++r) pa[r] += 4 * sak;
       }
+      if (k > 0) {  // the last one to three columns, their loads in flight together
+        double b[3], a[R][3];
 #pragma unroll
-      for (int u = 0; u < 4; ++u)
+        for (int u = 0; u < 3; ++u)
+          if (!kOrdered || u < k) {
+            const int o = kOrdered || u < k ? u : 0;  // shared sums: a repeated load for a branch
+            b[u] = kOrdered && !kScale ? flip(pb[o * sbk]) : pb[o * sbk];
 #pragma unroll
-        for (int r = 0; r < R; ++r) s[r] = fma(a[r][u], b[u], s[r]);
-      pb += 4 * sbk;
+            for (int r = 0; r < R; ++r) a[r][u] = kScale ? pa[r][o * sak] * cur.alpha : pa[r][o * sak];
+          }
 #pragma unroll
-      for (int r = 0; r < R; ++r) pa[r] += 4 * sak;
-    }
-    if (k > 0) {  // the last one to three columns, their loads in flight together
-      double b[3], a[R][3];
+        for (int u = 0; u < 3; ++u)
+          if (u < k) {
 #pragma unroll
-      for (int u = 0; u < 3; ++u)
-        if (!kOrdered || u < k) {
-          const int o = kOrdered || u < k ? u : 0;  // shared sums: a repeated load for a branch
-          b[u] = kOrdered ? flip(pb[o * sbk]) : pb[o * sbk];
-#pragma unroll
-          for (int r = 0; r < R; ++r) a[r][u] = pa[r][o * sak];
-        }
-#pragma unroll
-      for (int u = 0; u < 3; ++u)
-        if (u < k) {
-#pragma unroll
-          for (int r = 0; r < R; ++r) s[r] = fma(kOrdered && fa != 1.0 ? __dmul_rn(a[r][u], fa) : a[r][u], b[u], s[r]);
-        }
-    }
+            for (int r = 0; r < R; ++r) s[r] = fma(a[r][u], b[u], s[r]);
+          }
+      }
+    };
+    if (kOrdered && !unit) sum(std::true_type{});
+    else sum(std::false_type{});
 #pragma unroll
     for (int r = 0; r < R; ++r) acc[r] = kOrdered ? s[r] : fma(cur.alpha, s[r], acc[r]);
   }
