@@ -371,11 +371,10 @@ __device__ __forceinline__ void gemm_sum(const GemmTask* __restrict__ tasks, int
 // does everything.  One CTA per 32-element slice, one row per lane: in each round
 // kRoundWarps - 1 warps fetch one chunk each (up to four columns of one task; A scaled by
 // alpha on the way) into shared memory while the last warp sums the previous round's chunks
-// in order.  The chunks' table (task, first column) is made at upload.  Measured (phase 2,
-// loads when a task starts / rounds): Hubbard L=8, D=64 236 / 47 us (one warp with three
-// chunks in flight 165 us); random L=12, D=350 318 / 115 us, L=12, D=500 1.65 / 0.53 ms, L=16,
-// D=600 2.88 / 1.81 ms.  Short lists (phase 1, one task per sum) start faster the other way: 28
-// / 41 us.
+// in order.  The chunks' table (task, first column) is made at upload.  Measured (phase 2, lanes
+// / rounds): Hubbard L=8, D=64 165 / 47 us; random L=12, D=350 443 / 288 us, L=12, D=500 1.26 / 0.53
+// ms.  Short lists (phase 1, one task per sum) start faster the other way (25 / 41 us), and so do
+// tables that fill the SMs (OrderedCost).
 constexpr int kRoundWarps = 8;
 
 template <bool kRemap>
@@ -552,12 +551,36 @@ int rows_per_lane(int m, int n, bool strided_b) {
 // its start.  Groups above it are shared by up to max_ns warps, groups below it give one
 // warp several of their 32-lane slices.  Longest jobs first.
 constexpr int64_t kGemmMinWork = 48, kGemmJobsTarget = 152 * 40;
-// ordered sums in rounds: lists of at least kGemmRoundTasks tasks in the mean, in tables of at
-// most kGemmMaxChunks chunks (the chunk table costs the host more than the rounds save on large
-// blocks: phase 2 of random L=28, D=1500, 5.6 million chunks, 84 / 79 ms).  The operator
-// updates' lists (two to ten tasks in the mean) keep the FP64 pipes busy as they are: 10 ms in
-// rounds, 6 ms without for one of random L=28, D=700.
+// Ordered sums in rounds: lists of at least kGemmRoundTasks tasks in the mean, in tables of at
+// most kGemmMaxChunks chunks (their table costs the host 8 bytes and a pass each; the operator
+// updates' lists, two to ten tasks in the mean, keep the FP64 pipes busy as they are: 10 ms in
+// rounds, 6 ms without for one of random L=28, D=700), and of those the ones that the
+// estimates below find shorter in rounds.  Rounds shorten the longest chain four- to tenfold but
+// scale every chunk of A, so that they retire FMAs at half the rate of the lanes: they are for
+// tables too small to fill the SMs.
 constexpr int64_t kGemmRoundTasks = 12, kGemmMaxChunks = 1 << 21;
+
+// Time of a table of ordered sums (cycles): what the FP64 pipes need for all of it (16 cycles
+// of an SM per warp FMA) and the longest chain, which the start of the last CTAs and uneven
+// SMs stretch.  Fitted to phase 2 of 30 tables, within 30 % but for the smallest; measured, lanes
+// / rounds: Hubbard L=8, D=64 165 / 47 us, L=12, D=300 3.2 / 1.9 ms, L=16, D=200 0.97 / 0.50 ms,
+// L=16, D=1000 15.7 / 28.5 ms and, a step on, 61 / 136 ms (staged tiles: 110 ms); random L=12,
+// D=500 1.26 / 0.53 ms, L=16, D=600 0.88 / 1.01 ms and 1.49 / 1.08 ms, L=16, D=1500 2.3 / 2.9 ms,
+// L=28, D=700 12.5 / 5.2 ms, L=28, D=1500 32 / 40 ms.
+struct OrderedCost {
+  double lane_fmas = 0.0, lane_chain = 0.0, round_fmas = 0.0, round_chain = 0.0;
+  // slices: 32-lane slices of the group, in lanes (rpl rows each) and in rounds
+  void add(int64_t lane_slices, int64_t slices, int rpl, int64_t tasks, int64_t columns, int64_t chunks) {
+    lane_fmas += (double)lane_slices * rpl * columns;
+    lane_chain = std::max(lane_chain, 1300.0 * tasks + 145.0 * rpl * columns);
+    round_fmas += 8.0 * slices * chunks;  // four FMAs and the scaling of four columns of A
+    round_chain = std::max(round_chain, 520.0 * chunks);
+  }
+  bool rounds() const {
+    constexpr double kPipe = 16.0 / 152;
+    return 1.35 * kPipe * round_fmas + round_chain < kPipe * lane_fmas + 1.3 * lane_chain;
+  }
+};
 
 // ks: columns of a group's tasks in all; rpl: its rows per lane; max_ns: warps that may share a
 // sum; max_nw: slices that a job may take.
@@ -606,20 +629,25 @@ GemmPlan* gemm_plan_upload(const std::vector<GemmTask>& t, std::vector<GemmGroup
   std::vector<int64_t> ks(g.size(), 0);
   std::vector<int> rpl(g.size(), 1);
   int64_t chunks = 0, live = 0;
+  OrderedCost cost;
   for (size_t q = 0; q < g.size(); ++q) {
     GemmGroup& G = g[q];
     if (G.m <= 0 || G.n <= 0) continue;
     bool strided = false;
+    int64_t c = 0;
     for (int k = G.task_begin; k < G.task_end; ++k) {
       ks[q] += t[k].A ? t[k].k : 1;
-      chunks += t[k].A ? (t[k].k + 3) / 4 : 1;
+      c += t[k].A ? (t[k].k + 3) / 4 : 1;
       strided = strided || (t[k].A && t[k].transB);
     }
+    chunks += c;
     if (ks[q] == 0) continue;
-    G.rpl = rpl[q] = rows_per_lane(G.m, G.n, strided);
+    const int R = G.rpl = rpl[q] = rows_per_lane(G.m, G.n, strided);
+    cost.add(((int64_t)((G.m + R - 1) / R) * G.n + 31) / 32, ((int64_t)G.m * G.n + 31) / 32, R,
+             G.task_end - G.task_begin, ks[q], c);
     ++live;
   }
-  p->rounds = (sums & GEMM_ORDERED) && p->ntasks >= kGemmRoundTasks * live && chunks <= kGemmMaxChunks;
+  p->rounds = (sums & GEMM_ORDERED) && p->ntasks >= kGemmRoundTasks * live && chunks <= kGemmMaxChunks && cost.rounds();
   if (sums & (GEMM_LANES | GEMM_ROUNDS)) p->rounds = (sums & GEMM_ROUNDS) != 0;
   const std::vector<int> one(p->rounds ? g.size() : 0, 1);  // rows per lane of the rounds
   try {
