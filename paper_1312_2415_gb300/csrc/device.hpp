@@ -3,6 +3,7 @@
 #pragma once
 #include <cstddef>
 #include <cstdint>
+#include <exception>
 #include <vector>
 
 namespace dmrg {
@@ -19,6 +20,9 @@ void dev_zero(void* p, size_t bytes, Stream s);
 void dev_sync(Stream s);
 size_t dev_bytes_in_use();     // device bytes held by the library (all contexts)
 void dev_set_cap(size_t bytes);  // 0 = no cap; otherwise dev_alloc beyond it throws bad_alloc
+// an allocation that failed (the cap, the device or the host), not another error; the device's
+// own leaves its status in cudaGetLastError, which this clears
+bool no_room(const std::exception& e);
 int64_t kernel_launches();  // number of this library's kernel launches so far
 int dev_check(const char** msg);  // 0 if no CUDA error is pending
 void* host_pinned_alloc(size_t bytes);

@@ -76,6 +76,12 @@ void dev_free(void* p, Stream s) {
   }
   ck(cudaFreeAsync(p, S(s)), "cudaFreeAsync");
 }
+bool no_room(const std::exception& e) {
+  if (dynamic_cast<const std::bad_alloc*>(&e)) return true;
+  if (std::string(e.what()).find("out of memory") == std::string::npos) return false;
+  cudaGetLastError();
+  return true;
+}
 size_t dev_bytes_in_use() {
   std::lock_guard<std::mutex> lk(g_mem_mu);
   return g_mem_in_use;
@@ -1613,11 +1619,6 @@ struct DevScratch {
   }
 };
 
-// an allocation that failed (the cap, the device or the host), not another error
-bool no_room(const std::exception& e) {
-  return dynamic_cast<const std::bad_alloc*>(&e) || std::string(e.what()).find("out of memory") != std::string::npos;
-}
-
 constexpr int kEigSmemN = 64;  // blocks up to this size are diagonalised in shared memory
 
 // Cyclic Jacobi (round-robin pairing, n/2 rotations per step) on one symmetric block per
@@ -2472,7 +2473,6 @@ void eig_refined(const std::vector<EigJob>& jobs, const std::vector<EigSource>& 
     again = refined_passes(jobs, src, nmax, s);
   } catch (const std::exception& e) {
     if (!no_room(e)) throw;
-    cudaGetLastError();
     again = jobs;  // the workspace has been released: the solver in place
   }
   eig_batched(again, s);

@@ -44,6 +44,7 @@
 
 #include <algorithm>
 #include <cstdint>
+#include <limits>
 #include <unordered_map>
 #include <stdexcept>
 #include <string>
@@ -881,19 +882,26 @@ size_t smem_bytes() {
 
 }  // namespace
 
+// Output tiles whose partial sums are in memory together: their runs of terms by class (S, M,
+// L; ranges of TcPlan::tiles) and their sums (a range of TcPlan::red).
+struct TcPass {
+  int nclass[3] = {0, 0, 0}, first[3] = {0, 0, 0}, grid[3] = {0, 0, 0};
+  int red = 0, nred = 0;
+};
+
 struct TcPlan {
-  TfTile* tiles = nullptr;     // runs of terms by class (S, M, L), in queue order
+  TfTile* tiles = nullptr;     // runs of terms by pass and class, in queue order
   TfTask* tasks = nullptr;
   TfSrc* srcs = nullptr;
   TfConv* xb = nullptr;
   TfTile* tiny = nullptr;      // tiles for k_tc_tiny
   TfReduce* red = nullptr;     // output tiles and their partial sums
   float* part = nullptr;
-  int ntiny = 0, nred = 0;
+  std::vector<TcPass> passes;  // one, unless the partial sums do not fit
+  int ntiny = 0;
   int* queue = nullptr;        // the persistent kernels' tile counters, one per class
   int* active = nullptr;       // per instance: 0 = skip its tiles
   int ninst = 0;
-  int nclass[3] = {0, 0, 0}, first[3] = {0, 0, 0}, grid[3] = {0, 0, 0};
   int nxb = 0;
   int launches = 0;  // kernels of one launch sequence
 };
@@ -909,7 +917,10 @@ int sm_count() {
 
 }  // namespace
 
-TcPlan* tc_plan_build(const std::vector<const TcHost*>& inst, Stream st) {
+namespace {
+// part_max: partial sums (floats) that may be in memory together (the largest tile's may be
+// more); *part_need: how many there are at most
+TcPlan* plan_build(const std::vector<const TcHost*>& inst, int64_t part_max, int64_t* part_need, Stream st) {
   TcPlan* P = new TcPlan;
   try {
     std::vector<TfSrc> s;
@@ -981,14 +992,32 @@ TcPlan* tc_plan_build(const std::vector<const TcHost*>& inst, Stream st) {
       run[c] = terms[c] / ((int64_t)8 * ctas[c]);
       run[c] = std::min<int64_t>(kMaxRun, std::max<int64_t>(kFlushTerms, run[c] / kFlushTerms * kFlushTerms));
     }
-    std::vector<TfTile> runs[3];
+    std::vector<TfTile> runs[3], all;
     std::vector<TfReduce> red;
     red.reserve(sorted.size());
-    int64_t part = 0;
+    int64_t part = 0, need = 0;  // of the current pass, of the largest
+    auto close = [&]() {  // ends a pass
+      TcPass ps;
+      for (int c = 0; c < 3; ++c) {
+        ps.first[c] = (int)all.size();
+        ps.nclass[c] = (int)runs[c].size();
+        ps.grid[c] = (int)std::min<size_t>(runs[c].size(), (size_t)ctas[c]);
+        all.insert(all.end(), runs[c].begin(), runs[c].end());
+        runs[c].clear();
+        P->launches += ps.nclass[c] > 0;
+      }
+      ps.red = P->passes.empty() ? 0 : P->passes.back().red + P->passes.back().nred;
+      ps.nred = (int)red.size() - ps.red;
+      P->launches += ps.nred > 0;
+      P->passes.push_back(ps);
+      need = std::max(need, part);
+      part = 0;
+    };
     for (size_t i = 0; i < sorted.size(); ++i) {
       const TfTile& q = sorted[i];
       const int T = q.t_end - q.t_begin, nf = std::max(1, (T + kFlushTerms - 1) / kFlushTerms);
       const int64_t mn = (int64_t)q.m * q.nv, step = run[(int)cl[i]];
+      if (part > 0 && part + nf * mn > part_max) close();
       red.push_back({q.y, part, q.ldy, q.m, q.nv, nf, q.inst, 0});
       int64_t t = 0;
       do {
@@ -1001,31 +1030,43 @@ TcPlan* tc_plan_build(const std::vector<const TcHost*>& inst, Stream st) {
       } while (t < T);
       part += nf * mn;
     }
-    std::vector<TfTile> all;
-    for (int c = 0; c < 3; ++c) {
-      P->first[c] = (int)all.size();
-      P->nclass[c] = (int)runs[c].size();
-      P->grid[c] = (int)std::min<size_t>(runs[c].size(), (size_t)ctas[c]);
-      all.insert(all.end(), runs[c].begin(), runs[c].end());
-    }
+    if (!red.empty()) close();
+    *part_need = need;
     P->queue = (int*)dev_alloc(3 * sizeof(int), st);
-    P->part = (float*)dev_alloc(sizeof(float) * std::max<int64_t>(part, 1), st);
+    P->part = (float*)dev_alloc(sizeof(float) * std::max<int64_t>(need, 1), st);
     P->ninst = (int)inst.size();
     P->active = upload(std::vector<int>(inst.size(), 1), st);
     P->tiles = upload(all, st);
     P->red = upload(red, st);
-    P->nred = (int)red.size();
     P->tasks = upload(single ? inst[0]->t : t, st);
     P->srcs = upload(single ? inst[0]->s : s, st);
     P->xb = upload(single ? inst[0]->xb : xb, st);
     P->nxb = (int)(single ? inst[0]->xb.size() : xb.size());
-    P->launches = (P->nxb > 0) + (P->nclass[0] > 0) + (P->nclass[1] > 0) + (P->nclass[2] > 0) + (P->nred > 0) +
-                  (P->ntiny > 0);
+    P->launches += (P->nxb > 0) + (P->ntiny > 0);
   } catch (...) {
     tc_plan_free(P, st);
     throw;
   }
   return P;
+}
+
+}  // namespace
+
+// The partial sums of all output tiles take some 8 % of a large plan (random L=28, D=2500: 0.25
+// of 3.2 GB).  Where they do not fit, the tiles go in passes that share a smaller array: the
+// same sums in the same order, with shorter queues.
+TcPlan* tc_plan_build(const std::vector<const TcHost*>& inst, Stream st) {
+  int64_t max = std::numeric_limits<int64_t>::max(), last = max;
+  for (;;) {
+    int64_t need = 0;
+    try {
+      return plan_build(inst, max, &need, st);
+    } catch (const std::exception& e) {
+      if (!no_room(e) || need == 0 || need >= last) throw;  // one tile's partial sums are the least
+    }
+    last = need;
+    max = need / 2;
+  }
 }
 
 int* tc_plan_active(TcPlan* p) { return p ? p->active : nullptr; }
@@ -1059,10 +1100,10 @@ void tc_set_attributes() {
 }
 
 template <class K>
-void tc_run(const TcPlan* p, int c, cudaStream_t cs) {
-  if (p->nclass[c] > 0)
-    k_tc_matvec<K><<<p->grid[c], K::kThreads, smem_bytes<K>(), cs>>>(p->tiles + p->first[c], p->tasks, p->srcs, p->part,
-                                                                    p->queue + c, p->active, p->nclass[c]);
+void tc_run(const TcPlan* p, const TcPass& q, int c, cudaStream_t cs) {
+  if (q.nclass[c] > 0)
+    k_tc_matvec<K><<<q.grid[c], K::kThreads, smem_bytes<K>(), cs>>>(p->tiles + q.first[c], p->tasks, p->srcs, p->part,
+                                                                    p->queue + c, p->active, q.nclass[c]);
 }
 
 void tc_enqueue(const TcPlan* p, void* const* ev, cudaStream_t cs) {
@@ -1071,12 +1112,12 @@ void tc_enqueue(const TcPlan* p, void* const* ev, cudaStream_t cs) {
   if (ev) event_record(ev[1], cs);
   if (p->ntiny > 0)
     k_tc_tiny<<<p->ntiny, kTinyWarps * 32, 0, cs>>>(p->tiny, p->tasks, p->srcs, p->active);
-  if (p->nred > 0) {
+  for (const TcPass& q : p->passes) {
     ck(cudaMemsetAsync(p->queue, 0, 3 * sizeof(int), cs), "tile queue reset");
-    tc_run<TileL>(p, 2, cs);
-    tc_run<TileM>(p, 1, cs);
-    tc_run<TileS>(p, 0, cs);
-    k_tc_reduce<<<p->nred, 256, 0, cs>>>(p->red, p->part, p->active);
+    tc_run<TileL>(p, q, 2, cs);
+    tc_run<TileM>(p, q, 1, cs);
+    tc_run<TileS>(p, q, 0, cs);
+    k_tc_reduce<<<q.nred, 256, 0, cs>>>(p->red + q.red, p->part, p->active);
   }
   if (ev) event_record(ev[2], cs);
   ck(cudaGetLastError(), "tc matvec launch");
