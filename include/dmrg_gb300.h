@@ -323,7 +323,8 @@ int dmrg_test_tc_timeout(int on);
  * (C offset, ldc, rows, columns, first task, end task); tasks: ntasks x 7 (A offset or -1 for
  * the identity, B offset, lda, ldb, inner size, transA, transB), alpha per task; C += sum of
  * alpha op(A) op(B).  upload: a sum of 1 (ordered sums), 2 (shared sums), 4 (C = the sum),
- * 8 (ordered: lane kernel), 16 (ordered: kernel in rounds); run: 1 or 2.  DMRG_EINVAL for
+ * and at most one of 8 (lane kernel), 16 (ordered: kernel in rounds), 32 (staged tiles);
+ * run: 1 or 2.  DMRG_EINVAL for
  * blocks outside data, DMRG_EINTERNAL for a run of a kind not uploaded. */
 int dmrg_test_block_products(const int64_t* tasks, const double* alpha, int ntasks, const int64_t* groups, int ngroups,
                              double* data, int64_t n, int upload, int run);

@@ -71,10 +71,11 @@ struct GemmPlan;  // device copy of a task/group table
 // long task lists are shared by several warps, whose partial sums are added in a fixed order
 // (shorter chains, other rounding).  A plan carries a job table for each kind it is run with.
 // GEMM_OVERWRITE (upload only): C_g = the sum instead of C_g += the sum (groups without
-// tasks are left as they are).  GEMM_LANES, GEMM_ROUNDS (upload only): which kernel sums the
-// ordered products, instead of the uploader's rule (tests: the bits are the same).  Running
-// a plan with a kind it was not uploaded with is an error.
-enum { GEMM_ORDERED = 1, GEMM_SHARED = 2, GEMM_OVERWRITE = 4, GEMM_LANES = 8, GEMM_ROUNDS = 16 };
+// tasks are left as they are).  GEMM_LANES, GEMM_ROUNDS, GEMM_TILES (upload only, one of them):
+// which kernel sums the groups, instead of the uploader's rule (the bits of ordered sums are
+// the same; large groups in staged tiles are ordered in either kind).  Running a plan with a
+// kind it was not uploaded with is an error.
+enum { GEMM_ORDERED = 1, GEMM_SHARED = 2, GEMM_OVERWRITE = 4, GEMM_LANES = 8, GEMM_ROUNDS = 16, GEMM_TILES = 32 };
 GemmPlan* gemm_plan_upload(const std::vector<GemmTask>& t, std::vector<GemmGroup>& g, Stream s,
                            int sums = GEMM_ORDERED);
 void gemm_plan_run(const GemmPlan* p, Stream s, int sums = GEMM_ORDERED);

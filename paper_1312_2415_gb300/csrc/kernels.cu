@@ -472,6 +472,87 @@ __global__ void __launch_bounds__(kRoundWarps * 32, 4)
   }
 }
 
+// The same sums (one chain per element, alpha multiplied into A first) of large blocks: a CTA
+// per 32 x 32 tile of C, the operands staged in shared memory sixteen columns at a time, 2 x 2
+// elements per thread.  Lanes read a block of 200 rows and columns (some 0.4 MB) through L1 once
+// per four rows of C; a tile reads it once per 32.  Padding to the tile is what it costs: by the
+// rule at kTileMin few groups come here.  Measured (lanes / tiles, Hubbard L=16, D=2500 after a
+// step, blocks of up to 245 rows): phase 1 677 / 585 ms, in Davidson 617 / 565 ms, the operator
+// update 697 / 631 ms.
+constexpr int kTileM = 32, kTileN = 32, kTileK = 16;
+
+template <bool kRemap>
+__global__ void __launch_bounds__(256)
+    k_gemm_tiles(const GemmTask* __restrict__ tasks, const GemmGroup* __restrict__ groups, const GemmJob* __restrict__ jobs,
+                 bool over, Remap rm) {
+  __shared__ double As[kTileK][kTileM + 1];
+  __shared__ double Bs[kTileK][kTileN + 1];
+  const GemmJob J = jobs[blockIdx.x];
+  const GemmGroup g = groups[J.group];
+  const int tn = (g.n + kTileN - 1) / kTileN;
+  const int row0 = (J.w0 / tn) * kTileM, col0 = (J.w0 % tn) * kTileN;
+  const int tid = threadIdx.x, ty = tid >> 4, tx = tid & 15;
+  double acc[2][2] = {{0.0, 0.0}, {0.0, 0.0}};
+  for (int t = g.task_begin; t < g.task_end; ++t) {
+    const GemmTask T = tasks[t];
+    const double* B = kRemap ? remap_ptr(T.B, rm) : T.B;
+    if (T.A == nullptr) {  // op(A) = identity
+#pragma unroll
+      for (int i = 0; i < 2; ++i)
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+          const int r = row0 + ty + 16 * i, c = col0 + tx + 16 * j;
+          if (r < g.m && c < g.n)
+            acc[i][j] = fma(T.alpha, T.transB ? B[(size_t)c * T.ldb + r] : B[(size_t)r * T.ldb + c], acc[i][j]);
+        }
+      continue;
+    }
+    const double* A = kRemap ? remap_ptr(T.A, rm) : T.A;
+    for (int k0 = 0; k0 < T.k; k0 += kTileK) {
+#pragma unroll
+      for (int u = 0; u < kTileM * kTileK / 256; ++u) {
+        const int e = tid + 256 * u;
+        const int kk = T.transA ? e / kTileM : e % kTileK, r = T.transA ? e % kTileM : e / kTileK;
+        const int gr = row0 + r, gk = k0 + kk;
+        double v = 0.0;
+        if (gr < g.m && gk < T.k) v = T.transA ? A[(size_t)gk * T.lda + gr] : A[(size_t)gr * T.lda + gk];
+        As[kk][r] = v * T.alpha;
+      }
+#pragma unroll
+      for (int u = 0; u < kTileN * kTileK / 256; ++u) {
+        const int e = tid + 256 * u;
+        const int kk = T.transB ? e % kTileK : e / kTileN, c = T.transB ? e / kTileK : e % kTileN;
+        const int gc = col0 + c, gk = k0 + kk;
+        double v = 0.0;
+        if (gc < g.n && gk < T.k) v = T.transB ? B[(size_t)gc * T.ldb + gk] : B[(size_t)gk * T.ldb + gc];
+        Bs[kk][c] = v;
+      }
+      __syncthreads();
+#pragma unroll
+      for (int kk = 0; kk < kTileK; ++kk) {
+        const double a0 = As[kk][ty], a1 = As[kk][ty + 16];
+        const double b0 = Bs[kk][tx], b1 = Bs[kk][tx + 16];
+        acc[0][0] = fma(a0, b0, acc[0][0]);
+        acc[0][1] = fma(a0, b1, acc[0][1]);
+        acc[1][0] = fma(a1, b0, acc[1][0]);
+        acc[1][1] = fma(a1, b1, acc[1][1]);
+      }
+      __syncthreads();
+    }
+  }
+  double* C = kRemap ? (double*)remap_ptr(g.C, rm) : g.C;
+#pragma unroll
+  for (int i = 0; i < 2; ++i)
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+      const int r = row0 + ty + 16 * i, c = col0 + tx + 16 * j;
+      if (r < g.m && c < g.n) {
+        double* p = C + (size_t)r * g.ldc + c;
+        *p = over ? acc[i][j] : *p + acc[i][j];
+      }
+    }
+}
+
 // buf: 128 doubles per warp of the CTA
 template <int R, bool kRemap, bool kOrdered>
 __device__ __forceinline__ void gemm_job(const GemmTask* __restrict__ tasks, const GemmGroup& g, const GemmJob& J,
@@ -588,6 +669,16 @@ struct OrderedCost {
   }
 };
 
+// Staged tiles: groups of at least kTileMin rows and columns of which padding to the tile (32 x
+// 32, 16 columns of A) leaves at least kTileEff, in tables with at least kTileCount such tiles, four
+// to five per place on the SMs.  From 96 rows on tiles give the large tables the same times within
+// 2 % but lose up to 6 % on updates of Hubbard L=24, D=4000; in tables of one product per symmetry
+// sector (the refined eigensolver's, up to 202 rows) they start too few CTAs: dmrg_truncate of
+// random L=28, D=1500 21.4 / 22.4 ms.
+constexpr int kTileMin = 160;
+constexpr double kTileEff = 0.8;
+constexpr int64_t kTileCount = 152 * 32;
+
 // ks: columns of a group's tasks in all; rpl: its rows per lane; max_ns: warps that may share a
 // sum; max_nw: slices that a job may take.
 std::vector<GemmJob> gemm_jobs(const std::vector<GemmGroup>& g, const std::vector<int64_t>& ks, const std::vector<int>& rpl,
@@ -631,30 +722,61 @@ GemmPlan* gemm_plan_upload(const std::vector<GemmTask>& t, std::vector<GemmGroup
   p->ntasks = (int64_t)t.size();
   p->kinds = sums & (GEMM_ORDERED | GEMM_SHARED);
   p->overwrite = (sums & GEMM_OVERWRITE) != 0;
-  // per group: columns in all, rows per lane; chunks of the whole table (rounds)
-  std::vector<int64_t> ks(g.size(), 0);
+  // per group: columns and chunks in all, rows per lane, staged tiles (0: none)
+  std::vector<int64_t> ks(g.size(), 0), chunk(g.size(), 0), tile(g.size(), 0);
   std::vector<int> rpl(g.size(), 1);
-  int64_t chunks = 0, live = 0;
-  OrderedCost cost;
+  const int forced = sums & (GEMM_LANES | GEMM_ROUNDS | GEMM_TILES);
+  int64_t ntiles = 0;
   for (size_t q = 0; q < g.size(); ++q) {
     GemmGroup& G = g[q];
     if (G.m <= 0 || G.n <= 0) continue;
     bool strided = false;
-    int64_t c = 0;
+    int64_t padded = 0;
     for (int k = G.task_begin; k < G.task_end; ++k) {
-      ks[q] += t[k].A ? t[k].k : 1;
-      c += t[k].A ? (t[k].k + 3) / 4 : 1;
+      const int cols = t[k].A ? t[k].k : 1;
+      ks[q] += cols;
+      chunk[q] += (cols + 3) / 4;
+      padded += t[k].A ? (cols + kTileK - 1) / kTileK * kTileK : 1;
       strided = strided || (t[k].A && t[k].transB);
     }
-    chunks += c;
     if (ks[q] == 0) continue;
-    const int R = G.rpl = rpl[q] = rows_per_lane(G.m, G.n, strided);
+    G.rpl = rpl[q] = rows_per_lane(G.m, G.n, strided);
+    const int64_t nt = (int64_t)((G.m + kTileM - 1) / kTileM) * ((G.n + kTileN - 1) / kTileN);
+    const bool large = G.m >= kTileMin && G.n >= kTileMin &&
+                       (double)G.m * G.n * ks[q] >= kTileEff * kTileM * kTileN * nt * padded;
+    if (forced ? forced == GEMM_TILES : large) ntiles += tile[q] = nt;
+  }
+  if (!forced && ntiles < kTileCount) ntiles = 0;
+  // what goes where: tiles by decreasing powers of two of their columns; the other groups'
+  // totals decide on rounds
+  std::vector<GemmJob> tile_bucket[48];
+  int64_t chunks = 0, live = 0, tasks = 0;
+  OrderedCost cost;
+  for (size_t q = 0; q < g.size(); ++q) {
+    if (ks[q] == 0) continue;
+    const GemmGroup& G = g[q];
+    if (ntiles > 0 && tile[q] > 0) {
+      int lg = 0;
+      while (ks[q] >> (lg + 1)) ++lg;
+      for (int64_t w = 0; w < tile[q]; ++w) tile_bucket[47 - std::min(lg, 47)].push_back({(int)q, (int)w, 1, 0, 1});
+      ks[q] = 0;  // not in the job tables
+      continue;
+    }
+    const int R = rpl[q];
     cost.add(((int64_t)((G.m + R - 1) / R) * G.n + 31) / 32, ((int64_t)G.m * G.n + 31) / 32, R,
-             G.task_end - G.task_begin, ks[q], c);
+             G.task_end - G.task_begin, ks[q], chunk[q]);
+    chunks += chunk[q];
+    tasks += G.task_end - G.task_begin;
     ++live;
   }
-  p->rounds = (sums & GEMM_ORDERED) && p->ntasks >= kGemmRoundTasks * live && chunks <= kGemmMaxChunks && cost.rounds();
-  if (sums & (GEMM_LANES | GEMM_ROUNDS)) p->rounds = (sums & GEMM_ROUNDS) != 0;
+  std::vector<GemmJob> tiles;
+  for (auto& v : tile_bucket) tiles.insert(tiles.end(), v.begin(), v.end());
+  if (tiles.size() > (size_t)std::numeric_limits<int>::max()) {
+    delete p;
+    throw std::runtime_error("block-product table exceeds 2^31 jobs");
+  }
+  p->rounds = (sums & GEMM_ORDERED) && tasks >= kGemmRoundTasks * live && chunks <= kGemmMaxChunks && cost.rounds();
+  if (forced) p->rounds = forced == GEMM_ROUNDS;
   const std::vector<int> one(p->rounds ? g.size() : 0, 1);  // rows per lane of the rounds
   try {
     for (int kind = 0; kind < 2; ++kind) {
@@ -668,6 +790,11 @@ GemmPlan* gemm_plan_upload(const std::vector<GemmTask>& t, std::vector<GemmGroup
       if (jobs.empty()) continue;
       p->jobs[kind] = (GemmJob*)dev_alloc(jobs.size() * sizeof(GemmJob), s);
       dev_h2d(p->jobs[kind], jobs.data(), jobs.size() * sizeof(GemmJob), s);
+    }
+    if (!tiles.empty()) {
+      p->ntiles = (int)tiles.size();
+      p->tiles = (GemmJob*)dev_alloc(tiles.size() * sizeof(GemmJob), s);
+      dev_h2d(p->tiles, tiles.data(), tiles.size() * sizeof(GemmJob), s);
     }
     if (p->rounds) {
       // the groups' chunk ranges (begin, end), then the chunks (task, first column); the
@@ -703,17 +830,22 @@ template <bool kRemap>
 void gemm_launch(const GemmPlan* p, const Remap& rm, int sums, Stream s) {
   const int kind = sums == GEMM_ORDERED ? 0 : 1;
   if (p && !(p->kinds & sums)) throw std::logic_error("block products run with sums they were not uploaded for");
-  if (!p || p->njobs[kind] == 0) return;
-  const int n = p->njobs[kind];
-  const GemmJob* jobs = p->jobs[kind];
-  if (kind == 0 && p->rounds) {
-    k_gemm_rounds<kRemap><<<n, kRoundWarps * 32, 0, S(s)>>>(p->tasks, p->groups, p->chunks, jobs, p->overwrite, rm);
-  } else {
-    const int grid = (n + kGemmWarps - 1) / kGemmWarps;
-    if (kind == 0) k_grouped_gemm<kRemap, true><<<grid, kGemmWarps * 32, 0, S(s)>>>(p->tasks, p->groups, jobs, n, p->overwrite, rm);
-    else k_grouped_gemm<kRemap, false><<<grid, kGemmWarps * 32, 0, S(s)>>>(p->tasks, p->groups, jobs, n, p->overwrite, rm);
+  if (!p) return;
+  if (p->ntiles > 0) {
+    k_gemm_tiles<kRemap><<<p->ntiles, 256, 0, S(s)>>>(p->tasks, p->groups, p->tiles, p->overwrite, rm);
+    ++g_launches;
   }
-  ++g_launches;
+  const int n = p->njobs[kind], grid = (n + kGemmWarps - 1) / kGemmWarps;
+  const GemmJob* jobs = p->jobs[kind];
+  if (n > 0) {
+    if (kind == 0 && p->rounds)
+      k_gemm_rounds<kRemap><<<n, kRoundWarps * 32, 0, S(s)>>>(p->tasks, p->groups, p->chunks, jobs, p->overwrite, rm);
+    else if (kind == 0)
+      k_grouped_gemm<kRemap, true><<<grid, kGemmWarps * 32, 0, S(s)>>>(p->tasks, p->groups, jobs, n, p->overwrite, rm);
+    else
+      k_grouped_gemm<kRemap, false><<<grid, kGemmWarps * 32, 0, S(s)>>>(p->tasks, p->groups, jobs, n, p->overwrite, rm);
+    ++g_launches;
+  }
   ck(cudaGetLastError(), "grouped_gemm launch");
 }
 }  // namespace
@@ -727,6 +859,7 @@ void gemm_plan_free(GemmPlan* p, Stream s) {
   dev_free(p->jobs[0], s);
   dev_free(p->jobs[1], s);
   dev_free(p->chunks, s);
+  dev_free(p->tiles, s);
   delete p;
 }
 

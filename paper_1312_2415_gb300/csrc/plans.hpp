@@ -25,7 +25,8 @@ struct GemmPlan {
   GemmGroup* groups = nullptr;
   GemmJob* jobs[2] = {nullptr, nullptr};  // ordered sums, shared sums
   GemmChunk* chunks = nullptr;
-  int njobs[2] = {0, 0};
+  GemmJob* tiles = nullptr;  // groups in staged tiles, for either kind: (group, tile)
+  int njobs[2] = {0, 0}, ntiles = 0;
   int kinds = 0;           // GEMM_ORDERED, GEMM_SHARED: the job tables it has
   bool overwrite = false;  // C = sum instead of C += sum
   bool rounds = false;  // ordered sums by k_gemm_rounds

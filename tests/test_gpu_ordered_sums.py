@@ -1,7 +1,7 @@
 """GPU: the grouped block products on their own.  Ordered sums (what steers a Davidson run) are
 one chain of fused multiply-adds per element, over the tasks and columns in table order with
-alpha multiplied into A first: the lane kernel, the kernel in rounds and the uploader's choice
-of the two must all give the bits of that chain computed on the host.  Shared sums may round
+alpha multiplied into A first: the lane kernel, the kernel in rounds, staged tiles and the
+uploader's choice of them must all give the bits of that chain computed on the host.  Shared sums may round
 differently: 1e-13 of sum |alpha A B| per element (lists of at most ~2,000 terms: 2e3 x 1.1e-16).
 
 Blocks of one row or column up to several 32-lane slices, one to 300 tasks, inner sizes with
@@ -12,7 +12,7 @@ import numpy as np
 import pytest
 
 pytestmark = pytest.mark.gpu
-ORDERED, SHARED, OVERWRITE, LANES, ROUNDS = 1, 2, 4, 8, 16
+ORDERED, SHARED, OVERWRITE, LANES, ROUNDS, TILES = 1, 2, 4, 8, 16, 32
 
 
 @pytest.fixture(scope="module")
@@ -35,11 +35,11 @@ def table(seed, shapes, alphas):
         data.append(rng.normal(size=rows * ld))
         size += rows * ld
         return size - rows * ld, ld
-    for m, n, nt, kmax in shapes:
+    for m, n, nt, kmax, *kmin in shapes:
         c, ldc = block(m, n)
         first = len(tasks)
         for _ in range(nt):
-            k = int(rng.integers(1, kmax + 1))
+            k = int(rng.integers(*(kmin or [1]), kmax + 1))
             ta, tb = (int(v) for v in rng.integers(0, 2, 2))
             if rng.random() < 0.15:
                 k, a, lda, ta = m, -1, 0, 0
@@ -96,10 +96,10 @@ def test_sums(hook, shapes, alphas, over):
     tab = table(len(shapes) + 7 * len(alphas), shapes, alphas)
     want, mag = host(*tab, over)
     flag = OVERWRITE if over else 0
-    for kind in (ORDERED, ORDERED | LANES, ORDERED | ROUNDS, ORDERED | SHARED, ORDERED | SHARED | ROUNDS):
+    for kind in (ORDERED, ORDERED | LANES, ORDERED | ROUNDS, ORDERED | TILES, ORDERED | SHARED, ORDERED | SHARED | ROUNDS):
         got = hook.test_block_products(*tab, kind | flag, ORDERED)
         assert np.array_equal(got.view(np.int64), want.view(np.int64)), (kind, np.abs(got - want).max())
-    for kind in (SHARED, ORDERED | SHARED):
+    for kind in (SHARED, ORDERED | SHARED, SHARED | TILES):
         got = hook.test_block_products(*tab, kind | flag, SHARED)
         assert (np.abs(got - want) <= 1e-13 * mag).all(), kind
 
@@ -110,3 +110,30 @@ def test_a_run_of_another_kind_is_an_error(hook):
         with pytest.raises(hook.DMRGError) as e:
             hook.test_block_products(*tab, upload, run)
         assert e.value.code == hook.EINTERNAL
+
+
+def test_large_blocks(hook):
+    """Blocks that the uploader's rule gives to staged tiles (at least 160 rows and columns with
+    little padding, enough of them), and blocks beside them that it gives to lanes (one row
+    less, much padding, small)."""
+    tab = table(3, [(192, 160, 2, 16, 15), (159, 160, 1, 3), (161, 161, 1, 4), (5, 7, 13, 6)], (0.37, -1.0))
+    want, mag = host(*tab, False)
+    for kind in (ORDERED, ORDERED | LANES, ORDERED | TILES, ORDERED | SHARED):
+        got = hook.test_block_products(*tab, kind, ORDERED)
+        assert np.array_equal(got.view(np.int64), want.view(np.int64)), (kind, np.abs(got - want).max())
+    for kind in (SHARED, SHARED | TILES):
+        assert (np.abs(hook.test_block_products(*tab, kind, SHARED) - want) <= 1e-13 * mag).all(), kind
+    # the first group 200 times over (6,000 tiles): the rule's own choice, on copies of its C
+    tasks, alpha, groups, data = tab
+    c, ldc, m, n, t0, t1 = groups[0]
+    copies = 200
+    many = np.array([(data.size + i * m * ldc, ldc, m, n, t0, t1) for i in range(copies)] + groups[1:].tolist())
+    block = data[c:c + m * ldc]
+    wide = np.concatenate([data] + [block] * copies)
+    for kind, run in ((ORDERED | SHARED, ORDERED), (SHARED, SHARED), (ORDERED | LANES, ORDERED)):
+        got = hook.test_block_products(tasks, alpha, many, wide, kind, run)
+        for i in range(copies):  # ordered in either kind where the rule takes tiles
+            part = got[data.size + i * m * ldc:][:m * ldc]
+            assert np.array_equal(part.view(np.int64), want[c:c + m * ldc].view(np.int64)), (kind, i)
+        rest = np.r_[got[:c], got[c + m * ldc:data.size]]
+        assert (np.abs(rest - np.r_[want[:c], want[c + m * ldc:]]) <= 1e-13 * np.r_[mag[:c], mag[c + m * ldc:]]).all()
