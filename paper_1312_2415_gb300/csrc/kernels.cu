@@ -717,7 +717,9 @@ std::vector<GemmJob> gemm_jobs(const std::vector<GemmGroup>& g, const std::vecto
 }
 }  // namespace
 
-GemmPlan* gemm_plan_upload(const std::vector<GemmTask>& t, std::vector<GemmGroup>& g, Stream s, int sums) {
+namespace {
+// *rounds: the plan sums in rounds (also where the upload fails)
+GemmPlan* plan_upload(const std::vector<GemmTask>& t, std::vector<GemmGroup>& g, Stream s, int sums, bool* rounds) {
   GemmPlan* p = new GemmPlan;
   p->ntasks = (int64_t)t.size();
   p->kinds = sums & (GEMM_ORDERED | GEMM_SHARED);
@@ -777,6 +779,7 @@ GemmPlan* gemm_plan_upload(const std::vector<GemmTask>& t, std::vector<GemmGroup
   }
   p->rounds = (sums & GEMM_ORDERED) && tasks >= kGemmRoundTasks * live && chunks <= kGemmMaxChunks && cost.rounds();
   if (forced) p->rounds = forced == GEMM_ROUNDS;
+  *rounds = p->rounds;
   const std::vector<int> one(p->rounds ? g.size() : 0, 1);  // rows per lane of the rounds
   try {
     for (int kind = 0; kind < 2; ++kind) {
@@ -823,6 +826,17 @@ GemmPlan* gemm_plan_upload(const std::vector<GemmTask>& t, std::vector<GemmGroup
     throw;
   }
   return p;
+}
+}  // namespace
+
+GemmPlan* gemm_plan_upload(const std::vector<GemmTask>& t, std::vector<GemmGroup>& g, Stream s, int sums) {
+  bool rounds = false;
+  try {
+    return plan_upload(t, g, s, sums, &rounds);
+  } catch (const std::exception& e) {
+    if (!rounds || (sums & GEMM_ROUNDS) || !no_room(e)) throw;
+  }
+  return plan_upload(t, g, s, sums | GEMM_LANES, &rounds);  // no room for the chunks (same bits)
 }
 
 namespace {

@@ -137,3 +137,30 @@ def test_large_blocks(hook):
             assert np.array_equal(part.view(np.int64), want[c:c + m * ldc].view(np.int64)), (kind, i)
         rest = np.r_[got[:c], got[c + m * ldc:data.size]]
         assert (np.abs(rest - np.r_[want[:c], want[c + m * ldc:]]) <= 1e-13 * np.r_[mag[:c], mag[c + m * ldc:]]).all()
+
+
+def test_rounds_without_room_for_their_table(hook):
+    """Under a device-memory cap that the lanes' tables fit under and the rounds' chunks do not,
+    the uploader takes lanes: nothing that fits is refused, and the bits are the same."""
+    tab = table(5, [(4, 8, 60, 64, 40)] * 3, (0.37, 1.0))
+    used = hook.device_memory_in_use()
+    want = hook.test_block_products(*tab, ORDERED, ORDERED)
+
+    def run(kind, cap):
+        hook.set_device_memory_cap(cap)
+        try:
+            return hook.test_block_products(*tab, kind, ORDERED)
+        except hook.DMRGError as e:
+            assert e.code == hook.ENOMEM and hook.device_memory_in_use() == used
+            return None
+        finally:
+            hook.set_device_memory_cap(0)
+    between = 0
+    for room in range(0, 64 * 1024, 512):
+        cap = used + 8 * tab[3].size + room
+        rule, lanes, rounds = run(ORDERED, cap), run(ORDERED | LANES, cap), run(ORDERED | ROUNDS, cap)
+        assert (rule is None) == (lanes is None)
+        between += lanes is not None and rounds is None
+        for got in (rule, lanes, rounds):
+            assert got is None or np.array_equal(got.view(np.int64), want.view(np.int64))
+    assert between > 0 and rule is not None and rounds is not None
