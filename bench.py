@@ -332,7 +332,7 @@ def matvec_kernel_rates(delta):
 #       --nvtx-include "steps/" -k regex:k_tc_matvec -c 150 --csv
 #       python bench.py --no-fp64 --no-e2e --no-cpu-baseline --no-batch
 NCU_TRAFFIC = {
-    (("random28", 2500), "2b31601acab1a423"): {
+    (("random28", 2500), "29148693d6b035fe"): {
         "bytes": 3.35e10, "how": "mean over the 48 matvecs of the timed steps (120 launches), ncu one pass"},
 }
 

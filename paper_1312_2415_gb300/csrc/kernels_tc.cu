@@ -1034,6 +1034,9 @@ TcPlan* plan_build(const std::vector<const TcHost*>& inst, int64_t part_max, int
     *part_need = need;
     P->queue = (int*)dev_alloc(3 * sizeof(int), st);
     P->part = (float*)dev_alloc(sizeof(float) * std::max<int64_t>(need, 1), st);
+    // a CTA that gives up leaves its partial sums as they are, and the reduction reads them
+    // before the host sees the error: they hold numbers from the start
+    dev_zero(P->part, sizeof(float) * std::max<int64_t>(need, 1), st);
     P->ninst = (int)inst.size();
     P->active = upload(std::vector<int>(inst.size(), 1), st);
     P->tiles = upload(all, st);
