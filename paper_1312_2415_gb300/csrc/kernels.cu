@@ -219,16 +219,17 @@ void copy_batched(const std::vector<CopyJob>& jobs, Stream s) {
 //
 // C_g += sum_t alpha_t op(A_t) op(B_t) over tables of thousands of small blocks (1 to ~150
 // rows, tens to thousands of tasks per output).  An SM retires two FP64 FMAs per cycle, 16
-// cycles for one warp's FMA, while L1 serves a warp's operand in 1 to 4: neither register
-// tiling nor staging in shared memory buys anything, but every idle lane and every wait on
-// a chain of tasks does cost.  So the output elements of a group are laid on lanes without
-// padding to a tile: a lane owns R rows of one column (R = 1, 2 or 4, chosen per group so
-// that the fewest lanes idle), the operands come straight from L1 / L2 with no barrier
-// anywhere in the sum, and groups with long task lists are shared by 2 to 8 warps of a CTA,
-// whose partial sums are added in a fixed order (deterministic, no atomics).  Measured
-// against 32 x 32 tiles staged in shared memory with two barriers per 16 columns (H_eff x,
-// whole call): Hubbard L=8, D=64 769 -> 98 us; random L=12, D=500 17.4 -> 1.2 ms; random
-// L=28, D=1500 281 -> 128 ms (0.90 TFLOP/s; cuBLAS DGEMM reaches 1.10 on large squares).  Four
+// cycles for one warp's FMA, while L1 serves a warp's operand in 1 to 4: below about 160 rows
+// neither register tiling nor staging in shared memory buys anything, but every idle lane,
+// every wait on a chain of tasks and every further FP64 operation does cost.  So the output
+// elements of a group are laid on lanes without padding to a tile: a lane owns R rows of one
+// column (R = 1, 2 or 4, chosen per group so that the fewest lanes idle), the operands come
+// straight from L1 / L2 with no barrier anywhere in the sum, and groups with long task lists
+// are shared by 2 to 8 warps of a CTA, whose partial sums are added in a fixed order
+// (deterministic, no atomics).  Larger groups go in staged tiles, short tables of long ordered
+// lists in rounds (below).  Measured against staged tiles for every size (H_eff x, whole call):
+// Hubbard L=8, D=64 769 -> 98 us; random L=12, D=500 17.4 -> 1.2 ms; random L=28, D=1500
+// 281 -> 128 ms (0.90 TFLOP/s; cuBLAS DGEMM reaches 1.10 on large squares).  Four
 // CTAs of 64 registers per SM against two of 128: phase 1 95 -> 83 ms, phase 2 39 -> 43 ms
 // there.  The last one to three columns of a task are loaded together, not one at a time:
 // phase 2 50 -> 39 ms.
