@@ -6,6 +6,7 @@
 #include <cmath>
 #include <cstdio>
 #include <limits>
+#include <memory>
 #include <mutex>
 #include <new>
 #include <stdexcept>
@@ -721,7 +722,14 @@ std::vector<GemmJob> gemm_jobs(const std::vector<GemmGroup>& g, const std::vecto
 namespace {
 // *rounds: the plan sums in rounds (also where the upload fails)
 GemmPlan* plan_upload(const std::vector<GemmTask>& t, std::vector<GemmGroup>& g, Stream s, int sums, bool* rounds) {
-  GemmPlan* p = new GemmPlan;
+  auto drop = [s](GemmPlan* q) {  // what there is of the plan, on every way out but the last
+    try {
+      gemm_plan_free(q, s);
+    } catch (...) {
+    }
+  };
+  std::unique_ptr<GemmPlan, decltype(drop)> hold(new GemmPlan, drop);
+  GemmPlan* p = hold.get();
   p->ntasks = (int64_t)t.size();
   p->kinds = sums & (GEMM_ORDERED | GEMM_SHARED);
   p->overwrite = (sums & GEMM_OVERWRITE) != 0;
@@ -774,59 +782,52 @@ GemmPlan* plan_upload(const std::vector<GemmTask>& t, std::vector<GemmGroup>& g,
   }
   std::vector<GemmJob> tiles;
   for (auto& v : tile_bucket) tiles.insert(tiles.end(), v.begin(), v.end());
-  if (tiles.size() > (size_t)std::numeric_limits<int>::max()) {
-    delete p;
+  if (tiles.size() > (size_t)std::numeric_limits<int>::max())
     throw std::runtime_error("block-product table exceeds 2^31 jobs");
-  }
   p->rounds = (sums & GEMM_ORDERED) && tasks >= kGemmRoundTasks * live && chunks <= kGemmMaxChunks && cost.rounds();
   if (forced) p->rounds = forced == GEMM_ROUNDS;
   *rounds = p->rounds;
   const std::vector<int> one(p->rounds ? g.size() : 0, 1);  // rows per lane of the rounds
-  try {
-    for (int kind = 0; kind < 2; ++kind) {
-      if (!(sums & (kind == 0 ? GEMM_ORDERED : GEMM_SHARED))) continue;
-      const std::vector<GemmJob> jobs =
-          gemm_jobs(g, ks, kind == 0 && p->rounds ? one : rpl, kind == 0 ? 1 : kGemmWarps,
-                    kind == 0 && p->rounds ? 1 : 32767);
-      if (jobs.size() > (size_t)std::numeric_limits<int>::max() - kGemmWarps)
-        throw std::runtime_error("block-product table exceeds 2^31 jobs");
-      p->njobs[kind] = (int)jobs.size();
-      if (jobs.empty()) continue;
-      p->jobs[kind] = (GemmJob*)dev_alloc(jobs.size() * sizeof(GemmJob), s);
-      dev_h2d(p->jobs[kind], jobs.data(), jobs.size() * sizeof(GemmJob), s);
-    }
-    if (!tiles.empty()) {
-      p->ntiles = (int)tiles.size();
-      p->tiles = (GemmJob*)dev_alloc(tiles.size() * sizeof(GemmJob), s);
-      dev_h2d(p->tiles, tiles.data(), tiles.size() * sizeof(GemmJob), s);
-    }
-    if (p->rounds) {
-      // the groups' chunk ranges (begin, end), then the chunks (task, first column); the
-      // ranges are relative to the table
-      std::vector<GemmChunk> ch(g.size());
-      for (size_t q = 0; q < g.size(); ++q) {
-        ch[q].begin = (int)ch.size();
-        if (ks[q] > 0)
-          for (int k = g[q].task_begin; k < g[q].task_end; ++k)
-            for (int k0 = 0; k0 < (t[k].A ? t[k].k : 1); k0 += 4) ch.push_back(GemmChunk{{k}, {k0}});
-        ch[q].end = (int)ch.size();
-      }
-      p->chunks = (GemmChunk*)dev_alloc(std::max<size_t>(ch.size(), 1) * sizeof(GemmChunk), s);
-      dev_h2d(p->chunks, ch.data(), ch.size() * sizeof(GemmChunk), s);
-    }
-    if (!t.empty()) {
-      p->tasks = (GemmTask*)dev_alloc(t.size() * sizeof(GemmTask), s);
-      dev_h2d(p->tasks, t.data(), t.size() * sizeof(GemmTask), s);
-    }
-    if (!g.empty()) {
-      p->groups = (GemmGroup*)dev_alloc(g.size() * sizeof(GemmGroup), s);
-      dev_h2d(p->groups, g.data(), g.size() * sizeof(GemmGroup), s);
-    }
-  } catch (...) {
-    gemm_plan_free(p, s);
-    throw;
+  for (int kind = 0; kind < 2; ++kind) {
+    if (!(sums & (kind == 0 ? GEMM_ORDERED : GEMM_SHARED))) continue;
+    const std::vector<GemmJob> jobs =
+        gemm_jobs(g, ks, kind == 0 && p->rounds ? one : rpl, kind == 0 ? 1 : kGemmWarps,
+                  kind == 0 && p->rounds ? 1 : 32767);
+    if (jobs.size() > (size_t)std::numeric_limits<int>::max() - kGemmWarps)
+      throw std::runtime_error("block-product table exceeds 2^31 jobs");
+    p->njobs[kind] = (int)jobs.size();
+    if (jobs.empty()) continue;
+    p->jobs[kind] = (GemmJob*)dev_alloc(jobs.size() * sizeof(GemmJob), s);
+    dev_h2d(p->jobs[kind], jobs.data(), jobs.size() * sizeof(GemmJob), s);
   }
-  return p;
+  if (!tiles.empty()) {
+    p->ntiles = (int)tiles.size();
+    p->tiles = (GemmJob*)dev_alloc(tiles.size() * sizeof(GemmJob), s);
+    dev_h2d(p->tiles, tiles.data(), tiles.size() * sizeof(GemmJob), s);
+  }
+  if (p->rounds) {
+    // the groups' chunk ranges (begin, end), then the chunks (task, first column); the
+    // ranges are relative to the table
+    std::vector<GemmChunk> ch(g.size());
+    for (size_t q = 0; q < g.size(); ++q) {
+      ch[q].begin = (int)ch.size();
+      if (ks[q] > 0)
+        for (int k = g[q].task_begin; k < g[q].task_end; ++k)
+          for (int k0 = 0; k0 < (t[k].A ? t[k].k : 1); k0 += 4) ch.push_back(GemmChunk{{k}, {k0}});
+      ch[q].end = (int)ch.size();
+    }
+    p->chunks = (GemmChunk*)dev_alloc(std::max<size_t>(ch.size(), 1) * sizeof(GemmChunk), s);
+    dev_h2d(p->chunks, ch.data(), ch.size() * sizeof(GemmChunk), s);
+  }
+  if (!t.empty()) {
+    p->tasks = (GemmTask*)dev_alloc(t.size() * sizeof(GemmTask), s);
+    dev_h2d(p->tasks, t.data(), t.size() * sizeof(GemmTask), s);
+  }
+  if (!g.empty()) {
+    p->groups = (GemmGroup*)dev_alloc(g.size() * sizeof(GemmGroup), s);
+    dev_h2d(p->groups, g.data(), g.size() * sizeof(GemmGroup), s);
+  }
+  return hold.release();
 }
 }  // namespace
 
