@@ -673,10 +673,12 @@ struct OrderedCost {
 
 // Staged tiles: groups of at least kTileMin rows and columns of which padding to the tile (32 x
 // 32, 16 columns of A) leaves at least kTileEff, in tables with at least kTileCount such tiles, four
-// to five per place on the SMs.  From 96 rows on tiles give the large tables the same times within
-// 2 % but lose up to 6 % on updates of Hubbard L=24, D=4000; in tables of one product per symmetry
-// sector (the refined eigensolver's, up to 202 rows) they start too few CTAs: dmrg_truncate of
-// random L=28, D=1500 21.4 / 22.4 ms.
+// to five per place on the SMs.  Measured (none / from 160 / from 192 / from 224 rows): phase 1 of
+// Hubbard L=16, D=2500 674 / 589 / 645 / 676 ms, its update 696 / 632 / 632 / 638 ms, the energy of
+// swept random L=28, D=2500 677 / 656 / 675 ms; from 96 rows on the same within 2 %, but up to 6 %
+// more for updates of Hubbard L=24, D=4000.  In tables of one product per symmetry sector (the
+// refined eigensolver's, up to 202 rows) tiles are too few CTAs: dmrg_truncate of random L=28,
+// D=1500 21.4 / 22.4 ms.
 constexpr int kTileMin = 160;
 constexpr double kTileEff = 0.8;
 constexpr int64_t kTileCount = 152 * 32;
